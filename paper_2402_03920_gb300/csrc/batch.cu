@@ -27,7 +27,7 @@ namespace qisg {
 namespace {
 
 constexpr int kBatchBlock = 256;
-static_assert(kBatchBlock <= kLanesMaxThreads, "the LANES class-code buffer holds kLanesMaxThreads threads");
+static_assert(kBatchBlock == kLanesThreads, "a LANES tile takes kLanesThreads threads");
 
 struct InstDev {
   unsigned long long *spins;   // [g][site]
@@ -40,7 +40,7 @@ struct InstDev {
   unsigned long long t;        // sweeps done (mutable)
   long long remaining;         // sweeps left; < 0: no limit (mutable)
   uint2 key;
-  FastDiv hpd;
+  FastDiv hpd, hld;
   int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, spb, N;
   int tau_ap;   // antiperiodic along tau: the wrap tau bond flips sign
   int active;
@@ -67,6 +67,7 @@ __device__ void batch_tile(const InstDev &I, int colour, int j0, int n, unsigned
   S.ctr_w = DOM_SWEEP << 28;   // sample 0: sample block 0
   S.t = (uint32_t)__ldcg(&I.t);
   S.hpd = I.hpd;
+  S.hld = I.hld;
   S.L = I.L;
   S.Lt = I.Lt;
   S.plane = I.plane;
@@ -77,8 +78,12 @@ __device__ void batch_tile(const InstDev &I, int colour, int j0, int n, unsigned
   S.rpw = I.rpw;
   S.n_groups = I.n_groups;
   S.tau_ap = I.tau_ap;
-  if (I.n_rep == 4)   // the common case (every uneven-batch and serving instance): loops unrolled
-    lanes_tile<unsigned long long, true, BLUE, 4>(S, colour, j0, n, 0, colour == 0 && j0 == 0, smem);
+  // four replicas (every uneven-batch and serving instance): one quad and
+  // the registers of the word groups there are
+  if (I.n_rep == 4 && I.n_groups == 1)
+    lanes_tile<unsigned long long, true, BLUE, 4, 1>(S, colour, j0, n, 0, colour == 0 && j0 == 0, smem);
+  else if (I.n_rep == 4)
+    lanes_tile<unsigned long long, true, BLUE, 4, 2>(S, colour, j0, n, 0, colour == 0 && j0 == 0, smem);
   else
     lanes_tile<unsigned long long, true, BLUE>(S, colour, j0, n, 0, colour == 0 && j0 == 0, smem);
 }
@@ -264,6 +269,7 @@ int build_tables(qisg_batch *B) {
     });
   B->max_plane = 4;
   B->max_slots = B->max_rep = B->max_spb_groups = 1;
+  B->smem = 0;
   for (int i : order) {
     const InstDev &I = B->slots[i].dev;
     const int per = kBatchBlock * B->tile_rows;
@@ -273,6 +279,7 @@ int build_tables(qisg_batch *B) {
     B->max_plane = std::max(B->max_plane, I.plane);
     B->max_slots = std::max(B->max_slots, I.n_slots);
     B->max_rep = std::max(B->max_rep, I.n_rep);
+    B->smem = std::max(B->smem, lanes_tile_smem(I.n_slots, I.n_rep));
     B->max_spb_groups = std::max(B->max_spb_groups, I.spb * I.n_groups);
   }
   int rc = QISG_OK;
@@ -299,8 +306,7 @@ int build_tables(qisg_batch *B) {
   if (rc) return rc;
   B->n_tiles = (int)tiles.size();
   B->n_chains = (int)chains.size();
-  B->smem = lanes_tile_smem(B->max_plane, B->max_slots, B->max_rep);
-  if (B->smem > 200 * 1024) return fail(QISG_EINVAL, "instance too large for the batch kernel's shared memory");
+  if (!lanes_plane_fits(B->max_plane, B->max_slots, B->max_rep, 200 * 1024)) return fail(QISG_EINVAL, "instance too large for the batch kernel's shared memory");
   cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->smem);
   int per_sm = 0;
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kBatchBlock, B->smem),
@@ -416,6 +422,7 @@ int setup_slot(qisg_batch *B, int i) {
   I.plane = d.L * d.L;
   I.half_plane = I.plane / 2;
   I.hpd = FastDiv((uint32_t)I.half_plane);
+  I.hld = FastDiv((uint32_t)(I.L / 2));
   I.n_slots = n;
   I.n_rep = d.n_replicas;
   I.rpw = rpw;

@@ -11,6 +11,7 @@
 //   U      u64 [a][r][w][2]            unsatisfied spatial / tau bonds of walker w
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "lanes_core.cuh"
 #include "qisg_internal.cuh"
@@ -19,7 +20,7 @@ namespace qisg {
 namespace {
 
 constexpr int kBlock = 256;
-static_assert(kBlock <= kLanesMaxThreads, "the LANES class-code buffer holds kLanesMaxThreads threads");
+static_assert(kBlock == kLanesThreads, "a LANES tile takes kLanesThreads threads");
 
 template <typename Word>
 struct LanesArgs {
@@ -31,7 +32,7 @@ struct LanesArgs {
   const unsigned long long *d_t;
   uint2 key;
   int64_t N, half_N;
-  FastDiv half_plane_div;
+  FastDiv half_plane_div, half_L_div;
   int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, sites_per_block;
   int tau_ap;
 };
@@ -48,9 +49,9 @@ __device__ __forceinline__ uint32_t bit_at(Word w, int lane) {
 
 // One half sweep (colour 0 = red, 1 = blue) of samples a0 + blockIdx.y:
 // block x is the tile of colour sites [x * tile_sites, (x+1) * tile_sites),
-// one thread per site (lanes_core.cuh).  Block 0 of the red pass clears the
+// one or four threads per site (lanes_core.cuh).  Block 0 of the red pass clears the
 // sample's bond counters, which the blue pass fills.
-template <typename Word, bool BLUE, int NREP, int NGC>
+template <typename Word, bool BLUE, int NREP, int NGC, int TPS>
 __global__ void __launch_bounds__(kBlock) lanes_half_sweep_kernel(LanesArgs<Word> p, int colour,
                                                                   int count_only, int64_t a0, int tile_sites) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -65,6 +66,7 @@ __global__ void __launch_bounds__(kBlock) lanes_half_sweep_kernel(LanesArgs<Word
   S.ctr_w = (DOM_SWEEP << 28) | (uint32_t)(a >> 6);
   S.t = (uint32_t)*p.d_t;
   S.hpd = p.half_plane_div;
+  S.hld = p.half_L_div;
   S.L = p.L;
   S.Lt = p.Lt;
   S.plane = p.plane;
@@ -77,7 +79,7 @@ __global__ void __launch_bounds__(kBlock) lanes_half_sweep_kernel(LanesArgs<Word
   S.tau_ap = p.tau_ap;
   const int64_t j0 = (int64_t)blockIdx.x * tile_sites;
   const int n = (int)(p.half_N - j0 < tile_sites ? p.half_N - j0 : tile_sites);
-  lanes_tile<Word, false, BLUE, NREP, NGC>(S, colour, (int)j0, n, count_only, colour == 0 && blockIdx.x == 0, smem_raw);
+  lanes_tile<Word, false, BLUE, NREP, NGC, TPS>(S, colour, (int)j0, n, count_only, colour == 0 && blockIdx.x == 0, smem_raw);
 }
 
 // Overlaps of the configurations at slot s (Appendix E.1): count the sites
@@ -257,6 +259,7 @@ LanesArgs<Word> make_args(qisg_handle *h) {
   p.plane = h->L * h->L;
   p.half_plane = p.plane / 2;
   p.half_plane_div = FastDiv((uint32_t)p.half_plane);
+  p.half_L_div = FastDiv((uint32_t)(h->L / 2));
   p.n_slots = h->n_slots;
   p.n_rep = h->n_rep;
   p.rpw = h->rpw;
@@ -266,51 +269,67 @@ LanesArgs<Word> make_args(qisg_handle *h) {
   return p;
 }
 
+template <typename Word, bool BLUE, int NREP, int NGC>
+void launch_half_sweep(const LanesArgs<Word> &p, dim3 grid, size_t smem, cudaStream_t st, int count_only, int64_t a0,
+                       int tile_sites, int tps) {
+  if (tps == 4)
+    lanes_half_sweep_kernel<Word, BLUE, NREP, NGC, 4><<<grid, kBlock, smem, st>>>(p, BLUE, count_only, a0, tile_sites);
+  else
+    lanes_half_sweep_kernel<Word, BLUE, NREP, NGC, 1><<<grid, kBlock, smem, st>>>(p, BLUE, count_only, a0, tile_sites);
+}
+
+template <typename Word, bool BLUE>
+int set_smem_limits() {
+  const void *fns[] = {(const void *)lanes_half_sweep_kernel<Word, BLUE, 0, 0, 1>, (const void *)lanes_half_sweep_kernel<Word, BLUE, 0, 0, 4>,
+                       (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 1, 1>, (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 1, 4>,
+                       (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 0, 1>, (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 0, 4>};
+  for (const void *f : fns) {
+    const int rc = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024), "shared memory");
+    if (rc) return rc;
+  }
+  return QISG_OK;
+}
+
 template <typename Word>
 int half_sweep_t(qisg_handle *h, int colour, int count_only) {
   LanesArgs<Word> p = make_args<Word>(h);
-  const size_t smem = lanes_tile_smem(p.plane, h->n_slots, h->n_rep);
-  // tiles of rows x 256 sites (rows <= 16, the counters' limit), as long as
-  // the grid keeps about four blocks per SM
+  if (!lanes_plane_fits(p.plane, h->n_slots, h->n_rep, 227 * 1024))
+    return fail(QISG_EINVAL, "LANES plane tables exceed shared memory");
+  const size_t smem = lanes_tile_smem(h->n_slots, h->n_rep);
   const int64_t n_launch_samples = h->per_sample_launch ? 1 : h->n_samples;
+  // four threads per site while one would leave the SMs half empty
+  const int tps = p.half_N * n_launch_samples < 1024LL * h->n_sm ? 4 : 1;
+  // tiles of rows x (256 / tps) sites (rows <= 16, the counters' limit), as
+  // long as the grid keeps about four blocks per SM
+  const int per = kBlock / tps;
   int rows = 16;
-  while (rows > 1 && ((p.half_N + 256LL * rows - 1) / (256LL * rows)) * n_launch_samples < 4LL * h->n_sm) rows >>= 1;
-  const int tile_sites = 256 * rows;
+  while (rows > 1 && ((p.half_N + per * (int64_t)rows - 1) / (per * (int64_t)rows)) * n_launch_samples < 4LL * h->n_sm) rows >>= 1;
+  const int tile_sites = per * rows;
   const int64_t blocks = (p.half_N + tile_sites - 1) / tile_sites;
   if (blocks > 0x7FFFFFFF) return fail(QISG_EINVAL, "lattice too large for one launch");
-  if (smem > 227 * 1024) return fail(QISG_EINVAL, "LANES plane tables exceed shared memory");
   static bool attr_set = false;
   if (!attr_set) {
-    cudaFuncSetAttribute(lanes_half_sweep_kernel<Word, false, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(lanes_half_sweep_kernel<Word, true, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(lanes_half_sweep_kernel<Word, false, 4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(lanes_half_sweep_kernel<Word, true, 4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(lanes_half_sweep_kernel<Word, false, 4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(lanes_half_sweep_kernel<Word, true, 4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    int rc = set_smem_limits<Word, false>();
+    if (!rc) rc = set_smem_limits<Word, true>();
+    if (rc) return rc;
     attr_set = true;
   }
   for (int64_t a0 = 0; a0 < h->n_samples; a0 += (h->per_sample_launch ? 1 : 65535)) {
     const int64_t na = h->per_sample_launch ? 1 : std::min<int64_t>(65535, h->n_samples - a0);
     const int tok = prof_begin(h, sweep_kind(colour));
     const dim3 grid((unsigned)blocks, (unsigned)na);
-    // compile-time replica count (loops unrolled) and word-group count (fewer
-    // registers) for the common cases
-    if (h->n_rep == 4 && h->n_groups == 1) {
-      if (colour == 1)
-        lanes_half_sweep_kernel<Word, true, 4, 1><<<grid, kBlock, smem, h->stream>>>(p, 1, count_only, a0, tile_sites);
-      else
-        lanes_half_sweep_kernel<Word, false, 4, 1><<<grid, kBlock, smem, h->stream>>>(p, 0, count_only, a0, tile_sites);
-    } else if (h->n_rep == 4) {
-      if (colour == 1)
-        lanes_half_sweep_kernel<Word, true, 4, 0><<<grid, kBlock, smem, h->stream>>>(p, 1, count_only, a0, tile_sites);
-      else
-        lanes_half_sweep_kernel<Word, false, 4, 0><<<grid, kBlock, smem, h->stream>>>(p, 0, count_only, a0, tile_sites);
-    } else {
-      if (colour == 1)
-        lanes_half_sweep_kernel<Word, true, 0, 0><<<grid, kBlock, smem, h->stream>>>(p, 1, count_only, a0, tile_sites);
-      else
-        lanes_half_sweep_kernel<Word, false, 0, 0><<<grid, kBlock, smem, h->stream>>>(p, 0, count_only, a0, tile_sites);
-    }
+    // a compile-time word-group count (fewer registers) for four replicas
+    auto go = [&](auto nrep, auto ngc) {
+      constexpr int R = decltype(nrep)::value, G = decltype(ngc)::value;
+      if (colour == 1) launch_half_sweep<Word, true, R, G>(p, grid, smem, h->stream, count_only, a0, tile_sites, tps);
+      else launch_half_sweep<Word, false, R, G>(p, grid, smem, h->stream, count_only, a0, tile_sites, tps);
+    };
+    using I0 = std::integral_constant<int, 0>;
+    using I1 = std::integral_constant<int, 1>;
+    using I4 = std::integral_constant<int, 4>;
+    if (h->n_rep == 4 && h->n_groups == 1) go(I4{}, I1{});
+    else if (h->n_rep == 4) go(I4{}, I0{});
+    else go(I0{}, I0{});
     prof_end(h, sweep_kind(colour), tok);
     h->launches++;
   }

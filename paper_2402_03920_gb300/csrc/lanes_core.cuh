@@ -1,4 +1,4 @@
-// Half sweep of one sample in the LANES packing, one thread per site.
+// Half sweep of one sample in the LANES packing.
 //
 // A 32- or 64-bit word holds replicas x walkers of the sample: lane =
 // (r - g*rpw) * n_slots + w in word group g = r / rpw.  The thread of a site
@@ -6,14 +6,33 @@
 // counts u_s (4 spatial bonds) and u_t (2 tau bonds) of every lane, and then
 // visits every (slot s, replica r): the walker w at slot s of replica r is
 // lane (r, w), whose draw R (one Philox call per (slot, replica quad, site,
-// sweep)) is compared with the threshold T[s][u_s][u_t] (Sec. 2.1).  Before
-// that visit the thread spreads the five count planes into a byte per lane
-// in shared memory (the 5-bit class code u_s + 8 u_t, four lanes per word),
-// so a lane's class is one load and its threshold one more, from a 32-entry
-// row per slot.  The flip mask of the site is built in registers and
-// applied once.  In the blue pass
-// the unsatisfied bonds after the flip are accumulated per lane in bit-sliced
-// counters and flushed per tile (every bond has exactly one blue end).
+// sweep)) is compared with the threshold T[s][u_s][u_t] (Sec. 2.1).
+//
+// What bounds it: integer issue, one Philox call per four updates and the
+// look-up of each lane's threshold.  So
+//   * the classes that always flip (u_t >= 1, u_s >= 2) share codes, which
+//     leaves a 4-bit class code; the four code planes become a byte per lane
+//     (code * 4, the byte offset in a 16-entry threshold row) by a 4 x 4
+//     nibble transposition, one operation per lane, kept in shared memory;
+//   * lane offsets and flip bits of each (slot, replica) are uniform over the
+//     block and come from a small table, so an update is: code byte, its
+//     threshold, compare, set a bit of the replica's 32-bit flip mask;
+//   * the first two Philox rounds separate: with the counter (site, t, s | q
+//     << 16, w) their products depend on the site alone or on (s, q) alone,
+//     so a call costs eight rounds and two exclusive-ors.
+// 22.8 thread instructions per update on the uneven batch, 54 with a byte
+// spread of five planes, plane tables in shared memory and whole Philox calls:
+// 20 sweeps of 512 instances took 265.6 ms, now 155.4.
+//
+// In the blue pass the unsatisfied bonds after the flip are accumulated per
+// lane in bit-sliced counters; after at most seven sites per thread each
+// plane is transposed across the warp (32 x 32 bits, five shuffles), so a
+// lane's sum over the warp is one popcount per plane (every bond has exactly
+// one blue end).
+//
+// TPS = 1: a thread per site.  TPS = 4: four warps share 32 sites, each
+// taking every fourth slot (and one 32-bit half of the words), for launches
+// with too few sites to fill the GPU.
 #pragma once
 
 #include "qisg_internal.cuh"
@@ -21,11 +40,12 @@
 namespace qisg {
 
 constexpr int kLanesMaxGroups = 2;    // word groups per site held in registers
-constexpr int kLanesKs = 7;           // u_s counter planes: <= 4 x 16 sites per thread
-constexpr int kLanesKt = 6;           // u_t counter planes: <= 2 x 16 sites per thread
-constexpr int kLanesMaxSitesPerThread = 16;
-constexpr int kLanesMaxThreads = 256;                    // block size the class-code buffer is sized for
-constexpr int kLanesCodeWords = kLanesMaxGroups * 16;    // per thread: 2 groups x 64 lanes, 4 per word
+constexpr int kLanesMaxSitesPerThread = 16;   // tile rows
+constexpr int kLanesKs = 5;           // u_s counter planes: <= 4 x 7 sites per thread
+constexpr int kLanesKt = 4;           // u_t counter planes: <= 2 x 7 sites per thread
+constexpr int kLanesFlushSites = 7;   // sites per thread between flushes of the counters
+constexpr int kLanesThreads = 256;                       // block size
+constexpr int kLanesCodeWords = kLanesMaxGroups * 16;    // per site: 2 groups x 64 lanes, 4 per word
 
 template <typename Word>
 struct LanesSample {
@@ -37,202 +57,328 @@ struct LanesSample {
   uint2 key;
   uint32_t ctr_w;                // (DOM_SWEEP << 28) | (a >> 6)
   uint32_t t;                    // sweep index
-  FastDiv hpd;
+  FastDiv hpd, hld;              // by plane / 2 and by L / 2
   int L, Lt, plane, half_plane, N, n_slots, n_rep, rpw, n_groups;
   int tau_ap;                    // antiperiodic along tau: the wrap tau bond flips sign
 };
 
-// Shared memory of one tile: the thresholds by class code, walker labels,
-// counter sums, the per-thread class codes and the plane tables.
-__host__ __device__ inline size_t lanes_tile_smem(int plane, int n_slots, int n_rep) {
-  size_t o = (size_t)(n_slots * 32 + n_rep * n_slots) * 4;   // T5_s, wa_s
+// Shared memory of one tile: threshold rows by class code, the lane table,
+// the Philox words of each (slot, quad), counter sums, the flips that the
+// TPS = 4 form exchanges, and the class codes.
+__host__ __device__ inline size_t lanes_tile_smem(int n_slots, int n_rep) {
+  const size_t sq = (size_t)n_slots * ((n_rep + 3) / 4);
+  size_t o = sq * 48 + (size_t)n_slots * 64;                  // lane table and Philox words, threshold rows
   o += (size_t)2 * kLanesMaxGroups * 64 * 4;                  // acc_s, acc_t
-  o += (size_t)kLanesCodeWords * kLanesMaxThreads * 4;
-  o = (o + 7) & ~size_t(7);
-  o += (size_t)plane * (8 + 2 + 1);                           // nb, s2d, Js
+  o += (size_t)2 * kLanesMaxGroups * kLanesThreads * 4;       // fx
+  o += (size_t)kLanesCodeWords * kLanesThreads * 4;
   return (o + 15) & ~size_t(15);
 }
 
-// Bits 0..3 of x moved to bits 0, 8, 16, 24.
-__device__ __forceinline__ uint32_t spread4(uint32_t x) { return ((x & 0xFu) * 0x00204081u) & 0x01010101u; }
+// The largest planes the packing takes: 11 bytes per site of the plane
+// beside the fixed tables have to stay within `limit` bytes.
+inline bool lanes_plane_fits(int plane, int n_slots, int n_rep, size_t limit) {
+  size_t o = (size_t)(n_slots * 32 + n_rep * n_slots) * 4 + (size_t)2 * kLanesMaxGroups * 64 * 4 +
+             (size_t)kLanesCodeWords * kLanesThreads * 4;
+  o = ((o + 7) & ~size_t(7)) + (size_t)plane * 11;
+  return ((o + 15) & ~size_t(15)) <= limit;
+}
 
 template <bool CG, typename Word>
 __device__ __forceinline__ Word ld_word(const Word *p) {
   return CG ? __ldcg(p) : *p;
 }
 
-// Sites [j0, j0 + n) of one colour; every thread of the block must call it.
-// NREP > 0: the sample has exactly NREP replicas (a compile-time count lets
-// the per-slot replica loop unroll without bound checks).  NGC > 0: exactly
-// NGC word groups per site (registers for those only).
+// 32 x 32 bit transposition over the warp: bit i of lane l's result is bit l
+// of lane i's v.
+__device__ __forceinline__ uint32_t warp_transpose32(uint32_t v, int lane) {
+  uint32_t o = __shfl_xor_sync(0xffffffffu, v, 16);
+  v = __byte_perm(v, o, (lane & 16) ? 0x3276 : 0x5410);
+  o = __shfl_xor_sync(0xffffffffu, v, 8);
+  v = __byte_perm(v, o, (lane & 8) ? 0x3715 : 0x6240);
+#pragma unroll
+  for (int k = 4; k > 0; k >>= 1) {
+    const uint32_t m = k == 4 ? 0x0F0F0F0Fu : k == 2 ? 0x33333333u : 0x55555555u;
+    o = __shfl_xor_sync(0xffffffffu, v, k);
+    const bool hi = (lane & k) != 0;
+    o = __funnelshift_l(o, o, hi ? 32 - k : k);
+    v = mux(hi ? ~m : m, v, o);
+  }
+  return v;
+}
+
+// Class code planes of 32 lanes: code = u_s at u_t = 0, else 8 + (u_s & 1) +
+// 2 [u_t = 2] + 4 [u_s >= 2] (those with bit 2 set always flip).  The codes
+// times 4 go to eight words, a byte per lane: lane l is byte l >> 3 of word
+// 2 (l & 3) + ((l >> 2) & 1) (kLanesThreads words apart).
+__device__ __forceinline__ void lanes_store_codes(uint32_t *cw, uint32_t P0, uint32_t P1, uint32_t P2, uint32_t Q0,
+                                                  uint32_t Q1) {
+  const uint32_t nz = Q0 | Q1;
+  const uint32_t c1 = mux(nz, Q1, P1), c2 = P2 | (nz & P1);
+  // 4 x 4 transposition of the planes' nibbles: bit i of nibble k of word j
+  // becomes bit j of nibble k of plane i
+  const uint32_t a0 = mux(0x55555555u, P0, c1 << 1), a1 = mux(0x55555555u, P0 >> 1, c1);
+  const uint32_t a2 = mux(0x55555555u, c2, nz << 1), a3 = mux(0x55555555u, c2 >> 1, nz);
+  const uint32_t w[4] = {mux(0x33333333u, a0, a2 << 2), mux(0x33333333u, a1, a3 << 2),
+                         mux(0x33333333u, a0 >> 2, a2), mux(0x33333333u, a1 >> 2, a3)};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    cw[(2 * j) * kLanesThreads] = (w[j] << 2) & 0x3C3C3C3Cu;
+    cw[(2 * j + 1) * kLanesThreads] = (w[j] >> 2) & 0x3C3C3C3Cu;
+  }
+}
+
+// Sites [j0, j0 + n) of one colour; every thread of the block must call it
+// (kLanesThreads threads).  NREP > 0: the sample has exactly NREP <= 4
+// replicas (one quad).  NGC > 0: exactly NGC word groups per site (registers
+// for those only).
 // CG: read mutable state through L2 only (inside a persistent kernel).
 // zero_U: clear this sample's bond counters first (red pass, one tile).
-template <typename Word, bool CG, bool BLUE, int NREP = 0, int NGC = 0>
+template <typename Word, bool CG, bool BLUE, int NREP = 0, int NGC = 0, int TPS = 1>
 __device__ void lanes_tile(const LanesSample<Word> &S, int colour, int j0, int n, int count_only, bool zero_U,
                            unsigned char *smem) {
-  constexpr int W = (int)sizeof(Word) * 8;
+  constexpr int W = (int)sizeof(Word) * 8, HW = W / 32;
+  constexpr int MG = NGC > 0 ? NGC : kLanesMaxGroups;   // word groups held in registers
+  constexpr int MH = MG * HW;                             // 32-bit halves of them
+  constexpr int NH = TPS == 1 ? MH : (MH + TPS - 1) / TPS;   // halves of this thread
+  constexpr int SPI = kLanesThreads / TPS;                // sites per iteration of the block
+  static_assert(SPI % 32 == 0, "a warp's threads share their part of the slots");
   const int n_slots = S.n_slots, n_rep = NREP > 0 ? NREP : S.n_rep, plane = S.plane, hp = S.half_plane;
-  uint32_t *T5_s = reinterpret_cast<uint32_t *>(smem);   // [slot][code], code = u_s + 8 u_t
-  int *wa_s = reinterpret_cast<int *>(T5_s + n_slots * 32);
-  int *acc_s = wa_s + n_rep * n_slots;                 // [group][lane]
+  const int nq = NREP > 0 ? 1 : (n_rep + 3) >> 2, sq = n_slots * nq;
+  const int NG = NGC > 0 ? NGC : S.n_groups;             // 1 or 2
+  uint4 *inf = reinterpret_cast<uint4 *>(smem);          // [s][q][2]: {code offset, flip bit} of four replicas
+  uint4 *phx = inf + 2 * sq;                               // [s][q]: the (s, q) words of Philox rounds 1 and 2
+  uint32_t *T16 = reinterpret_cast<uint32_t *>(phx + sq);   // [slot][code]
+  int *acc_s = reinterpret_cast<int *>(T16 + n_slots * 16);   // [group][lane]
   int *acc_t = acc_s + kLanesMaxGroups * 64;
-  uint32_t *code_s = reinterpret_cast<uint32_t *>(acc_t + kLanesMaxGroups * 64);   // [word][thread]
-  size_t off = (size_t)(n_slots * 32 + n_rep * n_slots) * 4 + (size_t)2 * kLanesMaxGroups * 64 * 4 +
-               (size_t)kLanesCodeWords * kLanesMaxThreads * 4;
-  off = (off + 7) & ~size_t(7);
-  uint2 *nb = reinterpret_cast<uint2 *>(smem + off);
-  uint16_t *s2d = reinterpret_cast<uint16_t *>(nb + plane);
-  uint8_t *Js = reinterpret_cast<uint8_t *>(s2d + plane);
+  uint32_t *fx = reinterpret_cast<uint32_t *>(acc_t + kLanesMaxGroups * 64);   // [half][part][site]
+  uint32_t *code_s = fx + 2 * kLanesMaxGroups * kLanesThreads;                 // [word][site]
 
   __syncthreads();   // a previous tile is done with shared memory
-  for (int i = threadIdx.x; i < n_slots * 32; i += blockDim.x) {
-    const int sl = i >> 5, us = i & 7, ut = (i >> 3) & 3;
-    T5_s[i] = (us <= 4 && ut <= 2) ? S.T[sl * 15 + us * 3 + ut] : 0xFFFFFFFFu;
+  for (int i = threadIdx.x; i < n_slots * 16; i += kLanesThreads) {
+    const int c = i & 15, us = c < 8 ? c : c & 1, ut = c < 8 ? 0 : 1 + ((c >> 1) & 1);
+    T16[i] = (c < 8 ? us <= 4 : !(c & 4)) ? S.T[(i >> 4) * 15 + us * 3 + ut] : 0xFFFFFFFFu;
   }
-  for (int i = threadIdx.x; i < n_rep * n_slots; i += blockDim.x) wa_s[i] = CG ? __ldcg(S.walker + i) : S.walker[i];
+  for (int i = threadIdx.x; i < sq; i += kLanesThreads) {
+    const int s = i / nq, q = i - s * nq;
+    uint32_t e[8];
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const int r = 4 * q + jj;
+      uint32_t off = 0, bit = 0;
+      if (r < n_rep) {
+        const int w = CG ? __ldcg(S.walker + r * n_slots + s) : S.walker[r * n_slots + s];
+        const int g = r / S.rpw, l = (r - g * S.rpw) * n_slots + w;   // lane of group g
+        off = (uint32_t)((g * 16 + (l >> 5) * 8 + 2 * (l & 3) + ((l >> 2) & 1)) * kLanesThreads * 4 + ((l & 31) >> 3));
+        bit = 1u << w;
+      }
+      e[2 * jj] = off;
+      e[2 * jj + 1] = bit;
+    }
+    inf[2 * i] = make_uint4(e[0], e[1], e[2], e[3]);
+    inf[2 * i + 1] = make_uint4(e[4], e[5], e[6], e[7]);
+    const uint32_t cz = (uint32_t)s | ((uint32_t)q << 16);
+    const uint32_t x1 = __umulhi(kPhiloxM1, cz) ^ S.t ^ S.key.x;
+    phx[i] = make_uint4(kPhiloxM1 * cz, __umulhi(kPhiloxM0, x1), kPhiloxM0 * x1, 0u);
+  }
   if (BLUE)
-    for (int i = threadIdx.x; i < 2 * kLanesMaxGroups * 64; i += blockDim.x) acc_s[i] = 0;
-  for (int i2 = threadIdx.x; i2 < plane; i2 += blockDim.x) {
-    const int L = S.L;
-    const int y = i2 / L, x = i2 - y * L;
-    const int xp = x + 1 == L ? 0 : x + 1, xm = x == 0 ? L - 1 : x - 1;
-    const int yp = y + 1 == L ? 0 : y + 1, ym = y == 0 ? L - 1 : y - 1;
-    nb[i2] = make_uint2((uint32_t)(xp + L * y) | ((uint32_t)(xm + L * y) << 16),
-                        (uint32_t)(x + L * yp) | ((uint32_t)(x + L * ym) << 16));
-    s2d[((x + y) & 1) * hp + (i2 >> 1)] = (uint16_t)i2;
-    Js[i2] = S.J[i2];
-  }
+    for (int i = threadIdx.x; i < 2 * kLanesMaxGroups * 64; i += kLanesThreads) acc_s[i] = 0;
   if (zero_U)
-    for (int i = threadIdx.x; i < 2 * n_rep * n_slots; i += blockDim.x) S.U[i] = 0;
+    for (int i = threadIdx.x; i < 2 * n_rep * n_slots; i += kLanesThreads) S.U[i] = 0;
   __syncthreads();
 
-  constexpr int MG = NGC > 0 ? NGC : kLanesMaxGroups;   // word groups held in registers
-  const int NG = NGC > 0 ? NGC : S.n_groups;             // 1 or 2
-  const uint32_t Lt = (uint32_t)S.Lt;
-  VCount<Word, kLanesKs> cs[MG];
-  VCount<Word, kLanesKt> ct[MG];
+  const int sl = TPS == 1 ? (int)threadIdx.x : (int)threadIdx.x % SPI;   // site of the iteration
+  const int part = TPS == 1 ? 0 : (int)threadIdx.x / SPI;
+  const uint32_t Lt = (uint32_t)S.Lt, L = (uint32_t)S.L;
+  VCount<uint32_t, kLanesKs> cs[NH];
+  VCount<uint32_t, kLanesKt> ct[NH];
   if (BLUE)
 #pragma unroll
-    for (int g = 0; g < MG; ++g) {
-      cs[g].zero();
-      ct[g].zero();
+    for (int h = 0; h < NH; ++h) {
+      cs[h].zero();
+      ct[h].zero();
     }
 
-  for (int base = 0; base < n; base += blockDim.x) {
-    const int jr = base + threadIdx.x;
-    if (jr < n) {
-      const uint32_t j = (uint32_t)(j0 + jr);
-      const uint32_t tau = S.hpd.div(j);
-      const uint32_t i2 = s2d[((colour + tau) & 1) * hp + (j - tau * hp)];
-      const uint2 nv = nb[i2];
-      const uint32_t offt = tau * plane;
-      const uint32_t site = i2 + offt;
-      const uint32_t i_xp = (nv.x & 0xFFFFu) + offt, i_xm = (nv.x >> 16) + offt;
-      const uint32_t i_yp = (nv.y & 0xFFFFu) + offt, i_ym = (nv.y >> 16) + offt;
+  int n_it = 0;   // sites per thread in the counters
+  for (int base = 0; base < n; base += SPI) {
+    const bool live = base + sl < n;
+    uint32_t site = 0;
+    uint32_t sc[NH], P0[NH], P1[NH], P2[NH], Q0[NH], Q1[NH], fw[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) sc[h] = P0[h] = P1[h] = P2[h] = Q0[h] = Q1[h] = fw[h] = 0;
+    if (live) {
+      const uint32_t j = (uint32_t)(j0 + base + sl);
+      const uint32_t tau = S.hpd.div(j), rem = j - tau * (uint32_t)hp;
+      const uint32_t y = S.hld.div(rem), x = 2 * (rem - y * (L >> 1)) + ((y + tau + (uint32_t)colour) & 1u);
+      const uint32_t i2 = x + L * y, offt = tau * (uint32_t)plane;
+      const uint32_t ixp = x + 1 == L ? i2 + 1 - L : i2 + 1, ixm = x == 0 ? i2 + L - 1 : i2 - 1;
+      const uint32_t iyp = y + 1 == L ? x : i2 + L, iym = y == 0 ? i2 + plane - L : i2 - L;
+      site = i2 + offt;
       const uint32_t i_tp = i2 + (tau + 1 == Lt ? 0u : offt + plane);
       const uint32_t i_tm = i2 + (tau == 0 ? (Lt - 1) * plane : offt - plane);
       // the antiperiodic wrap bond is unsatisfied when its spins agree
-      const Word gtp = ones_if<Word>(S.tau_ap && tau + 1 == Lt), gtm = ones_if<Word>(S.tau_ap && tau == 0);
-      const uint8_t jh = Js[i2];
-      const Word Jxp = ones_if<Word>(jh & 1u), Jyp = ones_if<Word>(jh & 2u);
-      const Word Jxm = ones_if<Word>(Js[nv.x >> 16] & 1u);
-      const Word Jym = ones_if<Word>(Js[nv.y >> 16] & 2u);
-      Word sc[MG], P0[MG], P1[MG], P2[MG], Q0[MG], Q1[MG], fw[MG];
+      const uint32_t gtp = ones_if<uint32_t>(S.tau_ap && tau + 1 == Lt), gtm = ones_if<uint32_t>(S.tau_ap && tau == 0);
+      const uint32_t jh = S.J[i2];
+      const uint32_t Jxp = 0u - (jh & 1u), Jyp = 0u - (jh >> 1), Jxm = 0u - (S.J[ixm] & 1u);
+      const uint32_t Jym = 0u - ((uint32_t)S.J[iym] >> 1);
+      auto bonds = [&](int h, uint32_t c, uint32_t xp, uint32_t xm, uint32_t yp, uint32_t ym, uint32_t up, uint32_t dn) {
+        const uint32_t b1 = c ^ xp ^ Jxp, b2 = c ^ xm ^ Jxm, b3 = c ^ yp ^ Jyp, b4 = c ^ ym ^ Jym;
+        const uint32_t t1 = c ^ up ^ gtp, t2 = c ^ dn ^ gtm;
+        const uint32_t s1 = b1 ^ b2 ^ b3, c1 = maj3(b1, b2, b3), c2 = s1 & b4;
+        sc[h] = c;
+        P0[h] = s1 ^ b4;
+        P1[h] = c1 ^ c2;
+        P2[h] = c1 & c2;
+        Q0[h] = t1 ^ t2;
+        Q1[h] = t1 & t2;
+      };
+      if constexpr (TPS == 1) {
 #pragma unroll
-      for (int g = 0; g < MG; ++g) {
-        sc[g] = P0[g] = P1[g] = P2[g] = Q0[g] = Q1[g] = fw[g] = 0;
-        if (g < NG) {
-          const Word *w = S.spins + (size_t)g * S.N;
-          const Word c = ld_word<CG>(w + site);
-          const Word b1 = c ^ ld_word<CG>(w + i_xp) ^ Jxp;
-          const Word b2 = c ^ ld_word<CG>(w + i_xm) ^ Jxm;
-          const Word b3 = c ^ ld_word<CG>(w + i_yp) ^ Jyp;
-          const Word b4 = c ^ ld_word<CG>(w + i_ym) ^ Jym;
-          const Word t1 = c ^ ld_word<CG>(w + i_tp) ^ gtp;
-          const Word t2 = c ^ ld_word<CG>(w + i_tm) ^ gtm;
-          const Word s1 = b1 ^ b2 ^ b3, c1 = maj3(b1, b2, b3);
-          sc[g] = c;
-          P0[g] = s1 ^ b4;
-          const Word c2 = s1 & b4;
-          P1[g] = c1 ^ c2;
-          P2[g] = c1 & c2;
-          Q0[g] = t1 ^ t2;
-          Q1[g] = t1 & t2;
+        for (int g = 0; g < MG; ++g)
+          if (g < NG) {
+            const Word *w = S.spins + (size_t)g * S.N;
+            const Word c = ld_word<CG>(w + site), xp = ld_word<CG>(w + ixp + offt), xm = ld_word<CG>(w + ixm + offt);
+            const Word yp = ld_word<CG>(w + iyp + offt), ym = ld_word<CG>(w + iym + offt);
+            const Word up = ld_word<CG>(w + i_tp), dn = ld_word<CG>(w + i_tm);
+#pragma unroll
+            for (int k = 0; k < HW; ++k)
+              bonds(g * HW + k, (uint32_t)(c >> (32 * k)), (uint32_t)(xp >> (32 * k)), (uint32_t)(xm >> (32 * k)),
+                    (uint32_t)(yp >> (32 * k)), (uint32_t)(ym >> (32 * k)), (uint32_t)(up >> (32 * k)),
+                    (uint32_t)(dn >> (32 * k)));
+          }
+      } else if (part < NG * HW) {   // one half per part (MH <= TPS)
+        const int g = part / HW, k = part - g * HW;
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(S.spins + (size_t)g * S.N) + k;
+        auto ld = [&](uint32_t i) { return ld_word<CG>(w + (size_t)i * HW); };
+        bonds(0, ld(site), ld(ixp + offt), ld(ixm + offt), ld(iyp + offt), ld(iym + offt), ld(i_tp), ld(i_tm));
+      }
+    }
+    if (!count_only) {
+      if (live) {
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+          const int hh = TPS == 1 ? h : part;
+          if (hh < NG * HW)
+            lanes_store_codes(code_s + ((hh / HW) * 16 + (hh % HW) * 8) * kLanesThreads + sl, P0[h], P1[h], P2[h],
+                              Q0[h], Q1[h]);
         }
       }
-      if (!count_only) {
-        // class codes of every lane, a byte each: word g*16 + l/4 of this
-        // thread holds lanes l .. l+3 of group g
-        uint32_t *cw = code_s + threadIdx.x;
+      if (TPS > 1) __syncthreads();   // the codes of a site come from, and go to, several warps
+      Word flips[MG];
+#pragma unroll
+      for (int g = 0; g < MG; ++g) flips[g] = 0;
+      if (live) {
+        // Philox rounds 1 and 2 of the site: A, y2 and B depend on it alone
+        const uint2 key = S.key;
+        const uint32_t z1 = __umulhi(kPhiloxM0, site) ^ S.ctr_w ^ key.y;
+        const uint32_t A = __umulhi(kPhiloxM1, z1) ^ (key.x + kPhiloxW0), y2 = kPhiloxM1 * z1;
+        const uint32_t B = (kPhiloxM0 * site) ^ (key.y + kPhiloxW1);
+        const unsigned char *cb = reinterpret_cast<const unsigned char *>(code_s + sl);
+        for (int q = 0; q < nq; ++q) {
+          uint32_t f[4] = {0, 0, 0, 0};   // flip bits of the quad's replicas, by walker
+#pragma unroll 2
+          for (int s = part; s < n_slots; s += TPS) {
+            const int e = s * nq + q;
+            const uint4 ph = phx[e], i0 = inf[2 * e], i1 = inf[2 * e + 1];
+            uint4 c = make_uint4(A ^ ph.x, y2, ph.y ^ B, ph.z);
+            uint2 k = make_uint2(key.x + 2 * kPhiloxW0, key.y + 2 * kPhiloxW1);
+#pragma unroll
+            for (int i = 2; i < 10; ++i) {
+              const uint32_t lo0 = kPhiloxM0 * c.x, hi0 = __umulhi(kPhiloxM0, c.x);
+              const uint32_t lo1 = kPhiloxM1 * c.z, hi1 = __umulhi(kPhiloxM1, c.z);
+              c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
+              k.x += kPhiloxW0;
+              k.y += kPhiloxW1;
+            }
+            const unsigned char *row = reinterpret_cast<const unsigned char *>(T16 + s * 16);
+            // a draw flips iff R < T or T = 2^32 - 1: with R cut to 2^32 - 2
+            // (no finite T exceeds that) both are R < T
+            auto lane = [&](int jj, uint32_t off, uint32_t bit, uint32_t R) {
+              const uint32_t thr = *reinterpret_cast<const uint32_t *>(row + cb[off]);
+              if (min(R, 0xFFFFFFFEu) < thr) f[jj] |= bit;
+            };
+            lane(0, i0.x, i0.y, c.x);
+            lane(1, i0.z, i0.w, c.y);
+            lane(2, i1.x, i1.y, c.z);
+            lane(3, i1.z, i1.w, c.w);
+          }
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) {
+            const int r = 4 * q + jj;
+            if (r < n_rep) {
+              const int g = MG > 1 && r >= S.rpw ? 1 : 0;   // n_groups <= 2
+              const Word m = (Word)f[jj] << ((r - g * S.rpw) * n_slots);
+              if (MG > 1 && g) flips[MG - 1] |= m;
+              else flips[0] |= m;
+            }
+          }
+        }
+      }
+      if constexpr (TPS == 1) {
 #pragma unroll
         for (int g = 0; g < MG; ++g)
           if (g < NG) {
 #pragma unroll
-            for (int h = 0; h < W / 32; ++h) {
-              const uint32_t a0 = (uint32_t)(P0[g] >> (32 * h)), a1 = (uint32_t)(P1[g] >> (32 * h));
-              const uint32_t a2 = (uint32_t)(P2[g] >> (32 * h)), a3 = (uint32_t)(Q0[g] >> (32 * h));
-              const uint32_t a4 = (uint32_t)(Q1[g] >> (32 * h));
+            for (int k = 0; k < HW; ++k) fw[g * HW + k] = (uint32_t)(flips[g] >> (32 * k));
+            if (flips[g]) {
+              Word c = 0;
 #pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const uint32_t c = spread4(a0 >> (4 * i)) | (spread4(a1 >> (4 * i)) << 1) |
-                                   (spread4(a2 >> (4 * i)) << 2) | (spread4(a3 >> (4 * i)) << 3) |
-                                   (spread4(a4 >> (4 * i)) << 4);
-                cw[(g * 16 + h * 8 + i) * kLanesMaxThreads] = c;
-              }
+              for (int k = 0; k < HW; ++k) c |= (Word)(sc[g * HW + k] ^ fw[g * HW + k]) << (32 * k);
+              S.spins[(size_t)g * S.N + site] = c;
             }
           }
-        for (int s = 0; s < n_slots; ++s) {
-          const uint32_t *Trow = T5_s + s * 32;
-          for (int q = 0; 4 * q < n_rep; ++q) {
-            const uint4 R4 = philox(make_uint4(site, S.t, (uint32_t)s | ((uint32_t)q << 16), S.ctr_w), S.key);
+      } else {
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-              const int r = 4 * q + jj;
-              if (r >= n_rep) break;
-              const int g = (MG > 1 && r >= S.rpw) ? 1 : 0;   // n_groups <= 2
-              const int lane = (r - g * S.rpw) * n_slots + wa_s[r * n_slots + s];
-              const uint32_t word = cw[(g * 16 + (lane >> 2)) * kLanesMaxThreads];
-              const uint32_t thr = Trow[(word >> (8 * (lane & 3))) & 31u];
-              if (thr == 0xFFFFFFFFu || pick4(R4, jj) < thr) {
-                if (MG > 1 && g) fw[MG - 1] |= Word(1) << lane;
-                else fw[0] |= Word(1) << lane;
-              }
-            }
+        for (int hh = 0; hh < MH; ++hh) fx[hh * kLanesThreads + threadIdx.x] = (uint32_t)(flips[hh / HW] >> (32 * (hh % HW)));
+        __syncthreads();
+        if (live && part < NG * HW) {
+#pragma unroll
+          for (int u = 0; u < TPS; ++u) fw[0] |= fx[part * kLanesThreads + u * SPI + sl];
+          if (fw[0]) {
+            const int g = part / HW, k = part - g * HW;
+            reinterpret_cast<uint32_t *>(S.spins + (size_t)g * S.N)[(size_t)site * HW + k] = sc[0] ^ fw[0];
           }
         }
-#pragma unroll
-        for (int g = 0; g < MG; ++g)
-          if (g < NG && fw[g]) {
-            Word *w = S.spins + (size_t)g * S.N + site;
-            *w = sc[g] ^ fw[g];
-          }
       }
-      if (BLUE) {
+    }
+    if (BLUE) {
+      // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau);
+      // threads without a site add zeros
 #pragma unroll
-        for (int g = 0; g < MG; ++g)
-          if (g < NG) {
-            // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
-            const Word f = fw[g];
-            const Word v1 = P1[g] ^ (f & P0[g]);
-            const Word v2 = mux(f, ~(P0[g] | P1[g] | P2[g]), P2[g]);
-            const Word w1 = mux(f, ~(Q0[g] | Q1[g]), Q1[g]);
-            cs[g].add3(P0[g], v1, v2);
-            ct[g].add2(Q0[g], w1);
+      for (int h = 0; h < NH; ++h) {
+        const uint32_t f = fw[h];
+        cs[h].add3(P0[h], P1[h] ^ (f & P0[h]), mux(f, ~(P0[h] | P1[h] | P2[h]), P2[h]));
+        ct[h].add2(Q0[h], mux(f, ~(Q0[h] | Q1[h]), Q1[h]));
+      }
+      if (++n_it == kLanesFlushSites || base + SPI >= n) {
+        // the planes in use (u_s <= 4, u_t <= 2 a site)
+        const int ks = 32 - __clz(4 * n_it), kt = ks - 1, lane = threadIdx.x & 31;
+#pragma unroll
+        for (int h = 0; h < NH; ++h) {
+          const int hh = TPS == 1 ? h : part;
+          if (hh < NG * HW) {   // uniform over the warp
+            int us = 0, ut = 0;
+#pragma unroll
+            for (int i = 0; i < kLanesKs; ++i)
+              if (i < ks) us += __popc(warp_transpose32(cs[h].p[i], lane)) << i;
+#pragma unroll
+            for (int i = 0; i < kLanesKt; ++i)
+              if (i < kt) ut += __popc(warp_transpose32(ct[h].p[i], lane)) << i;
+            const int at = (hh / HW) * W + (hh % HW) * 32 + lane;
+            if (us) atomicAdd(&acc_s[at], us);
+            if (ut) atomicAdd(&acc_t[at], ut);
           }
+          cs[h].zero();
+          ct[h].zero();
+        }
+        n_it = 0;
       }
     }
   }
   if (BLUE) {
-#pragma unroll
-    for (int g = 0; g < MG; ++g)
-      if (g < NG) {   // uniform across the block
-        flush_counter<Word, kLanesKs, 1>(cs[g], acc_s + g * W);
-        flush_counter<Word, kLanesKt, 1>(ct[g], acc_t + g * W);
-      }
     __syncthreads();
-    for (int i = threadIdx.x; i < NG * W; i += blockDim.x) {
-      const int g = i / W, lane = i - g * W;
-      const int rl = lane / n_slots, w = lane - rl * n_slots;
+    for (int i = threadIdx.x; i < NG * W; i += kLanesThreads) {
+      const int g = i / W, l = i - g * W;
+      const int rl = l / n_slots, w = l - rl * n_slots;
       const int r = g * S.rpw + rl;
       if (rl >= S.rpw || r >= n_rep) continue;
       unsigned long long *u = S.U + ((size_t)r * n_slots + w) * 2;

@@ -107,6 +107,23 @@ def test_small_geometries_bit_exact(qisg, L, Lt, n_slots, n_rep, W, n_samples):
             assert_same_state(inst, st, what=f"L={L} Lt={Lt} after {st.t}")
 
 
+@pytest.mark.parametrize("L,Lt,n_slots,n_rep,W,n_samples,hi,n", [
+    (6, 10, 21, 5, 64, 900, 0.5, 3),    # one thread per site: two word groups, two quads, a tile of 180 sites
+    (8, 64, 2, 3, 64, 640, 0.5, 2),     # one thread per site, eight sites each: two flushes of the counters
+    (4, 6, 32, 4, 64, 3, 12.0, 6),      # four threads per site: 48 of 64 sites, thresholds 0 and 2^32 - 1
+    (6, 6, 1, 7, 32, 2, 0.5, 6),        # fewer slots than threads per site
+    (4, 6, 16, 4, 64, 6600, 12.0, 2),   # one thread per site with thresholds 0
+])
+def test_tile_forms_bit_exact(qisg, L, Lt, n_slots, n_rep, W, n_samples, hi, n):
+    inst, ladder = make(qisg, L, Lt, 0.2, hi, n_slots, 0.9, n_rep, n_samples, 5 + L, word_bits=W,
+                        layout=qisg.QISG_LAYOUT_LANES)
+    st = oracle_state(ladder, L, Lt, n_rep, 5 + L, 0, n_samples)
+    with inst:
+        inst.sweep(n)
+        oracle.run(st, n)
+        assert_same_state(inst, st, what=f"L={L} Lt={Lt} {n_slots} slots {n_rep} replicas")
+
+
 def test_per_sample_launch_equals_batched_launch(qisg):
     a, ladder = make(qisg, 8, 16, 0.25, 0.45, 8, 1.0, 4, 5, 9, layout=qisg.QISG_LAYOUT_LANES,
                      per_sample_launch=1)
