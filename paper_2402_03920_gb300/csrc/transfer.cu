@@ -10,22 +10,30 @@
 // configuration (top bit 0), jP = e^{k_tau} / (e^{k_tau} + e^{-k_tau}) and
 // jM = e^{-k_tau} / (...)  (Eq. (expH1) with exp(-2 k_tau) = tanh(k Gamma)).
 //
-// On this GPU the work is bound by FP64 issue, not by HBM (about 1.25 TFLOP/s
-// of FP64 against 6.7 TB/s): since jP + jM = 1, a round's pair update is
-// d = x - y, x' = y + jP d, y' = x - jP d, one subtraction and two fused
-// multiply-adds for two elements instead of four multiplies and two adds.
-// That is the paper's formula rearranged, so the result differs from the
-// plain evaluation by rounding only (relative 1e-15 in norm after 25
-// rounds).  Rounds are fused in shared-memory tiles so that the vector
-// crosses HBM once per pass instead of once per round: a tile
-// fixes all index bits except a low run [0, c) (c = 5: 32 consecutive
-// doubles, 256-byte segments) and the bits [lo, hi) of the pass's rounds;
-// the first pass takes bits [0, 12) whole.  The last pass pairs every tile
-// with its bit complement (the tile holding 2^{n} - 1 - n for each n) for
-// the parity factor.  w is not stored: each thread computes the bond energy
-// of its index with bit rotations and popcounts and looks exp((k/2) E) up in
-// a table of the 2 L^2 + 1 possible energies, computed once on the host in
-// FP64.  Rounds run in ascending j for every element, as in the paper.
+// What bounds it: FP64 issue (about 0.62e12 FP64 operations a second here;
+// the vector crosses HBM three times at L = 5, 0.12 ms of 6.8 TB/s).  So the
+// rounds are taken with the factor jP outside: with r = jM / jP a pair update
+// is x' = x + r y, y' = y + r x, one fused multiply-add per element, and jP^{L^2}
+// goes into the table of w used on load.  (jP x + jM y as y + jP (x - y) takes
+// three operations per pair: 1.351 ms at L = 5 in that form, 0.891 now.)  This is the
+// paper's formula rearranged: the results differ by rounding only (relative
+// 1e-15 in norm after 25 rounds), and the scaled values stay below the
+// plain ones until the last round.
+//
+// Rounds are fused in tiles so that the vector crosses HBM once per pass
+// instead of once per round: a tile fixes all index bits except a low run
+// [0, c) (c = 5: 32 consecutive doubles, 256-byte segments) and the bits
+// [lo, hi) of the pass's rounds; the first pass takes bits [0, 12) whole.
+// Within a tile a thread takes up to four rounds on 16 elements in registers
+// (three in the last pass, which holds a tile and its complement), so shared
+// memory is crossed once per four rounds and, where the run of low bits makes
+// a warp's accesses whole segments, the first group reads HBM and the last
+// group writes it directly.  The last pass pairs every tile with its bit
+// complement (the tile holding 2^{n} - 1 - n for each n) for the parity
+// factor, again in registers.  w is not stored: each thread computes the bond
+// energy of its index with bit rotations and popcounts and looks exp((k/2) E)
+// up in a table of the 2 L^2 + 1 possible energies, computed once on the host
+// in FP64.  Rounds run in ascending j for every element, as in the paper.
 #include <cmath>
 #include <vector>
 
@@ -38,7 +46,8 @@ constexpr int kTransferBlock = 256;
 constexpr int kTileLog = 12;   // 4096 doubles, 32 KB of shared memory
 
 struct TransferArgs {
-  double jP, jM, parity;
+  double r, pr;               // jM / jP and parity times it
+  double jPn;                 // jP^{L^2}
   double wtab[51];            // exp((k/2) E) for E = -2 L^2, -2 L^2 + 2, ..., 2 L^2 (L <= 5)
   int L2;                     // L^2
   int sumJ;                   // sum of the couplings
@@ -50,97 +59,169 @@ struct TransferArgs {
   int L;
 };
 
-// exp((k/2) E(n)) for the L^2-bit configuration n (bit i set <=> S_i = -1):
+// Table index of the L^2-bit configuration n (bit i set <=> S_i = -1):
 // E = sum_bonds J S S = sum J - 2 (sum of J over unsatisfied bonds).
-__device__ __forceinline__ double boltzmann(const TransferArgs &a, uint32_t n) {
+__device__ __forceinline__ int energy_index(const TransferArgs &a, uint32_t n) {
   const int L = a.L;
   const uint32_t vx = ((n >> 1) & a.not_row_last) | ((n << (L - 1)) & a.row_last);          // spin at (x1+1, x2)
   const uint32_t vy = ((n >> L) & a.not_col_last) | ((n << (L * (L - 1))) & a.col_last);    // spin at (x1, x2+1)
   const uint32_t ux = n ^ vx, uy = n ^ vy;                                                    // unsatisfied bonds
   const int s = __popc(ux & a.jxp) - __popc(ux & a.jxn) + __popc(uy & a.jyp) - __popc(uy & a.jyn);
   const int E = a.sumJ - 2 * s;
-  return a.wtab[(E + 2 * a.L2) >> 1];
+  return (E + 2 * a.L2) >> 1;
 }
+
+// One pass: the tile's geometry and what the pass does besides its rounds.
+struct PassArgs {
+  int c, lo, hi;      // tile bits: [0, c) and the rounds' bits [lo, hi)
+  int first, last;    // multiply by w on load / parity factor and w at the end
+  int nb;             // index bits
+};
 
 // Global index of tile element t: bits [0, c) of t -> bits [0, c), the next
-// (hi - lo) bits -> bits [lo, hi), the fixed bits f -> [c, lo) then [hi, n).
-__device__ __forceinline__ uint32_t tile_index(uint32_t t, uint32_t f, int c, int lo, int hi) {
-  const uint32_t low = t & ((1u << c) - 1u);
-  const uint32_t mid = t >> c;
-  const uint32_t f_lo = f & ((1u << (lo - c)) - 1u);   // bits [c, lo)
-  const uint32_t f_hi = f >> (lo - c);                  // bits [hi, n)
-  return low | (f_lo << c) | (mid << lo) | (f_hi << hi);
+// (hi - lo) bits -> bits [lo, hi), the fixed bits f -> [c, lo) then [hi, nb).
+__device__ __forceinline__ uint32_t tile_index(const PassArgs &q, uint32_t t, uint32_t f) {
+  const uint32_t low = t & ((1u << q.c) - 1u);
+  const uint32_t mid = t >> q.c;
+  const uint32_t f_lo = f & ((1u << (q.lo - q.c)) - 1u);   // bits [c, lo)
+  const uint32_t f_hi = f >> (q.lo - q.c);                  // bits [hi, nb)
+  return low | (f_lo << q.c) | (mid << q.lo) | (f_hi << q.hi);
 }
 
-// Rounds j in [lo, hi) (tile bit c + j - lo) on the tile in shared memory.
-__device__ __forceinline__ void tile_rounds(double *v, int T_log, int c, int lo, int hi, double jP, double jM) {
-  const int half = 1 << (T_log - 1);
-  for (int j = lo; j < hi; ++j) {
-    const int tb = c + (j - lo);
-    for (int p = threadIdx.x; p < half; p += blockDim.x) {
-      const int t0 = ((p >> tb) << (tb + 1)) | (p & ((1 << tb) - 1));
-      const int t1 = t0 | (1 << tb);
-      const double x = v[t0], y = v[t1];
-      const double d = __dsub_rn(x, y);
-      v[t0] = __fma_rn(jP, d, y);      // jP x + jM y with jM = 1 - jP
-      v[t1] = __fma_rn(-jP, d, x);     // jP y + jM x
+// Shared-memory place of tile element t: one double of padding per 16, so
+// that threads reading 16 consecutive elements each meet different banks.
+__device__ __forceinline__ uint32_t padded(uint32_t t) { return t + (t >> 4); }
+
+// G rounds on 2^G elements held in registers.
+template <int G>
+__device__ __forceinline__ void rounds(double (&v)[1 << G], double r) {
+#pragma unroll
+  for (int b = 0; b < G; ++b)
+#pragma unroll
+    for (int i = 0; i < (1 << G); ++i)
+      if (!(i & (1 << b))) {
+        const double x = v[i], y = v[i | (1 << b)];
+        v[i] = __fma_rn(r, y, x);
+        v[i | (1 << b)] = __fma_rn(r, x, y);
+      }
+}
+
+// G rounds on tile bits [tb, tb + G) of the whole tile (PAIR: of the tile and
+// its complement, element t of the one with element T - 1 - t of the other).
+// FROM / TO: elements come from src / go to dst instead of shared memory.
+// The tile of an unpaired last pass stays in shared memory (dst null).
+template <int G, bool PAIR, bool FROM, bool TO>
+__device__ __forceinline__ void stage(const double *src, double *dst, double *tile, const double *wt,
+                                      const TransferArgs &a, const PassArgs &q, int T_log, uint32_t f, int tb) {
+  constexpr int M = 1 << G;
+  const uint32_t T = 1u << T_log, top = (1u << q.nb) - 1u;
+  for (uint32_t p = threadIdx.x; p < T >> G; p += blockDim.x) {
+    const uint32_t t0 = ((p >> tb) << (tb + G)) | (p & ((1u << tb) - 1u));
+    double v[M], w[PAIR ? M : 1];
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const uint32_t t = t0 | ((uint32_t)m << tb);
+      if constexpr (FROM) {
+        const uint32_t i = tile_index(q, t, f);
+        v[m] = src[i];
+        if constexpr (PAIR) w[m] = src[top - i];
+      } else {
+        v[m] = tile[padded(t)];
+        if constexpr (PAIR) w[m] = tile[padded(T + (T - 1u - t))];
+      }
     }
-    __syncthreads();
+    if constexpr (FROM)
+      if (q.first) {
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+          const uint32_t i = tile_index(q, t0 | ((uint32_t)m << tb), f);
+          v[m] = __dmul_rn(v[m], wt[energy_index(a, i)]);
+          if constexpr (PAIR) w[m] = __dmul_rn(w[m], wt[energy_index(a, top - i)]);
+        }
+      }
+    rounds<G>(v, a.r);
+    if constexpr (PAIR) rounds<G>(w, a.r);   // the complement's bit pairs are this one's, swapped
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const uint32_t t = t0 | ((uint32_t)m << tb);
+      if constexpr (TO && PAIR) {
+        const uint32_t i = tile_index(q, t, f);
+        dst[i] = __dmul_rn(__fma_rn(a.pr, w[m], v[m]), wt[64 + energy_index(a, i)]);
+        dst[top - i] = __dmul_rn(__fma_rn(a.pr, v[m], w[m]), wt[64 + energy_index(a, top - i)]);
+      } else if constexpr (TO) {
+        dst[tile_index(q, t, f)] = v[m];
+      } else {
+        tile[padded(t)] = v[m];
+        if constexpr (PAIR) tile[padded(T + (T - 1u - t))] = w[m];
+      }
+    }
   }
 }
 
-// One pass over the rounds [lo, hi).  first: multiply by w on load.  last:
-// the parity factor and the multiply by w follow; the block then holds the
-// tile of fixed bits f and its complement (or, with no fixed bits, the
-// whole vector in one tile).
-__global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const double *__restrict__ src, double *dst,
-                                                                       const TransferArgs a, int c, int lo, int hi,
-                                                                       int n_fixed_bits, int first, int last) {
-  extern __shared__ double tile[];
-  const int T_log = c + (hi - lo);
-  const int T = 1 << T_log;
-  const uint32_t nF = 1u << n_fixed_bits;
-  const bool pair = last && n_fixed_bits > 0;
-  const uint32_t f = blockIdx.x;
-  const uint32_t fc = nF - 1u - f;   // complement tile (pair mode: f < fc)
-  double *A = tile, *B = tile + T;
-  for (int t = threadIdx.x; t < T; t += blockDim.x) {
-    const uint32_t i = tile_index((uint32_t)t, f, c, lo, hi);
-    const double x = src[i];
-    A[t] = first ? __dmul_rn(x, boltzmann(a, i)) : x;
-    if (pair) {
-      const uint32_t ib = tile_index((uint32_t)t, fc, c, lo, hi);
-      const double y = src[ib];
-      B[t] = first ? __dmul_rn(y, boltzmann(a, ib)) : y;
-    }
+template <bool PAIR, bool FROM, bool TO>
+__device__ __forceinline__ void stage_g(int g, const double *src, double *dst, double *tile, const double *wt,
+                                        const TransferArgs &a, const PassArgs &q, int T_log, uint32_t f, int tb) {
+  switch (g) {
+    case 1: stage<1, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
+    case 2: stage<2, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
+    case 3: stage<3, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
+    default:
+      if constexpr (!PAIR) stage<4, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb);
+  }
+}
+
+// Block f takes the tile of fixed bits f (PAIR: and its complement, f below
+// half of them).  PAIR: the last pass with fixed bits; a last pass without
+// any holds the whole vector in one tile.  src and dst may be the same: every
+// element is read by the block that writes it, before it does.
+template <bool PAIR>
+__global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const double *src, double *dst,
+                                                                       const __grid_constant__ TransferArgs a,
+                                                                       const PassArgs q) {
+  extern __shared__ double smem[];
+  double *wt = smem, *tile = smem + 128;   // w on load (scaled by jP^{L^2}), w at the end; then the tile(s)
+  const int T_log = q.c + (q.hi - q.lo);
+  const uint32_t T = 1u << T_log, f = blockIdx.x;
+  if (threadIdx.x < 51) {
+    wt[threadIdx.x] = __dmul_rn(a.wtab[threadIdx.x], a.jPn);
+    wt[64 + threadIdx.x] = a.wtab[threadIdx.x];
   }
   __syncthreads();
-  tile_rounds(A, T_log, c, lo, hi, a.jP, a.jM);
-  if (pair) tile_rounds(B, T_log, c, lo, hi, a.jP, a.jM);
-  if (last) {
-    const double pjM = __dmul_rn(a.parity, a.jM);
-    if (pair) {
-      // element t of A pairs with element T-1-t of B (all index bits inverted)
-      for (int t = threadIdx.x; t < T; t += blockDim.x) {
-        const double x = A[t], y = B[T - 1 - t];
-        const uint32_t ia = tile_index((uint32_t)t, f, c, lo, hi);
-        const uint32_t ib = tile_index((uint32_t)(T - 1 - t), fc, c, lo, hi);
-        dst[ia] = __dmul_rn(__dadd_rn(__dmul_rn(a.jP, x), __dmul_rn(pjM, y)), boltzmann(a, ia));
-        dst[ib] = __dmul_rn(__dadd_rn(__dmul_rn(a.jP, y), __dmul_rn(pjM, x)), boltzmann(a, ib));
-      }
-    } else {
-      // one tile holds the whole vector: element t pairs with T-1-t
-      for (int t = threadIdx.x; t < T / 2; t += blockDim.x) {
-        const double x = A[t], y = A[T - 1 - t];
-        const uint32_t ia = tile_index((uint32_t)t, f, c, lo, hi);
-        const uint32_t ib = tile_index((uint32_t)(T - 1 - t), f, c, lo, hi);
-        dst[ia] = __dmul_rn(__dadd_rn(__dmul_rn(a.jP, x), __dmul_rn(pjM, y)), boltzmann(a, ia));
-        dst[ib] = __dmul_rn(__dadd_rn(__dmul_rn(a.jP, y), __dmul_rn(pjM, x)), boltzmann(a, ib));
-      }
+  constexpr int GM = PAIR ? 3 : 4;
+  int tb = q.c, left = q.hi - q.lo;
+  const bool to_mem = PAIR || !q.last;   // the last group writes HBM
+  bool loaded = false;
+  if (!PAIR && tb < 4) {   // consecutive elements per thread: load whole segments first
+    for (uint32_t t = threadIdx.x; t < T; t += blockDim.x) {
+      const uint32_t i = tile_index(q, t, f);
+      const double x = src[i];
+      tile[padded(t)] = q.first ? __dmul_rn(x, wt[energy_index(a, i)]) : x;
     }
-  } else {
-    for (int t = threadIdx.x; t < T; t += blockDim.x) dst[tile_index((uint32_t)t, f, c, lo, hi)] = A[t];
+    loaded = true;
+    __syncthreads();
   }
+  while (left > 0) {
+    const int g = left < GM ? left : GM;
+    const bool end = left == g && to_mem;
+    if (!loaded && end)
+      stage_g<PAIR, true, true>(g, src, dst, tile, wt, a, q, T_log, f, tb);
+    else if (!loaded)
+      stage_g<PAIR, true, false>(g, src, dst, tile, wt, a, q, T_log, f, tb);
+    else if (end)
+      stage_g<PAIR, false, true>(g, src, dst, tile, wt, a, q, T_log, f, tb);
+    else
+      stage_g<PAIR, false, false>(g, src, dst, tile, wt, a, q, T_log, f, tb);
+    loaded = true;
+    tb += g;
+    left -= g;
+    if (!end) __syncthreads();
+  }
+  if (!PAIR && q.last)   // the whole vector in one tile: element t pairs with T-1-t
+    for (uint32_t t = threadIdx.x; t < T / 2; t += blockDim.x) {
+      const double x = tile[padded(t)], y = tile[padded(T - 1u - t)];
+      dst[t] = __dmul_rn(__fma_rn(a.pr, y, x), wt[64 + energy_index(a, t)]);
+      dst[T - 1u - t] = __dmul_rn(__fma_rn(a.pr, x, y), wt[64 + energy_index(a, T - 1u - t)]);
+    }
 }
 
 struct Pass {
@@ -180,9 +261,10 @@ extern "C" int qisg_transfer_matvec(const double *in, double *out, int L, double
   const int L2 = L * L, nb = L2 - 1;
   TransferArgs a{};
   const double ek = std::exp(k_tau), emk = std::exp(-k_tau);
-  a.jP = ek / (ek + emk);
-  a.jM = emk / (ek + emk);
-  a.parity = (double)parity;
+  const double jP = ek / (ek + emk), jM = emk / (ek + emk);
+  a.r = jM / jP;
+  a.pr = (double)parity * a.r;
+  a.jPn = std::pow(jP, (double)L2);
   for (int e = -2 * L2, i = 0; e <= 2 * L2; e += 2, ++i) a.wtab[i] = std::exp(0.5 * k * (double)e);
   a.L2 = L2;
   a.L = L;
@@ -205,10 +287,14 @@ extern "C" int qisg_transfer_matvec(const double *in, double *out, int L, double
     const int width = q.c + (q.hi - q.lo);
     const int fixed = nb - width;
     const bool last = p + 1 == plan.size();
-    const unsigned blocks = (unsigned)((last && fixed > 0) ? (1u << (fixed - 1)) : (1u << fixed));
-    const size_t smem = (size_t)((last && fixed > 0) ? 2 : 1) << width;
-    transfer_pass_kernel<<<blocks, kTransferBlock, smem * sizeof(double), st>>>(
-        p == 0 ? in : out, out, a, q.c, q.lo, q.hi, fixed, p == 0, last);
+    const bool pair = last && fixed > 0;
+    const unsigned blocks = pair ? 1u << (fixed - 1) : 1u << fixed;
+    const size_t T = (size_t)1 << width, smem = (128 + (pair ? 2 * T + 2 * T / 16 : T + T / 16)) * sizeof(double);
+    const PassArgs pa{q.c, q.lo, q.hi, p == 0, last, nb};
+    if (pair)
+      transfer_pass_kernel<true><<<blocks, kTransferBlock / 2, smem, st>>>(p == 0 ? in : out, out, a, pa);
+    else
+      transfer_pass_kernel<false><<<blocks, kTransferBlock, smem, st>>>(p == 0 ? in : out, out, a, pa);
     rc = cuda_check(cudaGetLastError(), "transfer matvec");
   }
   return rc;

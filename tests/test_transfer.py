@@ -3,9 +3,10 @@ oracle's round-by-round product: both sectors, every lattice size one GPU
 holds (2 <= L <= 5, so one, two and three passes over HBM), in place and out
 of place, equal and separate couplings.
 
-The kernel evaluates each round as y + jP (x - y) with fused multiply-adds
-(jP + jM = 1), the oracle as jP x + jM y: the two differ by rounding.  Each
-of the L^2 + 1 steps is a convex combination (jP, jM in (0, 1)), so it adds
+The kernel evaluates each round as x + r y, r = jM / jP, with the factors jP
+taken out (one fused multiply-add), the oracle as jP x + jM y: the two differ
+by rounding.  Each of the L^2 + 1 steps is a convex combination (jP, jM in
+(0, 1)) up to that common factor, so it adds
 at most a few units of 2^-53 of the vector's norm; the test bound,
 1e-13 in the max norm relative to the result's max norm, is about 500 such
 units for the 26 steps at L = 5 (the 1e-12 relative bound stated for FP64
@@ -37,6 +38,23 @@ def test_transfer_matvec_matches_oracle(L, k, kt, parity, inplace):
     torch.cuda.synchronize()
     got = d_out.cpu().numpy()
     assert np.max(np.abs(got - want)) <= 1e-13 * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("L,kt", [(3, 0.0), (4, 0.0), (4, 20.0), (5, 0.4)])
+def test_transfer_matvec_at_an_odd_address(L, kt):
+    """Vectors aligned to 8 bytes only; equal and vanishing flip weights."""
+    torch = need_gpu()
+    from paper_2402_03920_gb300 import qisg
+    J = oracle.init_couplings(L, 0, 1, 7)[0]
+    n = 1 << (L * L - 1)
+    v = np.random.default_rng(L).standard_normal(n)
+    buf = torch.zeros(2 * n + 2, dtype=torch.float64, device="cuda")
+    buf[1:n + 1] = torch.from_numpy(v).cuda()
+    qisg.transfer_matvec(buf.data_ptr() + 8, buf.data_ptr() + 8 * (n + 1), L, 0.3, kt, J, -1)
+    torch.cuda.synchronize()
+    want = oracle.transfer_matvec(L, 0.3, kt, J, -1, v)
+    assert np.max(np.abs(buf[n + 1:2 * n + 1].cpu().numpy() - want)) <= 1e-13 * np.max(np.abs(want))
+    assert buf[0] == 0 and buf[2 * n + 1] == 0
 
 
 def test_transfer_power_iteration_and_refusals():
