@@ -333,8 +333,10 @@ int qisg_block_means(qisg_handle *h, int64_t first, int64_t n, double *e_s, doub
  *   S2 = sum Q~^2, S4 = sum Q~^4   (L_tau Q_2(tau), L_tau Q_4(tau) of one
  *                                   configuration)
  *   SF = sum (|sum_x e^{i 2pi x_1/L} q~_x|^2 + |sum_x e^{i 2pi x_2/L} q~_x|^2)
- *        (2 L_tau F(tau)); FP64 from the column and row sums of q~, x in
- *        order 0 .. L-1, with a cos / sin table from the host's libm.
+ *        (2 L_tau F(tau)); from exact integer correlations of the column
+ *        and row sums of q~ and a cosine table from the host's libm (where
+ *        those terms cancel to less than 1/16 of their size, from the sums
+ *        over x in order 0 .. L-1 in FP64).
  * Averages over measurements and replicas are the caller's.  Host arrays
  * [n_a][n_replicas][n_slots][L_tau] (int64, int64, int64, double).  Spins
  * are unpacked on the device in chunks through a temporary buffer of at

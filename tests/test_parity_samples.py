@@ -415,3 +415,14 @@ def test_pt_in_blue_pass_with_pt_every_and_graph_off(qisg):
         sA, sB, sq, sq2, nm = a.measurements()
         assert nm == st.n_meas
         assert np.array_equal(sA, st.sumA) and np.array_equal(sq2, st.sumq2)
+
+
+@pytest.mark.parametrize("W", [32, 64])
+def test_spins_of_sample_ranges(qisg, W):
+    """Sample ranges that start and end inside a word of samples."""
+    inst, _ = make(qisg, 4, 6, 0.2, 0.5, 3, 1.0, 5, 150, 9, layout=qisg.QISG_LAYOUT_SAMPLES, word_bits=W)
+    with inst:
+        inst.sweep(5)
+        S = inst.spins()
+        for lo, n in ((0, 1), (31, 2), (30, 70), (63, 1), (65, 85), (149, 1)):
+            assert np.array_equal(inst.spins(lo, n), S[lo:lo + n]), (lo, n)

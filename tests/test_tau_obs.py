@@ -45,3 +45,36 @@ def test_tau_observables_match_oracle(qisg, layout, W, L, Lt, n_a, ap):
         sub = inst.tau_observables(lo, n)
         for g, w in zip(sub, got):
             assert np.array_equal(g, w[lo:lo + n])
+
+
+@pytest.mark.parametrize("L,Lt,n_slots,n_rep,pattern", [
+    (2, 2, 1, 1, "chain"),       # one lag, 256 threads share it
+    (2, 600, 1, 2, "chain"),     # more than 256 lags
+    (10, 50, 2, 2, "chain"), (14, 34, 1, 2, "chain"),
+    (18, 26, 1, 2, "chain"), (20, 1452, 1, 1, "chain"),   # the last: the largest L_tau shared memory takes at L = 20
+    (32, 66, 1, 1, "chain"),
+    (12, 20, 1, 2, "layers"), (20, 12, 1, 1, "layers"),   # uniform q~: SF is what its terms' rounding leaves
+    (8, 12, 1, 2, "stripes"),                             # one wave at half the wave number only
+])
+def test_tau_observables_of_given_states(qisg, L, Lt, n_slots, n_rep, pattern):
+    rng = np.random.default_rng(L * 1000 + Lt)
+    shape = (1, n_rep, n_slots, Lt, L, L)
+    if pattern == "chain":
+        S = np.cumprod(np.where(rng.random(shape) < 0.2, -1, 1), axis=3)
+    elif pattern == "layers":
+        S = np.broadcast_to(rng.choice([-1, 1], size=(1, n_rep, n_slots, Lt, 1, 1)), shape)
+    else:
+        S = rng.choice([-1, 1], size=(1, n_rep, n_slots, Lt, 1, 1)) * np.where(np.arange(L) % 2, -1, 1)
+        S = np.where(np.arange(Lt)[:, None, None] % 3 == 0, np.abs(S), np.broadcast_to(S, shape))
+    S = np.ascontiguousarray(S.reshape(1, n_rep, n_slots, Lt * L * L), dtype=np.int8)
+    wa = np.tile(np.arange(n_slots, dtype=np.int32), (1, n_rep, 1))
+    inst, _ = make(qisg, L, Lt, 0.2, 0.5, n_slots, 1.0, n_rep, 1, 3, layout=qisg.QISG_LAYOUT_SAMPLES, word_bits=32)
+    with inst:
+        inst.set_state(S, wa, 0)
+        got = inst.tau_observables()
+    want = oracle.tau_observables(L, Lt, S, wa)
+    for name, g, w in zip(("S1", "S2", "S4"), got[:3], want[:3]):
+        assert np.array_equal(g, w), name
+    # the integer sums leave a few roundings at most 16 times enlarged by
+    # cancellation (below 1e-13); other lags are the oracle's sums themselves
+    assert np.allclose(got[3], want[3], rtol=1e-12, atol=0), "SF"
