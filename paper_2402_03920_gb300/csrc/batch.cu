@@ -56,7 +56,7 @@ struct ChainRef {
 
 // One tile of a half sweep of instance I (sample 0, 64-bit LANES words).
 template <bool BLUE>
-__device__ void batch_tile(const InstDev &I, int colour, int j0, int n, unsigned char *smem) {
+__device__ void batch_tile(const InstDev &I, uint32_t t, int colour, int j0, int n, unsigned char *smem) {
   LanesSample<unsigned long long> S;
   S.spins = I.spins;
   S.T = I.T;
@@ -65,7 +65,7 @@ __device__ void batch_tile(const InstDev &I, int colour, int j0, int n, unsigned
   S.J = I.J;
   S.key = I.key;
   S.ctr_w = DOM_SWEEP << 28;   // sample 0: sample block 0
-  S.t = (uint32_t)__ldcg(&I.t);
+  S.t = t;
   S.hpd = I.hpd;
   S.hld = I.hld;
   S.L = I.L;
@@ -88,54 +88,70 @@ __device__ void batch_tile(const InstDev &I, int colour, int j0, int n, unsigned
     lanes_tile<unsigned long long, true, BLUE>(S, colour, j0, n, 0, colour == 0 && j0 == 0, smem);
 }
 
-__device__ __forceinline__ bool live(const InstDev &I) { return I.active && __ldcg(&I.remaining) != 0; }
+// The instance takes part in sweep sw of the launch (remaining is the
+// number of sweeps left when the launch began).
+__device__ __forceinline__ bool live(const InstDev &I, int sw) {
+  const long long rem = __ldcg(&I.remaining);
+  return I.active && (rem < 0 || rem > sw);
+}
 
 // The persistent kernel: n_sweeps x (red tiles | barrier | blue tiles |
-// barrier | PT chains | barrier | advance | barrier).  Block b takes the
-// contiguous tile range [bstart[b], bstart[b+1]) (ranges of about equal cost).
-// The tiles are bound by memory latency, so the kernel is held to the
-// registers of three blocks per SM: the extra resident warps outweigh the
-// spills of the blue tile's counters (measured: 4.30 -> 3.47 ps/update on the
-// 512-instance uneven batch, where two blocks per SM fit without the bound).
+// barrier | PT chains | barrier), then the sweep counters advance once.
+//
+// What bounds it: integer issue in the tiles, and before that how evenly the
+// phases end, since every block waits for the last one three times a sweep.
+// Tile costs differ several times across the instances and the SMs do not
+// run alike, so blocks take tiles one by one from a counter per colour, the
+// next one fetched while the current one runs (contiguous ranges of equal
+// estimated cost left the blocks a quarter of their time at the barriers).
+//
+// Three blocks per SM, spills of the two-group blue tile's counters accepted:
+// two or four blocks are within 2% of it.
 __global__ void __launch_bounds__(kBatchBlock, 3) batch_kernel(InstDev *insts, int n_inst, const Tile *tiles,
-                                                            int n_tiles, const int *bstart, const ChainRef *chains,
-                                                            int n_chains, int n_sweeps, unsigned *bar, int *err,
-                                                            long long wait_ns) {
+                                                            int n_tiles, const ChainRef *chains, int n_chains,
+                                                            int n_sweeps, unsigned *bar, int *err, long long wait_ns) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int64_t lo = bstart[blockIdx.x];
-  const int64_t hi = bstart[blockIdx.x + 1];
+  __shared__ unsigned s_next[2];
+  unsigned *taken = bar + 2;   // [colour]: tiles taken beyond the first of each block
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   for (int sw = 0; sw < n_sweeps; ++sw) {
     for (int colour = 0; colour < 2; ++colour) {
-      for (int64_t k = lo; k < hi; ++k) {
+      int buf = 0;
+      for (unsigned k = blockIdx.x; k < (unsigned)n_tiles; buf ^= 1) {
+        if (threadIdx.x == 0) s_next[buf] = gridDim.x + atomicAdd(taken + colour, 1u);
         const Tile tl = tiles[k];
         const InstDev &I = insts[tl.inst];
-        if (!live(I)) continue;
-        if (colour == 0)
-          batch_tile<false>(I, 0, tl.j0, tl.n, smem);
-        else
-          batch_tile<true>(I, 1, tl.j0, tl.n, smem);
+        if (live(I, sw)) {
+          const uint32_t t = (uint32_t)__ldcg(&I.t) + (uint32_t)sw;
+          if (colour == 0)
+            batch_tile<false>(I, t, 0, tl.j0, tl.n, smem);
+          else
+            batch_tile<true>(I, t, 1, tl.j0, tl.n, smem);
+        }
+        __syncthreads();   // s_next is written; the other entry is free again
+        k = s_next[buf];
       }
       if (!grid_barrier(bar, err, wait_ns)) return;
     }
+    if (blockIdx.x == 0 && threadIdx.x < 2) taken[threadIdx.x] = 0u;   // no block takes tiles before the next barrier
     for (int c = gwarp; c < n_chains; c += warps) {
       const ChainRef cr = chains[c];
       const InstDev &I = insts[cr.inst];
-      if (!live(I)) continue;
+      if (!live(I, sw)) continue;
       pt_chain<false, true, true>(I.walker + cr.r * I.n_slots, I.U + (size_t)cr.r * I.n_slots * 2, I.ptc, I.sq,
-                                  I.key, (uint32_t)__ldcg(&I.t), 0, cr.r, I.n_slots);
+                                  I.key, (uint32_t)__ldcg(&I.t) + (uint32_t)sw, 0, cr.r, I.n_slots);
     }
     if (!grid_barrier(bar, err, wait_ns)) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_inst; i += gridDim.x * blockDim.x) {
-      InstDev &I = insts[i];
-      const long long rem = __ldcg(&I.remaining);
-      if (I.active && rem != 0) {
-        I.t = __ldcg(&I.t) + 1ull;
-        if (rem > 0) I.remaining = rem - 1;
-      }
+  }
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_inst; i += gridDim.x * blockDim.x) {
+    InstDev &I = insts[i];
+    const long long rem = __ldcg(&I.remaining);
+    if (I.active && rem != 0) {
+      const long long done = rem < 0 || rem > n_sweeps ? n_sweeps : rem;
+      I.t = __ldcg(&I.t) + (unsigned long long)done;
+      if (rem > 0) I.remaining = rem - done;
     }
-    if (!grid_barrier(bar, err, wait_ns)) return;
   }
 }
 
@@ -235,8 +251,6 @@ struct qisg_batch {
   qisg::InstDev *d_inst = nullptr;
   qisg::Tile *d_tiles = nullptr;
   size_t tiles_cap = 0;
-  int *d_bstart = nullptr;   // first tile of each block (grid + 1 entries)
-  size_t bstart_cap = 0;
   int n_tiles = 0;
   qisg::ChainRef *d_chains = nullptr;
   size_t chains_cap = 0;
@@ -244,7 +258,7 @@ struct qisg_batch {
   unsigned *d_bar = nullptr;
   int *d_err = nullptr;
   bool dirty = true;
-  int tile_rows = 4;      // rows of spb sites per tile
+  int tile_rows = 0;      // rows of 256 sites per tile; 0: chosen for the batch (build_tables)
   int schedule = 0;       // 0: instance order; 1: largest instances first
   int grid = 0;
   size_t smem = 0;
@@ -267,12 +281,23 @@ int build_tables(qisg_batch *B) {
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
       return B->slots[a].dev.N * (int64_t)B->slots[a].dev.n_slots > B->slots[b].dev.N * (int64_t)B->slots[b].dev.n_slots;
     });
+  // rows per tile unless pinned: the most of 8, 4, 2, 1 that leave each block
+  // eight tiles a colour to share out (ms per sweep at 1 | 2 | 4 | 8 rows: 6
+  // instances 0.078 | 0.072 | 0.088 | 0.114, 24: 0.196 | 0.198 | 0.233 | 0.213,
+  // 96: 1.01 | 0.92 | 0.89 | 0.95, 512: 6.22 | 5.59 | 5.26 | 5.17)
+  int rows = B->tile_rows;
+  if (rows == 0) {
+    int64_t total = 0;
+    for (int i : order) total += (B->slots[i].dev.N / 2 + kBatchBlock - 1) / kBatchBlock;
+    rows = 8;
+    while (rows > 1 && total < (int64_t)8 * rows * 3 * B->n_sm) rows >>= 1;   // three blocks per SM
+  }
   B->max_plane = 4;
   B->max_slots = B->max_rep = B->max_spb_groups = 1;
   B->smem = 0;
   for (int i : order) {
     const InstDev &I = B->slots[i].dev;
-    const int per = kBatchBlock * B->tile_rows;
+    const int per = kBatchBlock * rows;
     const int half = I.N / 2;
     for (int j0 = 0; j0 < half; j0 += per) tiles.push_back(Tile{i, j0, std::min(per, half - j0)});
     for (int r = 0; r < I.n_rep; ++r) chains.push_back(ChainRef{i, r});
@@ -314,35 +339,6 @@ int build_tables(qisg_batch *B) {
   if (rc) return rc;
   if (per_sm < 1) return fail(QISG_EINVAL, "batch kernel does not fit on an SM");
   B->grid = per_sm * B->n_sm;
-  // contiguous tile ranges of about equal cost per block (a tile costs its
-  // sites times its lanes, plus a fixed share for its set-up), so that blocks
-  // reach the grid barriers together
-  std::vector<int> bstart((size_t)B->grid + 1, (int)tiles.size());
-  {
-    std::vector<double> cum(tiles.size() + 1, 0.0);
-    for (size_t k = 0; k < tiles.size(); ++k) {
-      const InstDev &I = B->slots[tiles[k].inst].dev;
-      cum[k + 1] = cum[k] + (double)tiles[k].n * (double)(I.n_rep * I.n_slots + 32) + 4096.0;
-    }
-    size_t k = 0;
-    for (int b = 0; b <= B->grid; ++b) {
-      const double target = cum.back() * (double)b / (double)B->grid;
-      while (k < tiles.size() && cum[k] < target) ++k;
-      bstart[(size_t)b] = (int)k;
-    }
-    bstart[(size_t)B->grid] = (int)tiles.size();
-  }
-  if (bstart.size() > B->bstart_cap) {
-    if (B->d_bstart) cudaFree(B->d_bstart);
-    B->d_bstart = nullptr;
-    B->bstart_cap = std::max<size_t>(bstart.size(), 2 * B->bstart_cap);
-    rc = cuda_check(cudaMalloc(&B->d_bstart, B->bstart_cap * sizeof(int)), "block table");
-    if (rc) return rc;
-  }
-  rc = cuda_check(cudaMemcpyAsync(B->d_bstart, bstart.data(), bstart.size() * sizeof(int), cudaMemcpyHostToDevice,
-                                  B->stream),
-                  "copy block table");
-  if (rc) return rc;
   B->dirty = false;
   return QISG_OK;
 }
@@ -506,11 +502,11 @@ int qisg_batch_create(qisg_batch **out, int capacity, size_t mem_budget, void *c
   }
   if (!rc) rc = cuda_check(cudaMalloc(&B->arena, B->budget), "arena");
   if (!rc) rc = cuda_check(cudaMalloc(&B->d_inst, sizeof(InstDev) * (size_t)capacity), "descriptors");
-  if (!rc) rc = cuda_check(cudaMalloc(&B->d_bar, 2 * sizeof(unsigned)), "barrier");
+  if (!rc) rc = cuda_check(cudaMalloc(&B->d_bar, 4 * sizeof(unsigned)), "barrier");
   if (!rc) rc = cuda_check(cudaMalloc(&B->d_err, sizeof(int)), "error flag");
   // on the batch's stream (it may be non-blocking, so a default-stream memset
   // would not be ordered before the first launch)
-  if (!rc) rc = cuda_check(cudaMemsetAsync(B->d_bar, 0, 2 * sizeof(unsigned), B->stream), "barrier");
+  if (!rc) rc = cuda_check(cudaMemsetAsync(B->d_bar, 0, 4 * sizeof(unsigned), B->stream), "barrier");
   if (!rc) rc = cuda_check(cudaMemsetAsync(B->d_err, 0, sizeof(int), B->stream), "error flag");
   if (!rc) rc = cuda_check(cudaMemsetAsync(B->d_inst, 0, sizeof(InstDev) * (size_t)capacity, B->stream),
                            "descriptors");
@@ -574,9 +570,9 @@ int qisg_batch_run(qisg_batch *B, int64_t n_sweeps) {
   int64_t left = n_sweeps;
   while (left > 0 && !rc) {
     int ns = (int)std::min<int64_t>(left, chunk);
-    void *args[] = {&B->d_inst, &B->capacity, &B->d_tiles, &B->n_tiles, &B->d_bstart, &B->d_chains, &B->n_chains,
+    void *args[] = {&B->d_inst, &B->capacity, &B->d_tiles, &B->n_tiles, &B->d_chains, &B->n_chains,
                     &ns, &B->d_bar, &B->d_err, &B->wait_ns};
-    rc = cuda_check(cudaMemsetAsync(B->d_bar, 0, 2 * sizeof(unsigned), B->stream), "reset barrier");
+    rc = cuda_check(cudaMemsetAsync(B->d_bar, 0, 4 * sizeof(unsigned), B->stream), "reset barrier");
     if (rc) break;
     rc = cuda_check(cudaLaunchCooperativeKernel((const void *)batch_kernel, dim3((unsigned)B->grid),
                                                 dim3(kBatchBlock), args, B->smem, B->stream),
@@ -721,7 +717,6 @@ void qisg_batch_destroy(qisg_batch *B) {
   if (B->arena) cudaFree(B->arena);
   if (B->d_inst) cudaFree(B->d_inst);
   if (B->d_tiles) cudaFree(B->d_tiles);
-  if (B->d_bstart) cudaFree(B->d_bstart);
   if (B->d_chains) cudaFree(B->d_chains);
   if (B->d_bar) cudaFree(B->d_bar);
   if (B->d_err) cudaFree(B->d_err);
