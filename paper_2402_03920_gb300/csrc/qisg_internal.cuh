@@ -22,7 +22,7 @@ namespace qisg {
 enum : uint32_t { DOM_J = 1, DOM_INIT = 2, DOM_SWEEP = 3, DOM_PT = 4, DOM_DAEMON = 5 };
 
 // Index bits of the SITES daemon tables (the words' top bits -> candidate bins).
-constexpr int kDaemonLutBits = 12;
+constexpr int kDaemonLutBits = 13;
 
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 constexpr uint32_t kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
@@ -30,7 +30,7 @@ constexpr uint32_t kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
 // Philox4x32-10 (Salmon et al., SC'11), the generator of Sec. 2.1.1.  The
 // low and high halves of each product are taken apart: measured faster here
 // than one wide multiply per product (the daemon kernels, whose Philox calls
-// sit between table lookups, use the wide form, philox_wide).
+// sit between table lookups, use the wide form).
 __device__ __forceinline__ uint4 philox(uint4 c, uint2 k) {
 #pragma unroll
   for (int i = 0; i < 10; ++i) {
@@ -666,7 +666,7 @@ struct qisg_handle {
   unsigned long long *d_t = nullptr;  // sweep counter; d_t[1]: its copy for the PT pass (fused mode)
   void *d_acc = nullptr;            // SAMPLES: PT lane masks of the last pass, Word [b][r][s]
   unsigned long long *d_dcum = nullptr;   // SITES: cumulative tables [n_slots][256]
-  uint2 *d_dlut = nullptr;                // SITES: prefix index [n_slots][2^kDaemonLutBits], then the spans (bytes)
+  uint32_t *d_dlut = nullptr;             // SITES: prefix index [n_slots][2^kDaemonLutBits]
   int *d_err = nullptr;
   // records at every measurement (Appendix A): PT walk history and maxit block sums
   int hist_len = 0, maxit = 0, blk_len = 0;

@@ -18,28 +18,32 @@
 // Each daemon word comes from one Philox4x32-10 call (the upper halves of
 // four 64-bit "50/50" words) and one xoroshiro128++ state step of the same
 // 128 bits (the lower halves); byte i of the word is n* of 64-bit word i,
-// the bin of the word in the cumulative table of the walker's slot.  n* is
-// found from an index of the top kDaemonLutBits bits, staged in shared
-// memory: the words with a given prefix fall in the bins [n_min, n_min +
-// span], so n* = n_min + #{q in [n_min, n_min + span): cumulative(q) <= word}.
-// With span <= 1 the entry holds the upper half of the one cut point and
-// n* = n_min + [upper half of the word > it]; with span >= 2 the upper
-// halves of the span cut points are compared one by one.  Only when an
-// upper half equals a cut point's does the lower half matter (a running
-// product of the XORs of the upper halves then becomes 0): the whole daemon
-// word is redone with the full 64-bit words, and the xoroshiro step is only
-// computed there.  The bytes are assembled by multiply-adds with run-time
-// factors, which keeps that work off the logic pipe.
+// the bin of the word in the cumulative table of the walker's slot.
+//
+// What bounds it: integer issue (three Philox calls and twelve look-ups per
+// word), so
+//   * n* is found from an index of the top kDaemonLutBits bits, staged in
+//     shared memory: the words with a given prefix fall in the bins [n_min,
+//     n_min + span], so n* = n_min + #{q in [n_min, n_min + span):
+//     cumulative(q) <= word}.  An entry is one 32-bit word: the cut point's
+//     upper half below the prefix in its top bits (all ones without a cut), a
+//     flag for span >= 2, and n_min.  With span <= 1 the byte is n_min plus
+//     one comparison of the word's bits below the prefix with the entry as
+//     it stands.  Only a flagged entry, or bits equal to the cut point's
+//     (then the lower halves matter), sends the daemon word to the exact
+//     path, which computes the xoroshiro step;
+//   * the first two Philox rounds of a word's three calls share their products
+//     with the site alone, and those with the system are the block's;
+//   * a thread walks up the tau' of one column (x, y), two planes a step, so
+//     the couplings and neighbour offsets are fixed, and the word above is
+//     the next step's word below.
 //
 // Device arrays (systems walker-major; PT exchanges slot labels only):
 //   spins  u32 [a][r][w][L^2 M]       bit = 1 <=> spin -1
 //   J      uint8 [a][x + L*y]          bit0: J(+x) = -1, bit1: J(+y) = -1
 //   U      u64 [a][r][w][2]            unsatisfied spatial / tau bonds of walker w
 //   cum    u64 [n_slots][256]          cumulative(0..254) of Sec. 2.1.1; [255] = 2^64-1
-//   lut    uint2 [n_slots][2^kDaemonLutBits]
-//                                      {n_min, | 2^31 when span >= 2; upper half of
-//                                       cumulative(n_min) when span = 1, else 2^32 - 1}
-//   span   uint8 [n_slots][2^kDaemonLutBits] (after lut)   span of each prefix
+//   lut    u32 [n_slots][2^kDaemonLutBits]   cut bits | span >= 2 << 8 | n_min
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -51,21 +55,21 @@ namespace {
 
 constexpr int kBlock = 256;
 
+constexpr uint32_t kSpanFlag = 0x100u;   // index entry: two or more cut points
+
 struct SitesArgs {
   uint32_t *spins;
   const uint8_t *J;
   const int32_t *walker;
   const unsigned long long *cum;
-  const uint2 *lut;
-  const uint8_t *span;
+  const uint32_t *lut;
   unsigned long long *U;
   const unsigned long long *d_t;
   uint2 key;
-  uint32_t m8, m16, m24;       // 2^8, 2^16, 2^24 at run time (byte assembly by multiply-adds)
-  FastDiv half_plane_div, half_L_div;
-  int L, M, plane, half_plane, n_words, half_words;
+  FastDiv plane_div, L_div, bps_div, ns_div, nr_div;
+  int L, M, plane, n_words;
   int n_slots, n_rep;
-  int blocks_per_sys, words_per_thread;
+  int n_seg, walk;             // segments per column and words of the colour in one (at most)
   int tau_ap;
 };
 
@@ -81,194 +85,160 @@ __device__ __forceinline__ uint4 xoroshiro_step(uint4 x) {
   return make_uint4((uint32_t)n0, (uint32_t)(n0 >> 32), (uint32_t)n1, (uint32_t)(n1 >> 32));
 }
 
-// Philox4x32-10 with 32 x 32 -> 64-bit products (the same function as
-// philox(): each round's high and low halves come from one wide multiply).
-__device__ __forceinline__ uint4 philox_wide(uint4 c, uint2 k) {
+// The exact bytes of a daemon word from its Philox output x: lower halves
+// from the xoroshiro step, then for every byte the count of the cut points at
+// or below the word among its prefix's candidates.  A candidate run ends at
+// the first cut point above the word (the cut points do not decrease).
+static __device__ __noinline__ uint32_t daemon_exact(uint4 x, const uint32_t *lut, const unsigned long long *cum) {
+  const uint4 lo = xoroshiro_step(x);
+  uint32_t b = 0;
 #pragma unroll
-  for (int i = 0; i < 10; ++i) {
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t hi = pick4(x, i);
+    const unsigned long long R = ((unsigned long long)hi << 32) | pick4(lo, i);
+    uint32_t n = lut[hi >> (32 - kDaemonLutBits)] & 0xFFu;
+    while (n < 255u && cum[n] <= R) ++n;
+    b |= n << (8 * i);
+  }
+  return b;
+}
+
+// One daemon word: byte i is n* of the 64-bit word whose upper half is Philox
+// output i.  c: the Philox state after two rounds; k: the third round's key.
+__device__ __forceinline__ uint32_t daemon_word(uint4 c, uint2 k, const uint32_t *lut, const unsigned long long *cum) {
+#pragma unroll
+  for (int i = 2; i < 10; ++i) {   // one wide product per half round: measured faster here than two halves
     const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c.x;
     const unsigned long long p1 = (unsigned long long)kPhiloxM1 * c.z;
     c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k.y, (uint32_t)p0);
     k.x += kPhiloxW0;
     k.y += kPhiloxW1;
   }
-  return c;
-}
-
-// Exact n* of 64-bit word i of a daemon word (the rare path): the lower
-// half from the xoroshiro step of the Philox output x, then the count of
-// the cut points at or below the word among the prefix's candidates.
-static __device__ __noinline__ uint32_t nstar_exact(uint4 x, int i, const uint2 *lut, const uint8_t *span,
-                                                    const unsigned long long *cum) {
-  const uint4 lo = xoroshiro_step(x);
-  const uint32_t hi = pick4(x, i), l = pick4(lo, i);
-  const unsigned long long R = ((unsigned long long)hi << 32) | l;
-  const uint32_t h = hi >> (32 - kDaemonLutBits);
-  uint32_t n = lut[h].x & 0xFFu;
-  const uint32_t end = n + span[h];
-  for (uint32_t q = n; q < end; ++q) n += (R >= cum[q]) ? 1u : 0u;
-  return n;
-}
-
-// n* of a 64-bit word from its upper half hi (entry e: e.x = n_min, bit 31
-// set when the cell holds two or more cut points; e.y = upper half of the
-// one cut point, else all ones).  *prod collects hi ^ (cut's upper half):
-// it becomes 0 when they tie (the lower halves then decide; a zero product
-// without a tie only sends the word to the exact path).
-__device__ __forceinline__ uint32_t nstar_hi(uint32_t hi, const uint2 *lut, const uint32_t *cut_hi,
-                                             const uint8_t *span, uint32_t *prod) {
-  const uint32_t h = hi >> (32 - kDaemonLutBits);
-  const uint2 e = lut[h];
-  uint32_t n = e.x + (hi > e.y ? 1u : 0u);
-  *prod *= hi ^ e.y;
-  if ((int)e.x < 0) {   // two or more cut points: compare their upper halves
-    const uint32_t n0 = e.x & 0xFFu, end = n0 + span[h];
-    n = n0;
-    for (uint32_t q = n0; q < end; ++q) {
-      const uint32_t c = cut_hi[q];
-      n += hi > c ? 1u : 0u;
-      *prod *= hi ^ c;
-    }
-  }
-  return n;
-}
-
-// Daemon word `which` (0: b4, 1: b8, 2: b12) of word-site ws of system
-// (a, r, slot s) in sweep t: byte i is n* of the 64-bit word whose upper
-// half is Philox output i.
-__device__ __forceinline__ uint32_t daemon_word(uint32_t ws, uint32_t t, uint32_t c2, uint32_t c3, uint2 key,
-                                                const uint2 *lut, const uint32_t *cut_hi, const uint8_t *span,
-                                                const unsigned long long *cum, uint32_t m8, uint32_t m16,
-                                                uint32_t m24) {
-  const uint4 x = philox_wide(make_uint4(ws, t, c2, c3), key);
-  uint32_t prod = 1;
-  const uint32_t b = nstar_hi(x.x, lut, cut_hi, span, &prod) + nstar_hi(x.y, lut, cut_hi, span, &prod) * m8 +
-                     nstar_hi(x.z, lut, cut_hi, span, &prod) * m16 + nstar_hi(x.w, lut, cut_hi, span, &prod) * m24;
-  if (prod != 0) return b;
-  return nstar_exact(x, 0, lut, span, cum) | (nstar_exact(x, 1, lut, span, cum) << 8) |
-         (nstar_exact(x, 2, lut, span, cum) << 16) | (nstar_exact(x, 3, lut, span, cum) << 24);
+  const uint32_t e0 = lut[c.x >> (32 - kDaemonLutBits)], e1 = lut[c.y >> (32 - kDaemonLutBits)];
+  const uint32_t e2 = lut[c.z >> (32 - kDaemonLutBits)], e3 = lut[c.w >> (32 - kDaemonLutBits)];
+  const uint32_t x0 = c.x << kDaemonLutBits, x1 = c.y << kDaemonLutBits;
+  const uint32_t x2 = c.z << kDaemonLutBits, x3 = c.w << kDaemonLutBits;
+  // n_min of the four bytes, plus one where the word's bits exceed the cut's
+  // (the entry's low bits do not reach the next cut value: x > e iff the
+  // fields compare so)
+  uint32_t b = __byte_perm(__byte_perm(e0, e1, 0x0040), __byte_perm(e2, e3, 0x0040), 0x5410);
+  b += x0 > e0 ? 1u : 0u;
+  b += x1 > e1 ? 1u << 8 : 0u;
+  b += x2 > e2 ? 1u << 16 : 0u;
+  b += x3 > e3 ? 1u << 24 : 0u;
+  const uint32_t tie = min(min(x0 ^ e0, x1 ^ e1), min(x2 ^ e2, x3 ^ e3));   // < 2^bits: equal fields
+  if ((tie >> kDaemonLutBits) == 0u || ((e0 | e1 | e2 | e3) & kSpanFlag)) b = daemon_exact(c, lut, cum);
+  return b;
 }
 
 __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a | b)); }
 
 // One half sweep (colour 0 = red, 1 = blue).  Block x serves system
-// x / blocks_per_sys (sys = (a n_rep + r) n_slots + w) and the colour words
-// [chunk * 256 * wpt, (chunk + 1) * 256 * wpt) of it, thread i taking words
-// chunk * 256 * wpt + i + 256 j.  The blue pass counts, per system, the
+// x / blocks_per_sys (sys = (a n_rep + r) n_slots + w) and 256 consecutive
+// (segment, column) pairs of it; a thread walks the colour's words of one
+// column in one segment along tau'.  The blue pass counts, per system, the
 // unsatisfied bonds of its words after the update: every bond has exactly
 // one blue end, so this is each bond once.  Chunk 0 of the red pass clears
 // the system's counters.  count_only: no update (energies of the stored
 // state).
 template <bool BLUE>
-__global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(SitesArgs p, int count_only) {
+__global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(const SitesArgs p, int count_only) {
   __shared__ unsigned long long cum_s[256];
-  __shared__ uint32_t cut_hi_s[256];
-  __shared__ __align__(16) uint8_t span_s[1 << kDaemonLutBits];
-  extern __shared__ __align__(16) uint2 lut_s[];   // [2^kDaemonLutBits]
-  __shared__ unsigned long long red_s[2][kBlock / 32];
-  const int64_t sys = blockIdx.x / p.blocks_per_sys;
-  const int chunk = (int)(blockIdx.x - sys * p.blocks_per_sys);
-  const int w = (int)(sys % p.n_slots);
-  const int64_t ar = sys / p.n_slots;   // a * n_rep + r
-  const int r = (int)(ar % p.n_rep);
-  const int64_t a = ar / p.n_rep;
-  const int colour = BLUE ? 1 : 0;
-  if (!BLUE && chunk == 0 && threadIdx.x < 2) p.U[sys * 2 + threadIdx.x] = 0;
+  extern __shared__ __align__(16) uint32_t lut_s[];   // [2^kDaemonLutBits]
+  __shared__ uint32_t red_s[2][kBlock / 32];
+  const uint32_t sys = p.bps_div.div(blockIdx.x), chunk = blockIdx.x - sys * p.bps_div.d;
+  const uint32_t ar = p.ns_div.div(sys), w = sys - ar * (uint32_t)p.n_slots;   // ar = a * n_rep + r
+  const uint32_t a = p.nr_div.div(ar), r = ar - a * (uint32_t)p.n_rep;
+  const uint32_t colour = BLUE ? 1u : 0u;
+  if (!BLUE && chunk == 0 && threadIdx.x < 2) p.U[(size_t)sys * 2 + threadIdx.x] = 0;
   if (!BLUE && count_only) return;
   // slot of walker w: lane l of every warp reads walker_at[a][r][l]
   const int lane = threadIdx.x & 31;
-  const int32_t wl = lane < p.n_slots ? __ldg(p.walker + ar * p.n_slots + lane) : -1;
-  const int s = max(__ffs(__ballot_sync(0xFFFFFFFFu, wl == w)) - 1, 0);   // rows are permutations
+  const int32_t wl = lane < p.n_slots ? __ldg(p.walker + (size_t)ar * p.n_slots + lane) : -1;
+  const int s = max(__ffs(__ballot_sync(0xFFFFFFFFu, wl == (int32_t)w)) - 1, 0);   // rows are permutations
   // stage the slot's tables
-  {
-    const unsigned long long *cg = p.cum + (size_t)s * 256;
-    for (int i = threadIdx.x; i < 256; i += kBlock) {
-      const unsigned long long v = __ldg(cg + i);
-      cum_s[i] = v;
-      cut_hi_s[i] = (uint32_t)(v >> 32);
-    }
+  if (!count_only) {
+    cum_s[threadIdx.x] = __ldg(p.cum + (size_t)s * 256 + threadIdx.x);
     const uint4 *lg = reinterpret_cast<const uint4 *>(p.lut + ((size_t)s << kDaemonLutBits));
     uint4 *ls = reinterpret_cast<uint4 *>(lut_s);
-    for (int i = threadIdx.x; i < (1 << kDaemonLutBits) / 2; i += kBlock) ls[i] = __ldg(lg + i);
-    const uint4 *sg = reinterpret_cast<const uint4 *>(p.span + ((size_t)s << kDaemonLutBits));
-    uint4 *ss = reinterpret_cast<uint4 *>(span_s);
-    for (int i = threadIdx.x; i < (1 << kDaemonLutBits) / 16; i += kBlock) ss[i] = __ldg(sg + i);
-  }
-  __syncthreads();
-  uint32_t *S = p.spins + sys * p.n_words;
-  const uint8_t *J = p.J + a * p.plane;
-  const uint32_t t = (uint32_t)*p.d_t;
-  const uint32_t c2 = (uint32_t)s | ((uint32_t)r << 16);
-  const uint32_t c3 = (DOM_DAEMON << 28) | (uint32_t)a;
-  const uint32_t ap_up = p.tau_ap ? 0x80000000u : 0u, ap_dn = p.tau_ap ? 1u : 0u;
-  unsigned long long us_cnt = 0, ut_cnt = 0;
-  const int base = chunk * kBlock * p.words_per_thread + threadIdx.x;
-  for (int j = 0; j < p.words_per_thread; ++j) {
-    const int idx = base + j * kBlock;
-    if (idx >= p.half_words) break;
-    // idx -> (tau', y, x) of the colour's words
-    const uint32_t tq = p.half_plane_div.div((uint32_t)idx);
-    const uint32_t rem = (uint32_t)idx - tq * (uint32_t)p.half_plane;
-    const uint32_t y = p.half_L_div.div(rem);
-    const uint32_t xh = rem - y * (uint32_t)(p.L >> 1);
-    const uint32_t x = 2 * xh + ((y + tq + (uint32_t)colour) & 1u);
-    const int L = p.L;
-    const int ws = (int)(x + (uint32_t)L * y + (uint32_t)p.plane * tq);
-    const int xp = (x == (uint32_t)(L - 1)) ? ws - (L - 1) : ws + 1;
-    const int xm = (x == 0) ? ws + (L - 1) : ws - 1;
-    const int yp = (y == (uint32_t)(L - 1)) ? ws - (L - 1) * L : ws + L;
-    const int ym = (y == 0) ? ws + (L - 1) * L : ws - L;
-    const bool top = tq == (uint32_t)(p.M - 1), bottom = tq == 0;
-    const int tp = top ? ws - (p.M - 1) * p.plane : ws + p.plane;
-    const int tm = bottom ? ws + (p.M - 1) * p.plane : ws - p.plane;
-    const uint32_t c = S[ws];
-    uint32_t nup = S[tp], ndn = S[tm];
-    if (top) nup = __funnelshift_r(nup, nup, 1) ^ ap_up;   // bit j <- bit j+1 of tau' = 0
-    if (bottom) ndn = __funnelshift_l(ndn, ndn, 1) ^ ap_dn;   // bit j <- bit j-1 of tau' = M-1
-    const int i2 = (int)(x + (uint32_t)L * y);
-    const uint32_t jc = __ldg(J + i2);
-    const uint32_t jxm = __ldg(J + (x == 0 ? i2 + L - 1 : i2 - 1));
-    const uint32_t jym = __ldg(J + (y == 0 ? i2 + (L - 1) * L : i2 - L));
-    // unsatisfied bond masks: J S S' = -1 <=> bit(S) ^ bit(S') ^ bit(J) = 1
-    uint32_t e1 = c ^ S[xp] ^ (0u - (jc & 1u));
-    uint32_t e2 = c ^ S[xm] ^ (0u - (jxm & 1u));
-    uint32_t e3 = c ^ S[yp] ^ (0u - ((jc >> 1) & 1u));
-    uint32_t e4 = c ^ S[ym] ^ (0u - ((jym >> 1) & 1u));
-    uint32_t e5 = c ^ nup;
-    uint32_t e6 = c ^ ndn;
-    uint32_t f = 0;
-    if (!count_only) {
-      // u = u0 + 2 u1 + 4 u2, bit-sliced over the 32 sites
-      const uint32_t s1 = e1 ^ e2 ^ e3, k1 = maj3(e1, e2, e3);
-      const uint32_t s2 = e4 ^ e5 ^ e6, k2 = maj3(e4, e5, e6);
-      const uint32_t u0 = s1 ^ s2, h = s1 & s2;
-      const uint32_t u1 = k1 ^ k2 ^ h, u2 = maj3(k1, k2, h);
-      const uint32_t ge3 = u2 | (u1 & u0);
-      const uint32_t eq2 = ~u2 & u1 & ~u0, eq1 = ~u2 & ~u1 & u0, eq0 = ~(u2 | u1 | u0);
-      // b4, b8, b12 in a rolled loop (one copy of the lookup code)
-      uint32_t b4 = 0, b8 = 0, b12 = 0;
-#pragma unroll 1
-      for (uint32_t which = 0; which < 3; ++which) {
-        const uint32_t dw = daemon_word((uint32_t)ws, t, c2, c3 | (which << 24), p.key, lut_s, cut_hi_s, span_s, cum_s,
-                                        p.m8, p.m16, p.m24);
-        b4 = b8;
-        b8 = b12;
-        b12 = dw;
-      }
-      f = ge3 | (b4 & (eq2 | (b8 & (eq1 | (b12 & eq0)))));
-      S[ws] = c ^ f;
-    }
-    if (BLUE) {
-      us_cnt += __popc(e1 ^ f) + __popc(e2 ^ f) + __popc(e3 ^ f) + __popc(e4 ^ f);
-      ut_cnt += __popc(e5 ^ f) + __popc(e6 ^ f);
-    }
-  }
-  if (BLUE) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      us_cnt += __shfl_xor_sync(0xFFFFFFFFu, us_cnt, o);
-      ut_cnt += __shfl_xor_sync(0xFFFFFFFFu, ut_cnt, o);
+    for (int i = 0; i < (1 << kDaemonLutBits) / 4 / kBlock; ++i) ls[i * kBlock + threadIdx.x] = __ldg(lg + i * kBlock + threadIdx.x);
+    __syncthreads();
+  }
+  const uint32_t P = (uint32_t)p.plane, L = (uint32_t)p.L, M = (uint32_t)p.M;
+  const uint32_t gq = chunk * (uint32_t)kBlock + threadIdx.x;   // (segment, column)
+  const uint32_t seg = p.plane_div.div(gq), i2 = gq - seg * P;
+  uint32_t us_cnt = 0, ut_cnt = 0;
+  if (seg < (uint32_t)p.n_seg) {
+    const uint32_t y = p.L_div.div(i2), x = i2 - y * L;
+    const uint32_t ixp = x + 1 == L ? i2 + 1 - L : i2 + 1, ixm = x == 0 ? i2 + L - 1 : i2 - 1;
+    const uint32_t iyp = y + 1 == L ? x : i2 + L, iym = y == 0 ? i2 + P - L : i2 - L;
+    const uint8_t *J = p.J + (size_t)a * P;
+    const uint32_t jc = __ldg(J + i2);
+    const uint32_t Jxp = 0u - (jc & 1u), Jxm = 0u - (__ldg(J + ixm) & 1u);
+    const uint32_t Jyp = 0u - ((jc >> 1) & 1u), Jym = 0u - ((__ldg(J + iym) >> 1) & 1u);
+    uint32_t *S = p.spins + (size_t)sys * p.n_words;
+    const uint32_t t = (uint32_t)*p.d_t;
+    const uint32_t c3 = (DOM_DAEMON << 28) | a;
+    // Philox rounds 1 and 2, the products of the system's counter word
+    const uint32_t c2 = (uint32_t)s | (r << 16);
+    const uint32_t y1 = kPhiloxM1 * c2 ^ (p.key.x + kPhiloxW0), h1 = __umulhi(kPhiloxM1, c2) ^ t ^ p.key.x;
+    const uint32_t X = __umulhi(kPhiloxM0, h1) ^ (p.key.y + kPhiloxW1), w2 = kPhiloxM0 * h1;
+    const uint32_t ap_up = p.tau_ap ? 0x80000000u : 0u, ap_dn = p.tau_ap ? 1u : 0u;
+    uint32_t tq = ((x + y + colour) & 1u) + 2u * seg * (uint32_t)p.walk;
+    const uint32_t end = min(M, 2u * (seg + 1) * (uint32_t)p.walk);
+    uint32_t dn = 0;
+    if (tq < end) {
+      dn = S[i2 + P * (tq == 0 ? M - 1 : tq - 1)];
+      if (tq == 0) dn = __funnelshift_l(dn, dn, 1) ^ ap_dn;   // bit j <- bit j-1 of tau' = M-1
     }
+    for (; tq < end; tq += 2) {
+      const uint32_t off = P * tq, ws = i2 + off;
+      const bool top = tq + 1 == M;
+      const uint32_t c = S[ws], sxp = S[ixp + off], sxm = S[ixm + off], syp = S[iyp + off], sym = S[iym + off];
+      const uint32_t above = S[top ? i2 : ws + P];
+      uint32_t b4 = 0, b8 = 0, b12 = 0;
+      if (!count_only) {
+        // rounds 1 and 2, the products of the word-site; the three words
+        // differ in the last counter word
+        const uint32_t zs = __umulhi(kPhiloxM0, ws) ^ p.key.y ^ c3, z2 = (kPhiloxM0 * ws) ^ X;
+        const uint2 k3 = make_uint2(p.key.x + 2 * kPhiloxW0, p.key.y + 2 * kPhiloxW1);
+        // b4, b8, b12 in a rolled loop (one copy of the look-up code)
+#pragma unroll 1
+        for (uint32_t which = 0; which < 3; ++which) {
+          const uint32_t z1 = zs ^ (which << 24);
+          const uint32_t dw = daemon_word(make_uint4(__umulhi(kPhiloxM1, z1) ^ y1, kPhiloxM1 * z1, z2, w2), k3, lut_s, cum_s);
+          b4 = b8;
+          b8 = b12;
+          b12 = dw;
+        }
+      }
+      const uint32_t up = top ? __funnelshift_r(above, above, 1) ^ ap_up : above;   // bit j <- bit j+1 of tau' = 0
+      // unsatisfied bond masks: J S S' = -1 <=> bit(S) ^ bit(S') ^ bit(J) = 1
+      const uint32_t e1 = c ^ sxp ^ Jxp, e2 = c ^ sxm ^ Jxm, e3 = c ^ syp ^ Jyp, e4 = c ^ sym ^ Jym;
+      const uint32_t e5 = c ^ up, e6 = c ^ dn;
+      uint32_t f = 0;
+      if (!count_only) {
+        // u = u0 + 2 u1 + 4 u2, bit-sliced over the 32 sites
+        const uint32_t s1 = e1 ^ e2 ^ e3, k1 = maj3(e1, e2, e3);
+        const uint32_t s2 = e4 ^ e5 ^ e6, k2 = maj3(e4, e5, e6);
+        const uint32_t u0 = s1 ^ s2, h = s1 & s2;
+        const uint32_t u1 = k1 ^ k2 ^ h, u2 = maj3(k1, k2, h);
+        const uint32_t ge3 = u2 | (u1 & u0);
+        const uint32_t eq2 = ~u2 & u1 & ~u0, eq1 = ~u2 & ~u1 & u0, eq0 = ~(u2 | u1 | u0);
+        f = ge3 | (b4 & (eq2 | (b8 & (eq1 | (b12 & eq0)))));
+        S[ws] = c ^ f;
+      }
+      if (BLUE) {
+        us_cnt += __popc(e1 ^ f) + __popc(e2 ^ f) + __popc(e3 ^ f) + __popc(e4 ^ f);
+        ut_cnt += __popc(e5 ^ f) + __popc(e6 ^ f);
+      }
+      dn = above;   // the next word of the walk is two planes up
+    }
+  }
+  if (BLUE) {   // at most 2^7 x walk per thread, walk <= 2^14: 32 bits hold the block's sum
+    us_cnt = __reduce_add_sync(0xFFFFFFFFu, us_cnt);
+    ut_cnt = __reduce_add_sync(0xFFFFFFFFu, ut_cnt);
     if (lane == 0) {
       red_s[0][threadIdx.x >> 5] = us_cnt;
       red_s[1][threadIdx.x >> 5] = ut_cnt;
@@ -277,7 +247,7 @@ __global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(SitesArgs p, i
     if (threadIdx.x < 2) {
       unsigned long long v = 0;
       for (int i = 0; i < kBlock / 32; ++i) v += red_s[threadIdx.x][i];
-      if (v) atomicAdd(p.U + sys * 2 + threadIdx.x, v);
+      if (v) atomicAdd(p.U + (size_t)sys * 2 + threadIdx.x, v);
     }
   }
 }
@@ -371,30 +341,30 @@ SitesArgs make_args(qisg_handle *h) {
   p.walker = h->d_walker;
   p.cum = h->d_dcum;
   p.lut = h->d_dlut;
-  p.span = reinterpret_cast<const uint8_t *>(h->d_dlut + ((size_t)h->n_slots << kDaemonLutBits));
   p.U = h->d_U;
   p.d_t = h->d_t;
   p.key = make_uint2((uint32_t)h->seed, (uint32_t)(h->seed >> 32));
-  p.m8 = 1u << 8;
-  p.m16 = 1u << 16;
-  p.m24 = 1u << 24;
   p.L = h->L;
   p.M = h->Lt / 32;
   p.plane = h->L * h->L;
-  p.half_plane = p.plane / 2;
   p.n_words = p.plane * p.M;
-  p.half_words = p.n_words / 2;
-  p.half_plane_div = FastDiv((uint32_t)p.half_plane);
-  p.half_L_div = FastDiv((uint32_t)(h->L / 2));
+  p.plane_div = FastDiv((uint32_t)p.plane);
+  p.L_div = FastDiv((uint32_t)h->L);
   p.n_slots = h->n_slots;
   p.n_rep = h->n_rep;
+  p.ns_div = FastDiv((uint32_t)h->n_slots);
+  p.nr_div = FastDiv((uint32_t)h->n_rep);
   p.tau_ap = h->tau_ap;
-  // words per thread: up to 8, while the grid keeps 8 blocks per SM
+  // words per walk: up to 8 (32 where a tile asks for it), while the grid
+  // keeps 8 blocks per SM
   const int64_t n_sys = h->n_samples * h->n_rep * h->n_slots;
-  int wpt = h->sweep_tile[0] > 0 ? h->sweep_tile[0] : 8;
-  while (wpt > 1 && n_sys * ((p.half_words + kBlock * wpt - 1) / (kBlock * wpt)) < 8LL * h->n_sm) wpt >>= 1;
-  p.words_per_thread = wpt;
-  p.blocks_per_sys = (p.half_words + kBlock * wpt - 1) / (kBlock * wpt);
+  const int half = p.M / 2;
+  int walk = std::min(half, h->sweep_tile[0] > 0 ? h->sweep_tile[0] : 8);
+  auto per_sys = [&](int g) { return ((int64_t)p.plane * ((half + g - 1) / g) + kBlock - 1) / kBlock; };
+  while (walk > 1 && n_sys * per_sys(walk) < 8LL * h->n_sm) walk >>= 1;
+  p.walk = walk;
+  p.n_seg = (half + walk - 1) / walk;
+  p.bps_div = FastDiv((uint32_t)per_sys(walk));
   return p;
 }
 
@@ -460,7 +430,7 @@ void daemon_cumulative(double k, uint64_t *cum) {
 // Prefix index of one cumulative table: entry h covers the words
 // [h 2^(64-bits), (h+1) 2^(64-bits)), whose n* lie in [n_min, n_max];
 // entry = n_min | (n_max - n_min) << 8.
-void daemon_lut(const uint64_t *cum, int bits, uint16_t *lut, uint32_t *cut_hi = nullptr) {
+void daemon_lut(const uint64_t *cum, int bits, uint16_t *lut) {
   auto ns = [&](uint64_t R) {
     uint32_t c = 0;
     while (c < 255 && cum[c] <= R) ++c;   // cum is non-decreasing
@@ -470,39 +440,32 @@ void daemon_lut(const uint64_t *cum, int bits, uint16_t *lut, uint32_t *cut_hi =
     const uint64_t lo = h << (64 - bits), hi = lo + ((~0ull) >> bits);
     const uint32_t a = ns(lo), b = ns(hi);
     lut[h] = (uint16_t)(a | ((b - a) << 8));
-    // upper half of the one cut point inside the cell, else all ones
-    if (cut_hi) cut_hi[h] = (b - a == 1) ? (uint32_t)(cum[a] >> 32) : 0xFFFFFFFFu;
   }
 }
 
 int sites_build_tables(qisg_handle *h) {
   const int n = h->n_slots, nl = 1 << kDaemonLutBits;
   std::vector<unsigned long long> cum((size_t)n * 256);
-  std::vector<uint2> lut((size_t)n * nl);
-  std::vector<uint8_t> span((size_t)n * nl);
+  std::vector<uint32_t> lut((size_t)n * nl);
   std::vector<uint16_t> l16((size_t)nl);
-  std::vector<uint32_t> chi((size_t)nl);
   for (int s = 0; s < n; ++s) {
     uint64_t c[256];
     daemon_cumulative(h->k[s], c);
     c[255] = ~0ull;
     for (int i = 0; i < 256; ++i) cum[(size_t)s * 256 + i] = c[i];
-    daemon_lut(c, kDaemonLutBits, l16.data(), chi.data());
+    daemon_lut(c, kDaemonLutBits, l16.data());
     for (int i = 0; i < nl; ++i) {
       const uint32_t nmin = l16[(size_t)i] & 0xFFu, sp = l16[(size_t)i] >> 8;
-      lut[(size_t)s * nl + i] = make_uint2(nmin | (sp >= 2 ? 0x80000000u : 0u), chi[(size_t)i]);
-      span[(size_t)s * nl + i] = (uint8_t)sp;
+      // the one cut point's upper half below the prefix, else all ones
+      const uint32_t cut = sp == 1 ? (uint32_t)(c[nmin] >> 32) << kDaemonLutBits : 0xFFFFFFFFu << kDaemonLutBits;
+      lut[(size_t)s * nl + i] = cut | (sp >= 2 ? kSpanFlag : 0u) | nmin;
     }
   }
   int rc = cuda_check(cudaMemcpyAsync(h->d_dcum, cum.data(), cum.size() * 8, cudaMemcpyHostToDevice, h->stream),
                       "copy cumulative tables");
   if (!rc)
-    rc = cuda_check(cudaMemcpyAsync(h->d_dlut, lut.data(), lut.size() * 8, cudaMemcpyHostToDevice, h->stream),
+    rc = cuda_check(cudaMemcpyAsync(h->d_dlut, lut.data(), lut.size() * 4, cudaMemcpyHostToDevice, h->stream),
                     "copy prefix index");
-  if (!rc)
-    rc = cuda_check(cudaMemcpyAsync(h->d_dlut + lut.size(), span.data(), span.size(), cudaMemcpyHostToDevice,
-                                    h->stream),
-                    "copy prefix spans");
   // the host vectors must outlive the copies
   if (!rc) rc = cuda_check(cudaStreamSynchronize(h->stream), "sync");
   return rc;
@@ -527,9 +490,9 @@ int sites_init(qisg_handle *h) {
 int sites_half_sweep(qisg_handle *h, int colour, int count_only) {
   const SitesArgs p = make_args(h);
   const int64_t n_sys = h->n_samples * h->n_rep * h->n_slots;
-  const int64_t blocks = n_sys * p.blocks_per_sys;
+  const int64_t blocks = n_sys * p.bps_div.d;
   if (blocks > 0x7FFFFFFF) return fail(QISG_EINVAL, "lattice too large for one launch");
-  constexpr size_t smem = sizeof(uint2) << kDaemonLutBits;
+  constexpr size_t smem = sizeof(uint32_t) << kDaemonLutBits;
   static bool attr_set = false;
   if (!attr_set) {
     cudaFuncSetAttribute(sites_half_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
