@@ -393,9 +393,9 @@ int qisg_profile_read(qisg_handle *h, int kind, double *total_ms, int64_t *n_tim
  * the same either way. */
 int qisg_set_graphs(qisg_handle *h, int enable);
 
-/* SAMPLES packing: launch the kernels of a sweep with programmatic dependent
- * launch (enable = 1, the default): each kernel is launched as the blocks of
- * the one before it leave, and waits for it on the device before it reads
+/* Launch the kernels of a sweep with programmatic dependent launch (enable =
+ * 1, the default): each kernel is launched as the blocks of the one before it
+ * leave, and waits for it on the device before it reads
  * its results, which hides part of the gaps between the red, blue, PT and
  * measurement launches (38.6 against 38.9 us per sweep at L = 16,
  * L_tau = 256, 32 samples x 4 replicas x 16 slots, on a GB300).  Results

@@ -35,6 +35,7 @@ struct LanesArgs {
   FastDiv half_plane_div, half_L_div;
   int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, sites_per_block;
   int tau_ap;
+  unsigned long long *t_copy;   // blue pass: copy t here for the PT pass that advances it (or null)
 };
 
 template <typename Word>
@@ -55,7 +56,9 @@ template <typename Word, bool BLUE, int NREP, int NGC, int TPS>
 __global__ void __launch_bounds__(kBlock) lanes_half_sweep_kernel(LanesArgs<Word> p, int colour,
                                                                   int count_only, int64_t a0, int tile_sites) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pdl_begin();
   const int64_t a = a0 + blockIdx.y;
+  if (BLUE && p.t_copy && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *p.t_copy = *p.d_t;
   LanesSample<Word> S;
   S.spins = p.spins + a * p.n_groups * p.N;
   S.T = p.T;
@@ -266,16 +269,15 @@ LanesArgs<Word> make_args(qisg_handle *h) {
   p.n_groups = h->n_groups;
   p.sites_per_block = kBlock / h->n_slots;
   p.tau_ap = h->tau_ap;
+  p.t_copy = nullptr;
   return p;
 }
 
 template <typename Word, bool BLUE, int NREP, int NGC>
-void launch_half_sweep(const LanesArgs<Word> &p, dim3 grid, size_t smem, cudaStream_t st, int count_only, int64_t a0,
-                       int tile_sites, int tps) {
-  if (tps == 4)
-    lanes_half_sweep_kernel<Word, BLUE, NREP, NGC, 4><<<grid, kBlock, smem, st>>>(p, BLUE, count_only, a0, tile_sites);
-  else
-    lanes_half_sweep_kernel<Word, BLUE, NREP, NGC, 1><<<grid, kBlock, smem, st>>>(p, BLUE, count_only, a0, tile_sites);
+void launch_half_sweep(bool pdl, const LanesArgs<Word> &p, dim3 grid, size_t smem, cudaStream_t st, int count_only,
+                       int64_t a0, int tile_sites, int tps) {
+  launch_kernel(pdl, tps == 4 ? lanes_half_sweep_kernel<Word, BLUE, NREP, NGC, 4> : lanes_half_sweep_kernel<Word, BLUE, NREP, NGC, 1>,
+                grid, dim3(kBlock), smem, st, p, BLUE ? 1 : 0, count_only, a0, tile_sites);
 }
 
 template <typename Word, bool BLUE>
@@ -290,15 +292,21 @@ int set_smem_limits() {
   return QISG_OK;
 }
 
+// One colour of samples a_lo .. a_lo + n_a - 1 on stream st, in_flight samples
+// running at a time.
 template <typename Word>
-int half_sweep_t(qisg_handle *h, int colour, int count_only) {
+int half_sweep_t(qisg_handle *h, int colour, int count_only, int64_t a_lo, int64_t n_a, int64_t in_flight, cudaStream_t st) {
   LanesArgs<Word> p = make_args<Word>(h);
+  if (colour == 1 && !count_only && lanes_pt_advances(h)) p.t_copy = h->d_t + 1;
   if (!lanes_plane_fits(p.plane, h->n_slots, h->n_rep, 227 * 1024))
     return fail(QISG_EINVAL, "LANES plane tables exceed shared memory");
   const size_t smem = lanes_tile_smem(h->n_slots, h->n_rep);
   const int64_t n_launch_samples = h->per_sample_launch ? 1 : h->n_samples;
-  // four threads per site while one would leave the SMs half empty
-  const int tps = p.half_N * n_launch_samples < 1024LL * h->n_sm ? 4 : 1;
+  // four threads per site where the sites in flight are few (one launch's, or
+  // those of the branches beside it).  us per sweep of one sample of 64
+  // systems, four | one thread per site: 4096 sites a colour 12.4 | 16.5,
+  // 16384: 14.4 | 16.5, 32768: 20.6 | 16.5, 147456: 49.1 | 35.4
+  const int tps = p.half_N * in_flight < 160LL * h->n_sm ? 4 : 1;
   // tiles of rows x (256 / tps) sites (rows <= 16, the counters' limit), as
   // long as the grid keeps about four blocks per SM
   const int per = kBlock / tps;
@@ -314,15 +322,15 @@ int half_sweep_t(qisg_handle *h, int colour, int count_only) {
     if (rc) return rc;
     attr_set = true;
   }
-  for (int64_t a0 = 0; a0 < h->n_samples; a0 += (h->per_sample_launch ? 1 : 65535)) {
-    const int64_t na = h->per_sample_launch ? 1 : std::min<int64_t>(65535, h->n_samples - a0);
+  for (int64_t a0 = a_lo; a0 < a_lo + n_a; a0 += (h->per_sample_launch ? 1 : 65535)) {
+    const int64_t na = h->per_sample_launch ? 1 : std::min<int64_t>(65535, a_lo + n_a - a0);
     const int tok = prof_begin(h, sweep_kind(colour));
     const dim3 grid((unsigned)blocks, (unsigned)na);
     // a compile-time word-group count (fewer registers) for four replicas
     auto go = [&](auto nrep, auto ngc) {
       constexpr int R = decltype(nrep)::value, G = decltype(ngc)::value;
-      if (colour == 1) launch_half_sweep<Word, true, R, G>(p, grid, smem, h->stream, count_only, a0, tile_sites, tps);
-      else launch_half_sweep<Word, false, R, G>(p, grid, smem, h->stream, count_only, a0, tile_sites, tps);
+      if (colour == 1) launch_half_sweep<Word, true, R, G>(h->pdl, p, grid, smem, st, count_only, a0, tile_sites, tps);
+      else launch_half_sweep<Word, false, R, G>(h->pdl, p, grid, smem, st, count_only, a0, tile_sites, tps);
     };
     using I0 = std::integral_constant<int, 0>;
     using I1 = std::integral_constant<int, 1>;
@@ -400,9 +408,18 @@ int lanes_init(qisg_handle *h) {
   return cuda_check(cudaGetLastError(), "lanes init");
 }
 
+static int half_sweep_range(qisg_handle *h, int colour, int count_only, int64_t a_lo, int64_t n_a, int64_t in_flight,
+                            cudaStream_t st) {
+  return h->W == 64 ? half_sweep_t<unsigned long long>(h, colour, count_only, a_lo, n_a, in_flight, st)
+                    : half_sweep_t<unsigned int>(h, colour, count_only, a_lo, n_a, in_flight, st);
+}
+
 int lanes_half_sweep(qisg_handle *h, int colour, int count_only) {
-  return h->W == 64 ? half_sweep_t<unsigned long long>(h, colour, count_only)
-                    : half_sweep_t<unsigned int>(h, colour, count_only);
+  return half_sweep_range(h, colour, count_only, 0, h->n_samples, h->per_sample_launch ? 1 : h->n_samples, h->stream);
+}
+
+bool lanes_pt_advances(const qisg_handle *h) {
+  return !h->per_sample_launch && h->pt_every > 0 && (h->t + 1) % (uint64_t)h->pt_every == 0;
 }
 
 int lanes_pt(qisg_handle *h, int explicit_pass) {
@@ -413,7 +430,45 @@ int lanes_pt(qisg_handle *h, int explicit_pass) {
     }
     return QISG_OK;
   }
-  return pt_pass(h, explicit_pass, 0, h->n_samples);
+  return pt_pass(h, explicit_pass, 0, h->n_samples, !explicit_pass && lanes_pt_advances(h) ? h->d_t : nullptr);
+}
+
+// One sweep of the per-instance form inside a stream capture: the launches of
+// different samples are independent (red, blue and PT of a sample follow one
+// another), so they are captured on kLanesBranches branches that fork from
+// h->stream and join it again.  One launch of the production lattice fills a
+// tenth of the GPU's threads and lasts a few microseconds; in a chain each
+// one waited for the one before it.  Production shape, 10 sweeps: 6.3 ms in a
+// chain, 2.57 | 2.28 | 2.27 on 4 | 8 | 16 branches.
+int lanes_forked_sweep(qisg_handle *h, int with_pt) {
+  int rc = QISG_OK;
+  if (!h->fork_ev) {
+    rc = cuda_check(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming), "event");
+    for (int b = 0; b < kLanesBranches && !rc; ++b) {
+      rc = cuda_check(cudaStreamCreateWithFlags(&h->branch[b], cudaStreamNonBlocking), "branch stream");
+      if (!rc) rc = cuda_check(cudaEventCreateWithFlags(&h->join_ev[b], cudaEventDisableTiming), "event");
+    }
+    if (rc) return rc;
+  }
+  const int64_t in_flight = std::min<int64_t>(kLanesBranches, h->n_samples);
+  cudaStream_t main = h->stream;
+  const bool pdl = h->pdl;
+  h->pdl = false;   // a launch after a join waits for several
+  rc = cuda_check(cudaEventRecord(h->fork_ev, main), "fork");
+  for (int b = 0; b < kLanesBranches && b < h->n_samples && !rc; ++b) {
+    rc = cuda_check(cudaStreamWaitEvent(h->branch[b], h->fork_ev, 0), "fork");
+    h->stream = h->branch[b];
+    for (int64_t a = b; a < h->n_samples && !rc; a += kLanesBranches) {
+      rc = half_sweep_range(h, 0, 0, a, 1, in_flight, h->branch[b]);
+      if (!rc) rc = half_sweep_range(h, 1, 0, a, 1, in_flight, h->branch[b]);
+      if (!rc && with_pt) rc = pt_pass(h, 0, a, 1);
+    }
+    h->stream = main;
+    if (!rc) rc = cuda_check(cudaEventRecord(h->join_ev[b], h->branch[b]), "join");
+    if (!rc) rc = cuda_check(cudaStreamWaitEvent(main, h->join_ev[b], 0), "join");
+  }
+  h->pdl = pdl;
+  return rc;
 }
 
 int lanes_measure(qisg_handle *h, int force_to_q) {

@@ -22,12 +22,16 @@ namespace {
 template <bool WIDE>
 __global__ void pt_lanes_kernel(int32_t *walker, unsigned long long *U, const PTConst *ptc, const double *sq,
                                 const unsigned long long *d_t, uint2 key, int64_t a0, int64_t n_chains,
-                                int n_rep, int n_slots, int explicit_pass) {
+                                int n_rep, int n_slots, int explicit_pass, unsigned long long *adv) {
+  pdl_begin();
+  // advance: the pass reads t from adv[1] (the blue pass's copy); no block
+  // reads adv[0], so block 0 sets it to t + 1 for the next sweep
+  if (adv && blockIdx.x == 0 && threadIdx.x == 0) adv[0] = adv[1] + 1ull;
   const int64_t chain = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (chain >= n_chains) return;   // whole warp
   const int64_t a = a0 + chain / n_rep;
   const int r = (int)(chain % n_rep);
-  const uint32_t t = (uint32_t)(explicit_pass ? *d_t - 1ull : *d_t);
+  const uint32_t t = (uint32_t)(adv ? adv[1] : explicit_pass ? *d_t - 1ull : *d_t);
   pt_chain<false, false, WIDE>(walker + (a * n_rep + r) * n_slots, U + (a * n_rep + r) * n_slots * 2, ptc, sq, key,
                                t, a, r, n_slots);
 }
@@ -104,12 +108,9 @@ int pt_pass(qisg_handle *h, int explicit_pass, int64_t a0, int64_t n_a, unsigned
     constexpr int kWarps = 4;
     const unsigned blocks = (unsigned)((n_chains + kWarps - 1) / kWarps);
     const PTConst *ptc = reinterpret_cast<const PTConst *>(h->d_ptc);
-    if (wide)
-      pt_lanes_kernel<true><<<blocks, 32 * kWarps, 0, h->stream>>>(h->d_walker, h->d_U, ptc, h->d_sq, h->d_t, key, a0,
-                                                                   n_chains, h->n_rep, h->n_slots, explicit_pass);
-    else
-      pt_lanes_kernel<false><<<blocks, 32 * kWarps, 0, h->stream>>>(h->d_walker, h->d_U, ptc, h->d_sq, h->d_t, key,
-                                                                    a0, n_chains, h->n_rep, h->n_slots, explicit_pass);
+    launch_kernel(h->pdl, wide ? pt_lanes_kernel<true> : pt_lanes_kernel<false>, dim3(blocks), dim3(32 * kWarps), 0,
+                  h->stream, h->d_walker, h->d_U, ptc, h->d_sq, h->d_t, key, a0, n_chains, h->n_rep, h->n_slots,
+                  explicit_pass, adv);
   }
   prof_end(h, QISG_KERNEL_PT, tok);
   h->launches++;

@@ -423,15 +423,21 @@ int one_sweep(qisg_handle *h, cudaEvent_t *ev = nullptr) {
   const bool lanes = h->layout != QISG_LAYOUT_SAMPLES;   // walker-major: LANES and SITES
   const bool sites = h->layout == QISG_LAYOUT_SITES;
   const uint64_t t = h->t;
+  const bool pt_due = h->pt_every > 0 && (t + 1) % (uint64_t)h->pt_every == 0;
+  // the captured per-instance form runs its samples side by side (timed
+  // launches need the graph to be a chain)
+  const bool forked = lanes && !sites && h->per_sample_launch && h->stream == h->cap_stream && !h->prof;
   int rc = ev ? cuda_check(cudaEventRecord(ev[0], h->stream), "record") : QISG_OK;
-  if (!rc) rc = sites ? sites_half_sweep(h, 0, 0) : lanes ? lanes_half_sweep(h, 0, 0) : samples_half_sweep(h, 0, 0);
+  if (forked) rc = lanes_forked_sweep(h, pt_due);
+  else if (!rc) rc = sites ? sites_half_sweep(h, 0, 0) : lanes ? lanes_half_sweep(h, 0, 0) : samples_half_sweep(h, 0, 0);
   if (!rc && ev) rc = cuda_check(cudaEventRecord(ev[1], h->stream), "record");
-  if (!rc) rc = sites ? sites_half_sweep(h, 1, 0) : lanes ? lanes_half_sweep(h, 1, 0) : samples_half_sweep(h, 1, 0);
+  if (!rc && !forked) rc = sites ? sites_half_sweep(h, 1, 0) : lanes ? lanes_half_sweep(h, 1, 0) : samples_half_sweep(h, 1, 0);
   if (!rc && ev) rc = cuda_check(cudaEventRecord(ev[2], h->stream), "record");
   bool advanced = false;
-  if (!rc && h->pt_every > 0 && (t + 1) % (uint64_t)h->pt_every == 0) {
+  if (!rc && pt_due) {
     if (lanes) {
-      rc = lanes_pt(h, 0);
+      if (!forked) rc = lanes_pt(h, 0);
+      advanced = lanes_pt_advances(h);   // the PT kernel advanced the counter
     } else {
       rc = samples_pt(h, 0, 1);   // the permute kernel advances the counter
       advanced = true;
@@ -548,9 +554,10 @@ int build_cycle(qisg_handle *h, int C) {
     std::vector<cudaGraphNode_t> nodes(n_nodes);
     if (!rc && n_nodes) rc = cuda_check(cudaGraphGetNodes(g, nodes.data(), &n_nodes), "graph nodes");
     // walk the linear chain from its root so that record nodes keep their order
-    // (edges may carry programmatic-launch data, so every query takes edge data)
+    // (edges may carry programmatic-launch data, so every query takes edge
+    // data); only profiled captures have record nodes
     std::vector<cudaGraphNode_t> order;
-    if (!rc) {
+    if (!rc && h->prof) {
       cudaGraphNode_t cur = nullptr;
       for (cudaGraphNode_t nd : nodes) {
         size_t nd_deps = 0;
@@ -1149,6 +1156,11 @@ void qisg_destroy(qisg_handle *h) {
     if (p) cudaFree(p);
   drop_cycle(h);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
+  for (int b = 0; b < kLanesBranches; ++b) {
+    if (h->branch[b]) cudaStreamDestroy(h->branch[b]);
+    if (h->join_ev[b]) cudaEventDestroy(h->join_ev[b]);
+  }
+  if (h->fork_ev) cudaEventDestroy(h->fork_ev);
   prof_clear(h);
   delete h;
 }

@@ -583,6 +583,8 @@ __device__ __forceinline__ SiteXYT site_of_colour(int64_t j, int L, int colour) 
 // ----------------------------------------------------------------------------
 // The handle.
 // ----------------------------------------------------------------------------
+constexpr int kLanesBranches = 8;   // branches of the captured per-instance sweep
+
 struct qisg_handle {
   // problem
   int L = 0, Lt = 0;
@@ -599,7 +601,7 @@ struct qisg_handle {
   // persistent form (SAMPLES, 32-bit words, PT every sweep): one cooperative
   // launch per run of sweeps between measurements
   bool persistent = false;
-  // SAMPLES sweep-path kernels launched with programmatic dependent launch
+  // sweep-path kernels launched with programmatic dependent launch
   bool pdl = true;
   unsigned *d_bar = nullptr;        // grid barrier of the persistent kernel
   long long wait_ns = 5000000000ll; // bound of each barrier wait
@@ -685,6 +687,8 @@ struct qisg_handle {
   // captured on cap_stream and replayed on stream
   bool use_graphs = true;
   cudaStream_t cap_stream = nullptr;
+  cudaStream_t branch[kLanesBranches] = {};   // per-instance LANES: branches of the captured sweep
+  cudaEvent_t fork_ev = nullptr, join_ev[kLanesBranches] = {};
   cudaGraph_t cyc_graph = nullptr;
   cudaGraphExec_t cyc_exec = nullptr;
   int cyc_sweeps = 0;
@@ -711,6 +715,8 @@ int cuda_check(cudaError_t e, const char *what);
 int lanes_init(qisg_handle *h);
 int lanes_half_sweep(qisg_handle *h, int colour, int count_only);
 int lanes_pt(qisg_handle *h, int explicit_pass);
+bool lanes_pt_advances(const qisg_handle *h);   // LANES, SITES: the PT pass of this sweep advances the counter
+int lanes_forked_sweep(qisg_handle *h, int with_pt);
 int lanes_measure(qisg_handle *h, int force_to_q);
 int lanes_energies_by_slot(qisg_handle *h);
 int lanes_get_spins(qisg_handle *h, int64_t a_lo, int64_t n_a, int8_t *S);

@@ -65,6 +65,7 @@ struct SitesArgs {
   const uint32_t *lut;
   unsigned long long *U;
   const unsigned long long *d_t;
+  unsigned long long *t_copy;  // blue pass: copy t here for the PT pass that advances it (or null)
   uint2 key;
   FastDiv plane_div, L_div, bps_div, ns_div, nr_div;
   int L, M, plane, n_words;
@@ -146,6 +147,8 @@ __global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(const SitesArg
   __shared__ unsigned long long cum_s[256];
   extern __shared__ __align__(16) uint32_t lut_s[];   // [2^kDaemonLutBits]
   __shared__ uint32_t red_s[2][kBlock / 32];
+  pdl_begin();
+  if (BLUE && p.t_copy && blockIdx.x == 0 && threadIdx.x == 0) *p.t_copy = *p.d_t;
   const uint32_t sys = p.bps_div.div(blockIdx.x), chunk = blockIdx.x - sys * p.bps_div.d;
   const uint32_t ar = p.ns_div.div(sys), w = sys - ar * (uint32_t)p.n_slots;   // ar = a * n_rep + r
   const uint32_t a = p.nr_div.div(ar), r = ar - a * (uint32_t)p.n_rep;
@@ -343,6 +346,7 @@ SitesArgs make_args(qisg_handle *h) {
   p.lut = h->d_dlut;
   p.U = h->d_U;
   p.d_t = h->d_t;
+  p.t_copy = nullptr;
   p.key = make_uint2((uint32_t)h->seed, (uint32_t)(h->seed >> 32));
   p.L = h->L;
   p.M = h->Lt / 32;
@@ -488,7 +492,8 @@ int sites_init(qisg_handle *h) {
 }
 
 int sites_half_sweep(qisg_handle *h, int colour, int count_only) {
-  const SitesArgs p = make_args(h);
+  SitesArgs p = make_args(h);
+  if (colour == 1 && !count_only && lanes_pt_advances(h)) p.t_copy = h->d_t + 1;
   const int64_t n_sys = h->n_samples * h->n_rep * h->n_slots;
   const int64_t blocks = n_sys * p.bps_div.d;
   if (blocks > 0x7FFFFFFF) return fail(QISG_EINVAL, "lattice too large for one launch");
@@ -500,10 +505,8 @@ int sites_half_sweep(qisg_handle *h, int colour, int count_only) {
     attr_set = true;
   }
   const int tok = prof_begin(h, sweep_kind(colour));
-  if (colour == 1)
-    sites_half_sweep_kernel<true><<<(unsigned)blocks, kBlock, smem, h->stream>>>(p, count_only);
-  else
-    sites_half_sweep_kernel<false><<<(unsigned)blocks, kBlock, smem, h->stream>>>(p, count_only);
+  launch_kernel(h->pdl, colour == 1 ? sites_half_sweep_kernel<true> : sites_half_sweep_kernel<false>,
+                dim3((unsigned)blocks), dim3(kBlock), smem, h->stream, p, count_only);
   prof_end(h, sweep_kind(colour), tok);
   h->launches++;
   return cuda_check(cudaGetLastError(), "sites half sweep");
