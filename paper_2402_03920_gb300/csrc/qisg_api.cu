@@ -359,7 +359,7 @@ int qisg_create(qisg_handle **out, int L, int L_tau, const qisg_slot *ladder, in
   // the persistent kernel's grid barrier (two words) and the blue pass's PT ticket
   if (!rc && layout == QISG_LAYOUT_SAMPLES) rc = dalloc(h, &h->d_bar, 3 * sizeof(unsigned));
   if (!rc && layout == QISG_LAYOUT_SITES) rc = dalloc(h, &h->d_dcum, (size_t)n_slots * 256 * 8);
-  if (!rc && layout == QISG_LAYOUT_SITES) rc = dalloc(h, &h->d_dlut, ((size_t)n_slots << kDaemonLutBits) * 4);
+  if (!rc && layout == QISG_LAYOUT_SITES) rc = dalloc(h, &h->d_dlut, (size_t)n_slots * kDaemonLutWords * 4);
   if (rc) {
     qisg_destroy(h);
     return rc;

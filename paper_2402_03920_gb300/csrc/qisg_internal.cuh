@@ -21,8 +21,11 @@ namespace qisg {
 // Philox counter domains: one per kind of draw.
 enum : uint32_t { DOM_J = 1, DOM_INIT = 2, DOM_SWEEP = 3, DOM_PT = 4, DOM_DAEMON = 5 };
 
-// Index bits of the SITES daemon tables (the words' top bits -> candidate bins).
-constexpr int kDaemonLutBits = 13;
+// Index bits of the SITES daemon tables (the words' top bits -> candidate bins),
+// and of the second index of the cells with several cut points (at most 127 of
+// them: each holds two of the 255).
+constexpr int kDaemonLutBits = 13, kDaemonSubBits = 4;
+constexpr int kDaemonLutWords = (1 << kDaemonLutBits) + (128 << kDaemonSubBits);   // per slot
 
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 constexpr uint32_t kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
@@ -668,7 +671,7 @@ struct qisg_handle {
   unsigned long long *d_t = nullptr;  // sweep counter; d_t[1]: its copy for the PT pass (fused mode)
   void *d_acc = nullptr;            // SAMPLES: PT lane masks of the last pass, Word [b][r][s]
   unsigned long long *d_dcum = nullptr;   // SITES: cumulative tables [n_slots][256]
-  uint32_t *d_dlut = nullptr;             // SITES: prefix index [n_slots][2^kDaemonLutBits]
+  uint32_t *d_dlut = nullptr;             // SITES: prefix index [n_slots][kDaemonLutWords]
   int *d_err = nullptr;
   // records at every measurement (Appendix A): PT walk history and maxit block sums
   int hist_len = 0, maxit = 0, blk_len = 0;

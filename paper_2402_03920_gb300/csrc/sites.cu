@@ -29,21 +29,27 @@
 //     upper half below the prefix in its top bits (all ones without a cut), a
 //     flag for span >= 2, and n_min.  With span <= 1 the byte is n_min plus
 //     one comparison of the word's bits below the prefix with the entry as
-//     it stands.  Only a flagged entry, or bits equal to the cut point's
-//     (then the lower halves matter), sends the daemon word to the exact
-//     path, which computes the xoroshiro step;
+//     it stands.  A flagged entry holds the number of the cell's row in a
+//     second index by the next kDaemonSubBits bits, of entries of the same
+//     form.  Only an entry flagged there too, or bits equal to the cut
+//     point's (then the lower halves matter), sends the daemon word to the
+//     exact path, which computes the xoroshiro step;
 //   * the first two Philox rounds of a word's three calls share their products
 //     with the site alone, and those with the system are the block's;
 //   * a thread walks up the tau' of one column (x, y), two planes a step, so
 //     the couplings and neighbour offsets are fixed, and the word above is
 //     the next step's word below.
+// 423 instructions per word of 32 updates (555 with 8-byte entries, a branch
+// per look-up, whole Philox calls and index arithmetic per word): 10 sweeps at
+// L = 16, L_tau = 8192, 16 samples 14.25 -> 11.5 ms.
 //
 // Device arrays (systems walker-major; PT exchanges slot labels only):
 //   spins  u32 [a][r][w][L^2 M]       bit = 1 <=> spin -1
 //   J      uint8 [a][x + L*y]          bit0: J(+x) = -1, bit1: J(+y) = -1
 //   U      u64 [a][r][w][2]            unsatisfied spatial / tau bonds of walker w
 //   cum    u64 [n_slots][256]          cumulative(0..254) of Sec. 2.1.1; [255] = 2^64-1
-//   lut    u32 [n_slots][2^kDaemonLutBits]   cut bits | span >= 2 << 8 | n_min
+//   lut    u32 [n_slots][kDaemonLutWords]   cut bits | span >= 2 << 8 | n_min by prefix, then the
+//                                      second index's rows of 2^kDaemonSubBits
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -56,6 +62,7 @@ namespace {
 constexpr int kBlock = 256;
 
 constexpr uint32_t kSpanFlag = 0x100u;   // index entry: two or more cut points
+static_assert((kDaemonLutWords / 4) % kBlock == 0, "the block stages whole 16-byte words");
 
 struct SitesArgs {
   uint32_t *spins;
@@ -115,10 +122,19 @@ __device__ __forceinline__ uint32_t daemon_word(uint4 c, uint2 k, const uint32_t
     k.x += kPhiloxW0;
     k.y += kPhiloxW1;
   }
-  const uint32_t e0 = lut[c.x >> (32 - kDaemonLutBits)], e1 = lut[c.y >> (32 - kDaemonLutBits)];
-  const uint32_t e2 = lut[c.z >> (32 - kDaemonLutBits)], e3 = lut[c.w >> (32 - kDaemonLutBits)];
+  uint32_t e0 = lut[c.x >> (32 - kDaemonLutBits)], e1 = lut[c.y >> (32 - kDaemonLutBits)];
+  uint32_t e2 = lut[c.z >> (32 - kDaemonLutBits)], e3 = lut[c.w >> (32 - kDaemonLutBits)];
   const uint32_t x0 = c.x << kDaemonLutBits, x1 = c.y << kDaemonLutBits;
   const uint32_t x2 = c.z << kDaemonLutBits, x3 = c.w << kDaemonLutBits;
+  if ((e0 | e1 | e2 | e3) & kSpanFlag) {   // cells with two or more cut points: by the next bits
+    auto finer = [&](uint32_t e, uint32_t x) {
+      return e & kSpanFlag ? lut[(1 << kDaemonLutBits) + ((e >> kDaemonLutBits) << kDaemonSubBits) + (x >> (32 - kDaemonSubBits))] : e;
+    };
+    e0 = finer(e0, x0);
+    e1 = finer(e1, x1);
+    e2 = finer(e2, x2);
+    e3 = finer(e3, x3);
+  }
   // n_min of the four bytes, plus one where the word's bits exceed the cut's
   // (the entry's low bits do not reach the next cut value: x > e iff the
   // fields compare so)
@@ -145,7 +161,7 @@ __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) { r
 template <bool BLUE>
 __global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(const SitesArgs p, int count_only) {
   __shared__ unsigned long long cum_s[256];
-  extern __shared__ __align__(16) uint32_t lut_s[];   // [2^kDaemonLutBits]
+  extern __shared__ __align__(16) uint32_t lut_s[];   // [kDaemonLutWords]
   __shared__ uint32_t red_s[2][kBlock / 32];
   pdl_begin();
   if (BLUE && p.t_copy && blockIdx.x == 0 && threadIdx.x == 0) *p.t_copy = *p.d_t;
@@ -162,10 +178,10 @@ __global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(const SitesArg
   // stage the slot's tables
   if (!count_only) {
     cum_s[threadIdx.x] = __ldg(p.cum + (size_t)s * 256 + threadIdx.x);
-    const uint4 *lg = reinterpret_cast<const uint4 *>(p.lut + ((size_t)s << kDaemonLutBits));
+    const uint4 *lg = reinterpret_cast<const uint4 *>(p.lut + (size_t)s * kDaemonLutWords);
     uint4 *ls = reinterpret_cast<uint4 *>(lut_s);
 #pragma unroll
-    for (int i = 0; i < (1 << kDaemonLutBits) / 4 / kBlock; ++i) ls[i * kBlock + threadIdx.x] = __ldg(lg + i * kBlock + threadIdx.x);
+    for (int i = 0; i < kDaemonLutWords / 4 / kBlock; ++i) ls[i * kBlock + threadIdx.x] = __ldg(lg + i * kBlock + threadIdx.x);
     __syncthreads();
   }
   const uint32_t P = (uint32_t)p.plane, L = (uint32_t)p.L, M = (uint32_t)p.M;
@@ -359,11 +375,13 @@ SitesArgs make_args(qisg_handle *h) {
   p.ns_div = FastDiv((uint32_t)h->n_slots);
   p.nr_div = FastDiv((uint32_t)h->n_rep);
   p.tau_ap = h->tau_ap;
-  // words per walk: up to 8 (32 where a tile asks for it), while the grid
-  // keeps 8 blocks per SM
+  // words per walk: up to 16 (a block stages 40 KB of tables for its 256
+  // walks; ms per sweep at 8 | 16 | 32 words: L = 16, L_tau = 8192 1.119 | 1.100
+  // | 1.096, L = 24, L_tau = 2048 0.641 | 0.643 | 0.701) while the grid keeps 8
+  // blocks per SM
   const int64_t n_sys = h->n_samples * h->n_rep * h->n_slots;
   const int half = p.M / 2;
-  int walk = std::min(half, h->sweep_tile[0] > 0 ? h->sweep_tile[0] : 8);
+  int walk = std::min(half, h->sweep_tile[0] > 0 ? h->sweep_tile[0] : 16);
   auto per_sys = [&](int g) { return ((int64_t)p.plane * ((half + g - 1) / g) + kBlock - 1) / kBlock; };
   while (walk > 1 && n_sys * per_sys(walk) < 8LL * h->n_sm) walk >>= 1;
   p.walk = walk;
@@ -448,21 +466,34 @@ void daemon_lut(const uint64_t *cum, int bits, uint16_t *lut) {
 }
 
 int sites_build_tables(qisg_handle *h) {
-  const int n = h->n_slots, nl = 1 << kDaemonLutBits;
+  const int n = h->n_slots;
   std::vector<unsigned long long> cum((size_t)n * 256);
-  std::vector<uint32_t> lut((size_t)n * nl);
-  std::vector<uint16_t> l16((size_t)nl);
+  std::vector<uint32_t> lut((size_t)n * kDaemonLutWords, 0u);
   for (int s = 0; s < n; ++s) {
     uint64_t c[256];
     daemon_cumulative(h->k[s], c);
     c[255] = ~0ull;
     for (int i = 0; i < 256; ++i) cum[(size_t)s * 256 + i] = c[i];
-    daemon_lut(c, kDaemonLutBits, l16.data());
-    for (int i = 0; i < nl; ++i) {
-      const uint32_t nmin = l16[(size_t)i] & 0xFFu, sp = l16[(size_t)i] >> 8;
+    auto nstar = [&](uint64_t R) { return (uint32_t)(std::upper_bound(c, c + 255, R) - c); };
+    // entry of the words with the top `bits` bits h: *span gets the number of
+    // cut points inside the cell
+    auto entry = [&](uint64_t h, int bits, uint32_t *span) {
+      const uint64_t lo = h << (64 - bits);
+      const uint32_t nmin = nstar(lo);
+      *span = nstar(lo + ((~0ull) >> bits)) - nmin;
       // the one cut point's upper half below the prefix, else all ones
-      const uint32_t cut = sp == 1 ? (uint32_t)(c[nmin] >> 32) << kDaemonLutBits : 0xFFFFFFFFu << kDaemonLutBits;
-      lut[(size_t)s * nl + i] = cut | (sp >= 2 ? kSpanFlag : 0u) | nmin;
+      const uint32_t cut = *span == 1 ? (uint32_t)(c[nmin] >> 32) << kDaemonLutBits : 0xFFFFFFFFu << kDaemonLutBits;
+      return cut | (*span >= 2 ? kSpanFlag : 0u) | nmin;
+    };
+    uint32_t *out = &lut[(size_t)s * kDaemonLutWords];
+    uint32_t row = 0, span;   // cells with two or more of the 255 cut points: at most 127
+    for (uint64_t i = 0; i < (1ull << kDaemonLutBits); ++i) {
+      out[i] = entry(i, kDaemonLutBits, &span);
+      if (span < 2) continue;
+      out[i] = (row << kDaemonLutBits) | kSpanFlag | (out[i] & 0xFFu);
+      uint32_t *sub = out + (1 << kDaemonLutBits) + (row++ << kDaemonSubBits);
+      for (uint64_t j = 0; j < (1ull << kDaemonSubBits); ++j)
+        sub[j] = entry((i << kDaemonSubBits) | j, kDaemonLutBits + kDaemonSubBits, &span);
     }
   }
   int rc = cuda_check(cudaMemcpyAsync(h->d_dcum, cum.data(), cum.size() * 8, cudaMemcpyHostToDevice, h->stream),
@@ -497,7 +528,7 @@ int sites_half_sweep(qisg_handle *h, int colour, int count_only) {
   const int64_t n_sys = h->n_samples * h->n_rep * h->n_slots;
   const int64_t blocks = n_sys * p.bps_div.d;
   if (blocks > 0x7FFFFFFF) return fail(QISG_EINVAL, "lattice too large for one launch");
-  constexpr size_t smem = sizeof(uint32_t) << kDaemonLutBits;
+  constexpr size_t smem = sizeof(uint32_t) * kDaemonLutWords;
   static bool attr_set = false;
   if (!attr_set) {
     cudaFuncSetAttribute(sites_half_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
