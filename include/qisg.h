@@ -436,8 +436,8 @@ int qisg_set_persistent(qisg_handle *h, int enable, int64_t wait_ns);
  * sweeps per candidate on the handle's own state; the red and blue passes are
  * timed and tuned separately.  Candidates: tiles 1, 2, 4, ..., 64 and the
  * default (0) and, for 32-bit words, the three blue kernel variants of each.
- * The tile is, for 64-bit words, the site groups of 4 each thread walks along
- * tau; for 32-bit words it selects the red pass's threads per site (1: four,
+ * The tile is, for 64-bit words, the site groups of 4 the blue pass's threads
+ * walk along tau (at most 16); for 32-bit words it selects the red pass's threads per site (1: four,
  * 2: two, 0: four while one thread per site would fill fewer than four waves
  * of 2048 threads per SM, else one) and the blue pass's sites per thread
  * (variants 0 and 2, a thread per replica quad walking at most `tile` sites,

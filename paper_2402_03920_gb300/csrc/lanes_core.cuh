@@ -88,24 +88,6 @@ __device__ __forceinline__ Word ld_word(const Word *p) {
   return CG ? __ldcg(p) : *p;
 }
 
-// 32 x 32 bit transposition over the warp: bit i of lane l's result is bit l
-// of lane i's v.
-__device__ __forceinline__ uint32_t warp_transpose32(uint32_t v, int lane) {
-  uint32_t o = __shfl_xor_sync(0xffffffffu, v, 16);
-  v = __byte_perm(v, o, (lane & 16) ? 0x3276 : 0x5410);
-  o = __shfl_xor_sync(0xffffffffu, v, 8);
-  v = __byte_perm(v, o, (lane & 8) ? 0x3715 : 0x6240);
-#pragma unroll
-  for (int k = 4; k > 0; k >>= 1) {
-    const uint32_t m = k == 4 ? 0x0F0F0F0Fu : k == 2 ? 0x33333333u : 0x55555555u;
-    o = __shfl_xor_sync(0xffffffffu, v, k);
-    const bool hi = (lane & k) != 0;
-    o = __funnelshift_l(o, o, hi ? 32 - k : k);
-    v = mux(hi ? ~m : m, v, o);
-  }
-  return v;
-}
-
 // Class code planes of 32 lanes: code = u_s at u_t = 0, else 8 + (u_s & 1) +
 // 2 [u_t = 2] + 4 [u_s >= 2] (those with bit 2 set always flip).  The codes
 // times 4 go to eight words, a byte per lane: lane l is byte l >> 3 of word

@@ -411,6 +411,24 @@ __device__ __forceinline__ Word maj3(Word a, Word b, Word c) {
   return (a & b) | (c & (a ^ b));
 }
 
+// 32 x 32 bit transposition over the warp: bit i of lane l's result is bit l
+// of lane i's v.
+__device__ __forceinline__ uint32_t warp_transpose32(uint32_t v, int lane) {
+  uint32_t o = __shfl_xor_sync(0xffffffffu, v, 16);
+  v = __byte_perm(v, o, (lane & 16) ? 0x3276 : 0x5410);
+  o = __shfl_xor_sync(0xffffffffu, v, 8);
+  v = __byte_perm(v, o, (lane & 8) ? 0x3715 : 0x6240);
+#pragma unroll
+  for (int k = 4; k > 0; k >>= 1) {
+    const uint32_t m = k == 4 ? 0x0F0F0F0Fu : k == 2 ? 0x33333333u : 0x55555555u;
+    o = __shfl_xor_sync(0xffffffffu, v, k);
+    const bool hi = (lane & k) != 0;
+    o = __funnelshift_l(o, o, hi ? 32 - k : k);
+    v = mux(hi ? ~m : m, v, o);
+  }
+  return v;
+}
+
 // Bit-sliced per-lane counter: plane p holds bit p of every lane's count.
 template <typename Word, int K>
 struct VCount {
@@ -627,7 +645,7 @@ struct qisg_handle {
   // per SM.
   int sweep_tile[2] = {0, 0};
   int sweep_variant[2] = {0, 0};
-  int blue_occ[2][7] = {};   // resident blocks per SM of the W = 32 blue kernel (variant 0 | 2, 3 .. 9 counter planes)
+  int blue_occ[3][7] = {};   // resident blocks per SM of the blue kernel (W = 32 variant 0 | 2, W = 64; 3 .. 9 counter planes)
   int sweep_min_blocks_per_sm = 4;
 
   // host tables (FP64, built once)

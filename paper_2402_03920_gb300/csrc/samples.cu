@@ -51,10 +51,7 @@ struct SamplesArgs {
   int tau_ap;                   // antiperiodic along tau: the wrap tau bond flips sign
   // division by the invariants of the index decomposition (32-bit indices)
   FastDiv fd_bps, fd_nq, fd_ns, fd_plane, fd_L, fd_sb;
-  // cleared by the red pass (nothing reads them until the blue pass / PT):
-  unsigned long long *zero_U;   // bond counters, n_zero_U words
-  int64_t n_zero_U;
-  Word *zero_acc;               // PT lane masks, n_zero_acc words
+  Word *zero_acc;               // PT lane masks cleared by this pass, n_zero_acc words
   int64_t n_zero_acc;
 };
 
@@ -80,16 +77,14 @@ __device__ __forceinline__ uint32_t accept_flag(uint32_t R, unsigned long long C
 }
 
 // Accept mask of one 32-bit word: a mux tree over the class planes (u_s in
-// us2 us1 us0, u_t in ut1 ut0) of the per-class accept masks.
+// us2 us1 us0, u_t in ut1 ut0) of the per-class accept masks.  nz = ut0 | ut1.
 __device__ __forceinline__ uint32_t accept_mask(uint32_t R, const unsigned long long *C, uint32_t us0, uint32_t us1,
-                                                uint32_t us2, uint32_t ut0, uint32_t ut1, uint32_t one) {
+                                                uint32_t us2, uint32_t nz, uint32_t ut1, uint32_t one) {
 #define QISG_A(c) accept_flag(R, C[c], one)
   const uint32_t row0 = mux(us2, QISG_A(4), mux(us1, mux(us0, QISG_A(3), QISG_A(2)), mux(us0, QISG_A(1), QISG_A(0))));
-  const uint32_t high = us1 | us2;
-  const uint32_t row1 = high | mux(us0, QISG_A(6), QISG_A(5));
-  const uint32_t row2 = high | mux(us0, QISG_A(8), QISG_A(7));
+  const uint32_t low = mux(us0, mux(ut1, QISG_A(8), QISG_A(6)), mux(ut1, QISG_A(7), QISG_A(5)));   // u_t > 0, u_s < 2
 #undef QISG_A
-  return mux(ut1, row2, mux(ut0, row1, row0));
+  return mux(nz, us1 | us2 | low, row0);
 }
 
 // Per-replica-class sum of the block's counters: thread (quad, j) holds
@@ -137,23 +132,21 @@ __device__ __forceinline__ void quad_sum_counters(const VCount<Word, K> &c, Word
 // bits wide (accept_flag), doubled for 64-bit words.
 template <typename Word>
 __device__ __forceinline__ Word accept_word(uint32_t R, const unsigned long long *C, Word us0, Word us1, Word us2,
-                                            Word ut0, Word ut1, uint32_t one) {
+                                            Word nz, Word ut1, uint32_t one) {
   if constexpr (sizeof(Word) == 4) {
-    return accept_mask(R, C, us0, us1, us2, ut0, ut1, one);
+    return accept_mask(R, C, us0, us1, us2, nz, ut1, one);
   } else {
     auto f = [&](int c) -> Word {
       const uint32_t m = accept_flag(R, C[c], one);
       return ((Word)m << 32) | (Word)m;
     };
     const Word row0 = mux(us2, f(4), mux(us1, mux(us0, f(3), f(2)), mux(us0, f(1), f(0))));
-    const Word high = us1 | us2;
-    const Word row1 = high | mux(us0, f(6), f(5));
-    const Word row2 = high | mux(us0, f(8), f(7));
-    return mux(ut1, row2, mux(ut0, row1, row0));
+    const Word low = mux(us0, mux(ut1, f(8), f(6)), mux(ut1, f(7), f(5)));
+    return mux(nz, us1 | us2 | low, row0);
   }
 }
 
-// One half sweep, column walk.  Block: one (b, s, q) word set; quad thread j
+// Blue half sweep, column walk (32-bit words, variant 1).  Block: one (b, s, q) word set; quad thread j
 // owns replica r = 4q + j.  Quad k owns one (x, y) column and a segment of
 // G sites of the colour along tau (tau = tau0, tau0 + 2, ...; tau0 = 2 G seg
 // + ((colour + x + y) & 1)), so the column's couplings and neighbour offsets
@@ -163,17 +156,18 @@ __device__ __forceinline__ Word accept_word(uint32_t R, const unsigned long long
 // exchanged in shared memory.  The thresholds of the slot come from the
 // parameter bank.  G2 = ceil(log2(G / 4)) sizes the per-thread energy
 // counters, summed per replica by a tree in shared memory.
-template <typename Word, bool BLUE, int G2>
-__global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<Word> p,
+template <int G2>
+__global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<uint32_t> p,
                                                                     const __grid_constant__ SlotThresholds th,
-                                                                    int colour, int count_only) {
+                                                                    int count_only) {
   pdl_begin();
-  constexpr int W = (int)sizeof(Word) * 8;
+  using Word = uint32_t;
+  constexpr int W = 32, colour = 1;
   constexpr int KS = G2 + 5;   // u_s sum <= 4 * 4 * 2^G2 per thread
   constexpr int KT = G2 + 4;   // u_t sum <= 2 * 4 * 2^G2 per thread
   __shared__ uint4 rnd[kBlock];   // one Philox call per thread and group of 4 steps
-  __shared__ Word buf[BLUE ? 4 * (KS + 6) * kQuads : 1];
-  __shared__ int accU[BLUE ? 2 * 4 * W : 1];
+  __shared__ Word buf[4 * (KS + 6) * kQuads];
+  __shared__ int accU[2 * 4 * W];
 
   const uint32_t bid = blockIdx.x;
   const uint32_t set = p.fd_bps.div(bid);
@@ -185,9 +179,8 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
   const int j = threadIdx.x & 3;
   const int quad = threadIdx.x >> 2;
   const int r = 4 * q + j;
-  {   // counters / masks the host asked this pass to clear
+  {   // masks the host asked this pass to clear
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_U; i += stride) p.zero_U[i] = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_acc; i += stride)
       p.zero_acc[i] = 0;
   }
@@ -221,10 +214,8 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
 
   VCount<Word, KS> cs;
   VCount<Word, KT> ct;
-  if (BLUE) {
-    cs.zero();
-    ct.zero();
-  }
+  cs.zero();
+  ct.zero();
 
   // word at tau0 - 1 (the first step's tau - 1); later steps reuse tau + 1
   Word prev_up = 0;
@@ -291,33 +282,30 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
         const Word ut0 = t1 ^ t2;
         const Word ut1 = t1 & t2;
         // accept mask: mux tree over (u_t, u_s) of the per-class masks
-        const Word flip = count_only ? Word(0) : accept_word<Word>(R, C, us0, us1, us2, ut0, ut1, p.one);
+        const Word nz = t1 | t2;
+        const Word flip = count_only ? Word(0) : accept_mask(R, C, us0, us1, us2, nz, ut1, p.one);
         if (!count_only) base[(size_t)site * 4] = sc ^ flip;
-        if (BLUE) {
-          // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
-          const Word vs1 = us1 ^ (flip & us0);
-          const Word vs2 = mux(flip, ~(us0 | us1 | us2), us2);
-          const Word vt1 = mux(flip, ~(ut0 | ut1), ut1);
-          cs.add3(us0, vs1, vs2);
-          ct.add2(ut0, vt1);
-        }
+        // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
+        const Word vs1 = us1 ^ (flip & us0);
+        const Word vs2 = mux(flip, ~(us0 | us1 | us2), us2);
+        const Word vt1 = mux(flip, ~nz, ut1);
+        cs.add3(us0, vs1, vs2);
+        ct.add2(ut0, vt1);
       }
     }
     __syncwarp();
   }
 
-  if (BLUE) {
-    quad_sum_counters<Word, KS>(cs, buf, accU);
-    quad_sum_counters<Word, KT>(ct, buf, accU + 4 * W);
-    for (int i = threadIdx.x; i < 4 * W; i += blockDim.x) {
-      const int jj = i / W, lane = i - jj * W;
-      const int rr = 4 * q + jj;
-      if (rr >= p.n_rep) continue;
-      const int64_t a = b * W + lane;
-      unsigned long long *u = p.U + ((a * p.n_rep + rr) * p.n_slots + s) * 2;
-      if (accU[i]) atomicAdd(u, (unsigned long long)accU[i]);
-      if (accU[4 * W + i]) atomicAdd(u + 1, (unsigned long long)accU[4 * W + i]);
-    }
+  quad_sum_counters<Word, KS>(cs, buf, accU);
+  quad_sum_counters<Word, KT>(ct, buf, accU + 4 * W);
+  for (int i = threadIdx.x; i < 4 * W; i += blockDim.x) {
+    const int jj = i / W, lane = i - jj * W;
+    const int rr = 4 * q + jj;
+    if (rr >= p.n_rep) continue;
+    const int64_t a = b * W + lane;
+    unsigned long long *u = p.U + ((a * p.n_rep + rr) * p.n_slots + s) * 2;
+    if (accU[i]) atomicAdd(u, (unsigned long long)accU[i]);
+    if (accU[4 * W + i]) atomicAdd(u + 1, (unsigned long long)accU[4 * W + i]);
   }
 }
 
@@ -333,7 +321,6 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
 // counters per replica; the block then sums them with a tree in shared
 // memory (vertical adds, 32 lanes per operation) instead of warp shuffles.
 constexpr int kBlock4 = 128;
-constexpr int kLog2Block4 = 7;
 
 struct Quad4 {
   uint4 c, up, xp, xm, yp, ym;
@@ -509,9 +496,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
     const uint32_t c2 = s1 & b4;
     const uint32_t us1 = c1 ^ c2;
     const uint32_t us2 = c1 & c2;
-    const uint32_t ut0 = t1 ^ t2;
-    const uint32_t ut1 = t1 & t2;
-    const uint32_t acc = accept_mask(R, C, us0, us1, us2, ut0, ut1, p.one);
+    const uint32_t acc = accept_mask(R, C, us0, us1, us2, t1 | t2, t1 & t2, p.one);
     *addr_mad(pd, zo[0], four) = sc ^ acc;
     *addr_mad(pd, zo[1], four) = fw[1];
     ps2 += SS;
@@ -616,9 +601,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
         const uint32_t c2 = s1 & b4;
         const uint32_t us1 = c1 ^ c2;
         const uint32_t us2 = c1 & c2;
-        const uint32_t ut0 = t1 ^ t2;
-        const uint32_t ut1 = t1 & t2;
-        const uint32_t acc = accept_mask(R, C, us0, us1, us2, ut0, ut1, p.one);
+        const uint32_t acc = accept_mask(R, C, us0, us1, us2, t1 | t2, t1 & t2, p.one);
         uint32_t *pd = db + (int64_t)sl * SS;
         pd[zo[0]] = sc ^ acc;
         pd[zo[1]] = fw[1];
@@ -810,9 +793,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
       const Word c2 = s1 & b4;
       const Word us1 = c1 ^ c2;
       const Word us2 = c1 & c2;
-      const Word ut0 = t1 ^ t2;
-      const Word ut1 = t1 & t2;
-      out[jj] = sc ^ accept_word<Word>(Rj[jj], C, us0, us1, us2, ut0, ut1, p.one);
+      out[jj] = sc ^ accept_word<Word>(Rj[jj], C, us0, us1, us2, t1 | t2, t1 & t2, p.one);
     }
     Word *pd = db + (int64_t)sl * SS;
     st_rp<Word, RP>(addr_scaled(pd, zo[0], wbytes), out);
@@ -838,57 +819,90 @@ __global__ void __launch_bounds__(kBlock4) samples_red_fusedq_kernel(const Fused
   red_fusedq_body<Word, RP, false>(p, th, blockIdx.x, *p.d_t);
 }
 
-// Sum the block's per-thread counters (NC counters of K planes in registers)
-// and add lane l of counter c into out[c * 32 + l]: tree over the 128
-// threads in shared memory, one more plane per level.
-template <int K, int NC, typename Word = uint32_t>
-__device__ __forceinline__ void block_sum_counters(const VCount<Word, K> *cnt, Word *buf, int *out) {
-  constexpr int KF = K + kLog2Block4;
-  constexpr int W = (int)sizeof(Word) * 8;
-  const int tid = threadIdx.x;
+// ---- per-lane sums of the block's bit-sliced counters ----
+//
+// The block's 128 threads hold NC counters of K planes each.  They go to
+// shared memory as rows [counter][plane][thread]; sixteen threads per counter
+// then add eight entries each (plane by plane, 32 lanes per operation), and
+// the planes of those partial sums are transposed across the warp, which
+// turns the sum over the warp's 2 x 16 rows into one population count per
+// plane and counter.  About 100 logic operations and 9 K shuffles per thread
+// for 8 counters; a tree of vertical adds over all 128 threads took a barrier
+// and some 30 instructions per plane and level (800 per thread at K = 6).
+
+// o = a + b, plane by plane.
+template <int K>
+__device__ __forceinline__ void planes_add(const uint32_t (&a)[K], const uint32_t (&b)[K], uint32_t (&o)[K + 1]) {
+  uint32_t carry = 0;
 #pragma unroll
-  for (int c = 0; c < NC; ++c)
-#pragma unroll
-    for (int i = 0; i < K; ++i) buf[(c * KF + i) * kBlock4 + tid] = cnt[c].p[i];
-  __syncthreads();
-#pragma unroll
-  for (int lvl = 0; lvl < kLog2Block4; ++lvl) {
-    const int half = kBlock4 >> (lvl + 1);
-    for (int w = tid; w < NC * half; w += kBlock4) {
-      const int c = w / half, e = w - c * half;
-      Word *a = buf + (size_t)c * KF * kBlock4 + e;
-      Word carry = 0;
-#pragma unroll
-      for (int i = 0; i < K + lvl; ++i) {
-        const Word x = a[i * kBlock4], y = a[i * kBlock4 + half];
-        a[i * kBlock4] = x ^ y ^ carry;
-        carry = maj3(x, y, carry);
-      }
-      a[(K + lvl) * kBlock4] = carry;
-    }
-    __syncthreads();
+  for (int i = 0; i < K; ++i) {
+    o[i] = a[i] ^ b[i] ^ carry;
+    carry = maj3(a[i], b[i], carry);
   }
-  for (int w = tid; w < NC * W; w += kBlock4) {
-    const int c = w / W, l = w - c * W;
-    int v = 0;
-#pragma unroll
-    for (int i = 0; i < KF; ++i) v |= (int)((buf[(c * KF + i) * kBlock4] >> l) & 1u) << i;
-    out[w] = v;
-  }
-  __syncthreads();   // buf is reused by the caller
+  o[K] = carry;
 }
 
-// Body of the pass for (virtual) block bid of sweep t; CG: read the spins
-// through L2 only (a persistent launch, where other blocks wrote them).
+// The eight entries of row r = [K][kBlock4] that this thread adds (entries of
+// its part, 16 apart; odd counters start one later so that the half-warps
+// meet different banks).
+template <int K>
+__device__ __forceinline__ void planes_sum8(const uint32_t *r, int odd, uint32_t (&acc)[K + 3]) {
+  r += threadIdx.x & 15;
+  uint32_t t[2][K + 2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t s[2][K + 1];
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      uint32_t x[K], y[K];
+      const int m = 4 * h + 2 * g;
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        x[i] = r[i * kBlock4 + 16 * ((m + odd) & 7)];
+        y[i] = r[i * kBlock4 + 16 * ((m + 1 + odd) & 7)];
+      }
+      planes_add<K>(x, y, s[g]);
+    }
+    planes_add<K + 1>(s[0], s[1], t[h]);
+  }
+  planes_add<K + 2>(t[0], t[1], acc);
+}
+
+// Totals of lane threadIdx.x & 31 of the two counters 2 pr and 2 pr + 1 whose
+// rows start at buf, over the threads of each residue modulo S (v[k S + i]:
+// counter 2 pr + k, residue i); every thread of the warp must call it.
+template <int K, int S = 1>
+__device__ __forceinline__ void planes_lane_sums(const uint32_t *buf, int pr, int (&v)[2 * S]) {
+  static_assert(S == 1 || S == 2, "one or two threads per site");
+  const int lane = threadIdx.x & 31, odd = lane >> 4;
+  uint32_t acc[K + 3];
+  planes_sum8<K>(buf + (size_t)(2 * pr + odd) * K * kBlock4, odd, acc);
+#pragma unroll
+  for (int k = 0; k < 2 * S; ++k) v[k] = 0;
+#pragma unroll
+  for (int i = 0; i < K + 3; ++i) {
+    const uint32_t w = warp_transpose32(acc[i], lane);   // bits 0 .. 15: counter 2 pr, thread parts in order
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int r = 0; r < S; ++r) v[k * S + r] += __popc(w & ((S == 1 ? 0xFFFFu : 0x5555u << r) << (16 * k))) << i;
+  }
+}
+
+// Body of the blue pass for (virtual) block bid of sweep t; CG: read the
+// spins through L2 only (a persistent launch, where other blocks wrote them).
+// A thread holds 16 bytes of a site: the four replicas' words (W = 32) or two
+// replicas' words (W = 64: TPQ = 2 threads per site, thread h with replicas
+// 2 h and 2 h + 1), four 32-bit words w in any case; word w has the draw of
+// replica w (W = 32) or 2 h + w / 2.
 // KS: counter planes of a thread's u_s sum (at most 4 G, so KS =
 // counter_planes(G)); the u_t sum (at most 2 G) takes one plane less.
-template <bool BLUE, int KS, bool PF, bool CG>
-__device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, const SlotThresholds &th, uint32_t bid,
-                                            unsigned long long t, int colour, int count_only) {
-  constexpr int KT = KS - 1;
-  constexpr int KF = KS + kLog2Block4;
-  __shared__ uint32_t buf[BLUE ? 4 * KF * kBlock4 : 1];
-  __shared__ int tot[BLUE ? 2 * 4 * 32 : 1];
+template <typename Word, int KS, bool PF, bool CG>
+__device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const SlotThresholds &th, uint32_t bid,
+                                            unsigned long long t, int count_only) {
+  constexpr int KT = KS - 1, TPQ = (int)sizeof(Word) / 4;
+  constexpr uint32_t kCols = kBlock4 / TPQ;   // columns per block
+  __shared__ uint32_t buf[4 * (KS + KT) * kBlock4];   // u_s counters, then u_t
 
   // block -> (b, s, q, chunk) and thread -> (segment, column) in 32 bits
   const uint32_t set = p.fd_bps.div(bid);
@@ -900,6 +914,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, cons
   const unsigned long long *C = th.v[s];
   const int L = p.L, plane = p.plane;
   const uint32_t Lt = (uint32_t)p.Lt, P = (uint32_t)plane;
+  const uint32_t h = TPQ == 1 ? 0u : threadIdx.x & 1u, col = threadIdx.x / TPQ;
   // segment segu and column i2 of the thread; segb is the block's segment
   // when a block holds one segment (else 0, with seg_rem = 0), so the walk
   // length G is the same for the whole block
@@ -908,10 +923,10 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, cons
   if (p.seg_blocks) {
     segb = p.fd_sb.div(chunk);
     segu = segb;
-    i2u = (chunk - segb * (uint32_t)p.seg_blocks) * (uint32_t)kBlock4 + threadIdx.x;
+    i2u = (chunk - segb * (uint32_t)p.seg_blocks) * kCols + col;
     live = i2u < P;
   } else {
-    const uint32_t gq = chunk * (uint32_t)kBlock4 + threadIdx.x;
+    const uint32_t gq = chunk * kCols + col;
     live = gq < P * (uint32_t)p.n_seg;
     segu = p.fd_plane.div(gq);
     segb = 0;
@@ -921,41 +936,66 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, cons
   const int y = (int)p.fd_L.div((uint32_t)i2), x = i2 - y * L;
   const int ixp = (x + 1 == L ? 0 : x + 1) + L * y, ixm = (x == 0 ? L - 1 : x - 1) + L * y;
   const int iyp = x + L * (y + 1 == L ? 0 : y + 1), iym = x + L * (y == 0 ? L - 1 : y - 1);
-  const uint4 *src = reinterpret_cast<const uint4 *>(p.spins) + ((b * p.n_slots + s) * p.n_q + q) * p.N;
-  const uint4 *pc = src + i2, *pxp = src + ixp, *pxm = src + ixm, *pyp = src + iyp, *pym = src + iym;
-  uint4 *wc = reinterpret_cast<uint4 *>(p.spins) + ((b * p.n_slots + s) * p.n_q + q) * p.N + i2;
-  const uint32_t *Jb = p.J + b * (int64_t)plane * 2;
-  uint32_t Jxp = 0, Jxm = 0, Jyp = 0, Jym = 0;
+  uint4 *src = reinterpret_cast<uint4 *>(p.spins) + ((b * p.n_slots + s) * p.n_q + q) * p.N * TPQ + h;
+  const uint4 *pc = src + i2 * TPQ, *pxp = src + ixp * TPQ, *pxm = src + ixm * TPQ, *pyp = src + iyp * TPQ,
+              *pym = src + iym * TPQ;
+  uint4 *wc = src + i2 * TPQ;
+  const Word *Jb = p.J + b * (int64_t)plane * 2;
+  uint32_t Jxp[TPQ], Jxm[TPQ], Jyp[TPQ], Jym[TPQ];   // by 32-bit half of the words
   const uint32_t tau0 = 2u * (segu * (uint32_t)p.seg_base + min(segu, (uint32_t)p.seg_rem)) +
-                        (uint32_t)((colour + x + y) & 1);
+                        (uint32_t)((1 + x + y) & 1);
   const int G = p.seg_base + (segb < (uint32_t)p.seg_rem ? 1 : 0);
   const uint32_t ctr_z = (uint32_t)s | ((uint32_t)q << 16);
-  const uint32_t ctr_w = (DOM_SWEEP << 28) | (uint32_t)((b * 32) >> 6);
+  const uint32_t ctr_w = (DOM_SWEEP << 28) | ((b * (uint32_t)p.W) >> 6);
 
   VCount<uint32_t, KS> cs[4];
   VCount<uint32_t, KT> ct[4];
-  if (BLUE)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      cs[j].zero();
-      ct[j].zero();
-    }
+  for (int j = 0; j < 4; ++j) {
+    cs[j].zero();
+    ct[j].zero();
+  }
 
+  [[maybe_unused]] const unsigned walkers = TPQ == 1 ? 0u : __ballot_sync(0xffffffffu, live);   // whole sites
   if (live) {
-    Jxp = Jb[2 * i2];
-    Jxm = Jb[2 * ixm];
-    Jyp = Jb[2 * i2 + 1];
-    Jym = Jb[2 * iym + 1];
-    uint32_t off = tau0 * P;
-    uint4 dn = ld_g<CG>(pc + (size_t)(tau0 == 0 ? (Lt - 1) * P : off - P));
+    {
+      const Word jxp = Jb[2 * i2], jxm = Jb[2 * ixm], jyp = Jb[2 * i2 + 1], jym = Jb[2 * iym + 1];
+#pragma unroll
+      for (int k = 0; k < TPQ; ++k) {
+        Jxp[k] = (uint32_t)(jxp >> (32 * k));
+        Jxm[k] = (uint32_t)(jxm >> (32 * k));
+        Jyp[k] = (uint32_t)(jyp >> (32 * k));
+        Jym[k] = (uint32_t)(jym >> (32 * k));
+      }
+    }
+    const uint32_t PS = P * TPQ;   // 16-byte words per plane
+    uint32_t off = tau0 * PS;      // of the current site's plane
+    const uint32_t anti = ones_if<uint32_t>(p.tau_ap);   // the antiperiodic wrap bond is unsatisfied when its spins agree
+    uint4 dn = ld_g<CG>(pc + (size_t)(tau0 == 0 ? (Lt - 1) * PS : off - PS));
+    if (tau0 == 0) {
+      dn.x ^= anti;
+      dn.y ^= anti;
+      dn.z ^= anti;
+      dn.w ^= anti;
+    }
     Quad4 cur;
     cur.c = ld_g<CG>(pc + off);
-    cur.up = ld_g<CG>(pc + (size_t)(tau0 + 1 == Lt ? 0u : off + P));
+    cur.up = ld_g<CG>(pc + (size_t)(tau0 + 1 == Lt ? 0u : off + PS));
     cur.xp = ld_g<CG>(pxp + off);
     cur.xm = ld_g<CG>(pxm + off);
     cur.yp = ld_g<CG>(pyp + off);
     cur.ym = ld_g<CG>(pym + off);
-    uint4 R4 = philox(make_uint4((uint32_t)i2 + off, (uint32_t)t, ctr_z, ctr_w), p.key);
+    // the draws of a site: one Philox call.  W = 64: two sites' calls are
+    // made by the two threads of the site, thread h the one of site k + h (k
+    // even), and each passes the other the two draws it needs
+    uint32_t zsite = (uint32_t)i2 + tau0 * P + (TPQ == 1 ? 0u : h * 2 * P);   // of the next call
+    auto call = [&]() {
+      const uint4 v = philox(make_uint4(zsite, (uint32_t)t, ctr_z, ctr_w), p.key);
+      zsite += 2 * P * TPQ;
+      return v;
+    };
+    uint4 R4 = call();
+    uint2 got = make_uint2(0u, 0u);
     // the even site's post-flip counts, held until the odd site's are added
     // with them (the prefetching walk of the per-pass launch)
     uint32_t h0[4], h1[4], h2[4], g0[4], g1[4];
@@ -965,32 +1005,48 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, cons
     auto site = [&](int k, Quad4 &cu, Quad4 &nx, auto phase) {
       constexpr int PH = decltype(phase)::value;
       const uint32_t tau = tau0 + 2u * (uint32_t)k;
-      // the draws of the walk's next site are made while this one is
-      // updated, so the Philox chain overlaps independent work
+      uint32_t R[4];   // draw of each word's replica
       uint4 R4n = R4;
-      if (k + 1 < G) R4n = philox(make_uint4((uint32_t)i2 + off + 2 * P, (uint32_t)t, ctr_z, ctr_w), p.key);
+      if constexpr (TPQ == 1) {
+        R[0] = R4.x;
+        R[1] = R4.y;
+        R[2] = R4.z;
+        R[3] = R4.w;
+        // the draws of the walk's next site are made while this one is
+        // updated, so the Philox chain overlaps independent work
+        if (k + 1 < G) R4n = call();
+      } else {
+        const bool odd = PH == 1 || (PH == 2 && (k & 1));
+        if (!odd) {
+          got.x = __shfl_xor_sync(walkers, h ? R4.x : R4.z, 1);
+          got.y = __shfl_xor_sync(walkers, h ? R4.y : R4.w, 1);
+        }
+        const bool own = odd == (h != 0);   // this thread made the site's call
+        R[0] = R[1] = own ? (h ? R4.z : R4.x) : got.x;
+        R[2] = R[3] = own ? (h ? R4.w : R4.y) : got.y;
+        if (odd && k + 1 < G) R4n = call();
+      }
       auto load_next = [&](Quad4 &q) {
-        const uint32_t offn = off + 2 * P;
+        const uint32_t offn = off + 2 * PS;
         q.c = ld_g<CG>(pc + offn);
-        q.up = ld_g<CG>(pc + (size_t)(tau + 3 == Lt ? 0u : offn + P));
+        q.up = ld_g<CG>(pc + (size_t)(tau + 3 == Lt ? 0u : offn + PS));
         q.xp = ld_g<CG>(pxp + offn);
         q.xm = ld_g<CG>(pxm + offn);
         q.yp = ld_g<CG>(pyp + offn);
         q.ym = ld_g<CG>(pym + offn);
       };
       if (PF && k + 1 < G) load_next(nx);
-      // the antiperiodic wrap bond is unsatisfied when its spins agree
-      const uint32_t gtp = ones_if<uint32_t>(p.tau_ap && tau + 1 == Lt), gtm = ones_if<uint32_t>(p.tau_ap && tau == 0);
+      const uint32_t gtp = tau + 1 == Lt ? anti : 0u;
       uint32_t f[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const uint32_t sc = q4(cu.c, j);
-        const uint32_t b1 = sc ^ q4(cu.xp, j) ^ Jxp;
-        const uint32_t b2 = sc ^ q4(cu.xm, j) ^ Jxm;
-        const uint32_t b3 = sc ^ q4(cu.yp, j) ^ Jyp;
-        const uint32_t b4 = sc ^ q4(cu.ym, j) ^ Jym;
+        const uint32_t b1 = sc ^ q4(cu.xp, j) ^ Jxp[j % TPQ];
+        const uint32_t b2 = sc ^ q4(cu.xm, j) ^ Jxm[j % TPQ];
+        const uint32_t b3 = sc ^ q4(cu.yp, j) ^ Jyp[j % TPQ];
+        const uint32_t b4 = sc ^ q4(cu.ym, j) ^ Jym[j % TPQ];
         const uint32_t t1 = sc ^ q4(cu.up, j) ^ gtp;
-        const uint32_t t2 = sc ^ q4(dn, j) ^ gtm;
+        const uint32_t t2 = sc ^ q4(dn, j);
         const uint32_t s1 = b1 ^ b2 ^ b3;
         const uint32_t c1 = maj3(b1, b2, b3);
         const uint32_t us0 = s1 ^ b4;
@@ -999,38 +1055,37 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, cons
         const uint32_t us2 = c1 & c2;
         const uint32_t ut0 = t1 ^ t2;
         const uint32_t ut1 = t1 & t2;
-        const uint32_t flip = count_only ? 0u : accept_mask(q4(R4, j), C, us0, us1, us2, ut0, ut1, p.one);
+        const uint32_t nz = t1 | t2;
+        const uint32_t flip = count_only ? 0u : accept_mask(R[j], C, us0, us1, us2, nz, ut1, p.one);
         f[j] = flip;
-        if (BLUE) {
-          // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
-          const uint32_t vs1 = us1 ^ (flip & us0);
-          const uint32_t vs2 = mux(flip, ~(us0 | us1 | us2), us2);
-          const uint32_t vt1 = mux(flip, ~(ut0 | ut1), ut1);
-          if constexpr (PH == 0) {
-            h0[j] = us0;
-            h1[j] = vs1;
-            h2[j] = vs2;
-            g0[j] = ut0;
-            g1[j] = vt1;
-          } else if constexpr (PH == 1) {
-            cs[j].add3x2(h0[j], h1[j], h2[j], us0, vs1, vs2);
-            ct[j].add2x2(g0[j], g1[j], ut0, vt1);
-          } else {
-            cs[j].add3(us0, vs1, vs2);
-            ct[j].add2(ut0, vt1);
-          }
+        // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
+        const uint32_t vs1 = us1 ^ (flip & us0);
+        const uint32_t vs2 = mux(flip, ~(us0 | us1 | us2), us2);
+        const uint32_t vt1 = mux(flip, ~nz, ut1);
+        if constexpr (PH == 0) {
+          h0[j] = us0;
+          h1[j] = vs1;
+          h2[j] = vs2;
+          g0[j] = ut0;
+          g1[j] = vt1;
+        } else if constexpr (PH == 1) {
+          cs[j].add3x2(h0[j], h1[j], h2[j], us0, vs1, vs2);
+          ct[j].add2x2(g0[j], g1[j], ut0, vt1);
+        } else {
+          cs[j].add3(us0, vs1, vs2);
+          ct[j].add2(ut0, vt1);
         }
       }
       if (!count_only) wc[off] = make_uint4(cu.c.x ^ f[0], cu.c.y ^ f[1], cu.c.z ^ f[2], cu.c.w ^ f[3]);
       R4 = R4n;
       dn = cu.up;
       if (!PF && k + 1 < G) load_next(nx);
-      off += 2 * P;
+      off += 2 * PS;
     };
     using Hold = std::integral_constant<int, 0>;
     using Pair = std::integral_constant<int, 1>;
     using One = std::integral_constant<int, 2>;
-    if constexpr (BLUE && PF && !CG) {
+    if constexpr (PF && !CG) {
       // two sites per iteration: the current and next sites' words swap
       // registers instead of being copied, and their counts enter the
       // counters together (not in the persistent kernel, whose register
@@ -1055,21 +1110,29 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<uint32_t> &p, cons
     }
   }
 
-  if (BLUE) {
-    block_sum_counters<KS, 4>(cs, buf, tot);
-    block_sum_counters<KT, 4>(ct, buf, tot + 4 * 32);
-    {
-      const int w = threadIdx.x;   // 128 = 4 replicas x 32 lanes
-      const int jj = w >> 5, lane = w & 31;
-      const int rr = 4 * q + jj;
-      const int64_t a = b * 32 + lane;
-      if (rr < p.n_rep) {
-        unsigned long long *u = p.U + ((a * p.n_rep + rr) * p.n_slots + s) * 2;
-        if (tot[w]) atomicAdd(u, (unsigned long long)tot[w]);
-        if (tot[4 * 32 + w]) atomicAdd(u + 1, (unsigned long long)tot[4 * 32 + w]);
-      }
-    }
+  if (CG) __syncthreads();   // the previous virtual block's sums are read
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+#pragma unroll
+    for (int i = 0; i < KS; ++i) buf[(j * KS + i) * kBlock4 + threadIdx.x] = cs[j].p[i];
+#pragma unroll
+    for (int i = 0; i < KT; ++i) buf[(4 * KS + j * KT + i) * kBlock4 + threadIdx.x] = ct[j].p[i];
   }
+  __syncthreads();
+  // warp 0: u_s of words 0, 1; 1: of 2, 3; 2 and 3: u_t
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, pr = warp & 1;
+  int v[2 * TPQ];
+  if (warp < 2) planes_lane_sums<KS, TPQ>(buf, pr, v);
+  else planes_lane_sums<KT, TPQ>(buf + 4 * KS * kBlock4, pr, v);
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int hh = 0; hh < TPQ; ++hh) {   // word 2 pr + k of thread hh of the site
+      const int rr = 4 * q + (TPQ == 1 ? 2 * pr + k : 2 * hh + pr), n = v[k * TPQ + hh];
+      const int64_t a = (int64_t)b * p.W + (TPQ == 1 ? 0 : 32 * k) + lane;
+      if (rr < p.n_rep && n)
+        atomicAdd(p.U + ((a * p.n_rep + rr) * p.n_slots + s) * 2 + (warp >> 1), (unsigned long long)n);
+    }
 }
 
 
@@ -1142,21 +1205,20 @@ __device__ __forceinline__ void pt_in_blue_tail(const PTFold &f, uint2 key, unsi
   if (tk == nb - 1 && threadIdx.x == 0) *f.d_t = t + 1;   // every block read t at its start
 }
 
-template <bool BLUE, int KS, bool PF, int MINB = 0>
-__global__ void __launch_bounds__(kBlock4, MINB) samples_sweep4_kernel(SamplesArgs<uint32_t> p,
+template <typename Word, int KS, bool PF, int MINB = 0>
+__global__ void __launch_bounds__(kBlock4, MINB) samples_sweep4_kernel(const SamplesArgs<Word> p,
                                                                   const __grid_constant__ SlotThresholds th,
-                                                                  int colour, int count_only, const PTFold f) {
+                                                                  int count_only, const PTFold f) {
   pdl_begin();
-  {   // counters / masks the host asked this pass to clear (nothing reads them before the next pass)
+  {   // masks the host asked this pass to clear (nothing reads them before the next pass)
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_U; i += stride) p.zero_U[i] = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_acc; i += stride)
       p.zero_acc[i] = 0;
   }
   const unsigned long long t = *p.d_t;
   if (p.t_copy && blockIdx.x == 0 && threadIdx.x == 0) *p.t_copy = t;
-  sweep4_body<BLUE, KS, PF, false>(p, th, blockIdx.x, t, colour, count_only);
-  if (BLUE && f.P > 0) pt_in_blue_tail(f, p.key, t);
+  sweep4_body<Word, KS, PF, false>(p, th, blockIdx.x, t, count_only);
+  if (sizeof(Word) == 4 && f.P > 0) pt_in_blue_tail(f, p.key, t);
 }
 
 
@@ -1254,19 +1316,16 @@ __global__ void __launch_bounds__(kBlock4) samples_permute4_kernel(uint4 *spins,
 // Overlaps (Appendix E.1) of every replica pair at one slot, for up to 4
 // replicas (one replica quad): a thread reads the quad of G sites of one
 // (b, s) once and counts, per pair, the sites where the two configurations
-// differ (per lane, bit-sliced); the block sums its threads' counters (tree
-// in shared memory, in two batches of three pairs) and adds lane a's counts
-// into qcnt[a][s][p].  Pairs p in the order (0,1), (0,2), (0,3), (1,2),
+// differ (per lane, bit-sliced); the block sums its threads' counters and
+// adds lane a's counts into qcnt[a][s][p].  Pairs p in the order (0,1), (0,2), (0,3), (1,2),
 // (1,3), (2,3) restricted to the replicas present.
 template <typename Word, int K>
 __global__ void __launch_bounds__(kBlock4) samples_overlap4_kernel(const Word *spins, long long *qcnt, int64_t N,
                                                                     int n_slots, int n_rep, int64_t n_samples,
                                                                     int sites_per_thread, int blocks_per_set) {
   pdl_begin();
-  constexpr int W = (int)sizeof(Word) * 8;
-  constexpr int KF = K + kLog2Block4;
-  __shared__ Word buf[3 * KF * kBlock4];
-  __shared__ int tot[6 * W];
+  constexpr int W = (int)sizeof(Word) * 8, HW = W / 32;
+  __shared__ uint32_t buf[6 * HW * K * kBlock4];
   const int64_t set = blockIdx.x / blocks_per_set;   // (b, s)
   const int chunk = (int)(blockIdx.x - set * blocks_per_set);
   const int s = (int)(set % n_slots);
@@ -1310,19 +1369,30 @@ __global__ void __launch_bounds__(kBlock4) samples_overlap4_kernel(const Word *s
       c[pp].add3(b0, c1 ^ c2, c1 & c2);
     }
   }
-  block_sum_counters<K, 3, Word>(c, buf, tot);
-  block_sum_counters<K, 3, Word>(c + 3, buf, tot + 3 * W);
-  // the pair index of (x, y) among the replicas present
+  // counter HW pp + h: pair pp, lanes 32 h .. 32 h + 31
+#pragma unroll
+  for (int pp = 0; pp < 6; ++pp)
+#pragma unroll
+    for (int h = 0; h < HW; ++h)
+#pragma unroll
+      for (int i = 0; i < K; ++i)
+        buf[((pp * HW + h) * K + i) * kBlock4 + threadIdx.x] = (uint32_t)(c[pp].p[i] >> (32 * h));
+  __syncthreads();
   const int n_pairs = n_rep * (n_rep - 1) / 2;
-  for (int w = threadIdx.x; w < 6 * W; w += blockDim.x) {
-    const int pp = w / W, lane = (int)(w - pp * W);
-    const int x = pp < 3 ? 0 : pp < 5 ? 1 : 2;
-    const int y = pp < 3 ? pp + 1 : pp < 5 ? pp - 1 : 3;
-    if (y >= n_rep || !tot[w]) continue;
-    const int p = x * n_rep - x * (x + 1) / 2 + (y - x - 1);
-    const int64_t a = b * W + lane;
-    if (a < n_samples) atomicAdd(reinterpret_cast<unsigned long long *>(&qcnt[(a * n_slots + s) * n_pairs + p]),
-                                 (unsigned long long)tot[w]);
+  for (int pr = threadIdx.x >> 5; pr < 3 * HW; pr += kBlock4 / 32) {
+    int v[2];
+    planes_lane_sums<K>(buf, pr, v);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int n = v[k], pp = (2 * pr + k) / HW, h = (2 * pr + k) % HW;
+      // the pair index of (x, y) among the replicas present
+      const int x = pp < 3 ? 0 : pp < 5 ? 1 : 2;
+      const int y = pp < 3 ? pp + 1 : pp < 5 ? pp - 1 : 3;
+      const int p = x * n_rep - x * (x + 1) / 2 + (y - x - 1);
+      const int64_t a = b * W + 32 * h + (threadIdx.x & 31);
+      if (y < n_rep && n && a < n_samples)
+        atomicAdd(reinterpret_cast<unsigned long long *>(&qcnt[(a * n_slots + s) * n_pairs + p]), (unsigned long long)n);
+    }
   }
 }
 
@@ -1573,7 +1643,7 @@ __global__ void __launch_bounds__(kBlock4, 3) samples_persistent_kernel(const Pe
     SamplesArgs<uint32_t> bp = a.blue;
     bp.spins = a.buf[cur ^ 1];
     for (int vb = blockIdx.x; vb < a.blue_blocks; vb += gridDim.x)
-      sweep4_body<true, KS, true, true>(bp, th, vb, t, 1, 0);
+      sweep4_body<uint32_t, KS, true, true>(bp, th, vb, t, 0);
     if (!grid_barrier(a.bar, a.err, a.wait_ns)) return;
     for (int64_t c = gwarp; c < n_chains; c += warps) {   // whole warps: c is uniform over the warp
       const int64_t sa = c / a.n_rep;
@@ -1607,8 +1677,6 @@ SamplesArgs<Word> make_args(qisg_handle *h, int colour) {
   p.n_rep = h->n_rep;
   p.n_q = h->n_q;
   p.W = h->W;
-  p.zero_U = h->d_U;
-  p.n_zero_U = h->n_a_pad * h->n_rep * h->n_slots * 2;
   p.zero_acc = reinterpret_cast<Word *>(h->d_acc);
   p.n_zero_acc = h->n_b * h->n_rep * h->n_slots;
   p.one = 1u;
@@ -1653,28 +1721,21 @@ int counter_planes(int G) {
   return std::max(k, 3);
 }
 
-template <typename Word, bool BLUE, int G2>
-void launch_sweep(bool pdl, const SamplesArgs<Word> &p, const SlotThresholds &th, unsigned blocks, cudaStream_t st,
-                  int colour, int count_only) {
-  launch_kernel(pdl, samples_half_sweep_kernel<Word, BLUE, G2>, dim3(blocks), dim3(kBlock), 0, st, p, th, colour,
-                count_only);
-}
-
-template <typename Word, bool BLUE>
-void launch_sweep_g(bool pdl, const SamplesArgs<Word> &p, const SlotThresholds &th, unsigned blocks, cudaStream_t st,
-                    int colour, int count_only) {
-  // counter planes for G sites per thread: G2 = ceil(log2(G / 4))
+// The column walk with counter planes for G sites per thread: G2 = ceil(log2(G / 4)).
+void launch_sweep_g(bool pdl, const SamplesArgs<uint32_t> &p, const SlotThresholds &th, unsigned blocks, cudaStream_t st,
+                    int count_only) {
   int g2 = 0;
   while ((4 << g2) < p.seg_sites) ++g2;
+  auto go = [&](auto kern) { launch_kernel(pdl, kern, dim3(blocks), dim3(kBlock), 0, st, p, th, count_only); };
   switch (g2) {
-    case 0: launch_sweep<Word, BLUE, 0>(pdl, p, th, blocks, st, colour, count_only); break;
-    case 1: launch_sweep<Word, BLUE, 1>(pdl, p, th, blocks, st, colour, count_only); break;
-    case 2: launch_sweep<Word, BLUE, 2>(pdl, p, th, blocks, st, colour, count_only); break;
-    case 3: launch_sweep<Word, BLUE, 3>(pdl, p, th, blocks, st, colour, count_only); break;
-    case 4: launch_sweep<Word, BLUE, 4>(pdl, p, th, blocks, st, colour, count_only); break;
-    case 5: launch_sweep<Word, BLUE, 5>(pdl, p, th, blocks, st, colour, count_only); break;
-    case 6: launch_sweep<Word, BLUE, 6>(pdl, p, th, blocks, st, colour, count_only); break;
-    default: launch_sweep<Word, BLUE, 7>(pdl, p, th, blocks, st, colour, count_only); break;
+    case 0: go(samples_half_sweep_kernel<0>); break;
+    case 1: go(samples_half_sweep_kernel<1>); break;
+    case 2: go(samples_half_sweep_kernel<2>); break;
+    case 3: go(samples_half_sweep_kernel<3>); break;
+    case 4: go(samples_half_sweep_kernel<4>); break;
+    case 5: go(samples_half_sweep_kernel<5>); break;
+    case 6: go(samples_half_sweep_kernel<6>); break;
+    default: go(samples_half_sweep_kernel<7>); break;
   }
 }
 
@@ -1700,60 +1761,72 @@ constexpr int blue_min_blocks() {
   return MINB > 0 ? MINB : (PF && KS <= 7) ? 3 : 0;
 }
 
-// Blocks of the W = 32 blue kernel (variant 0 or 2, ks = 3 .. 9 counter
-// planes) resident on one SM, cached in the handle.
+// The blue kernel for ks = 3 .. 9 counter planes (variant 0 or 2; 64-bit words
+// have variant 0 only).
+template <typename Word>
+auto blue_kernel(int ks, int variant) {
+  using Fn = void (*)(SamplesArgs<Word>, SlotThresholds, int, PTFold);
+  Fn fn = nullptr;
+#define QISG_CASE(n)                                                                                      \
+  case n:                                                                                                 \
+    fn = (Fn)samples_sweep4_kernel<Word, n, true, blue_min_blocks<true, 0, n>()>;                          \
+    if constexpr (sizeof(Word) == 4)                                                                      \
+      if (variant == 2) fn = (Fn)samples_sweep4_kernel<Word, n, false, 4>;                                  \
+    break;
+  switch (std::min(std::max(ks, 3), 9)) {
+    QISG_CASE(3) QISG_CASE(4) QISG_CASE(5) QISG_CASE(6) QISG_CASE(7) QISG_CASE(8) QISG_CASE(9)
+  }
+#undef QISG_CASE
+  return fn;
+}
+
+// Blocks of that kernel resident on one SM, cached in the handle.
+template <typename Word>
 int blue_blocks_per_sm(qisg_handle *h, int ks, int variant) {
-  const int v = variant == 2 ? 1 : 0;
+  const int v = sizeof(Word) == 8 ? 2 : variant == 2 ? 1 : 0;
   ks = std::min(std::max(ks, 3), 9);
   int &c = h->blue_occ[v][ks - 3];
   if (c > 0) return c;
-  const void *fn = nullptr;
-#define QISG_OCC(n)                                                                                   \
-  case n:                                                                                             \
-    fn = v ? (const void *)samples_sweep4_kernel<true, n, false, 4>                                   \
-           : (const void *)samples_sweep4_kernel<true, n, true, blue_min_blocks<true, 0, n>()>;         \
-    break;
-  switch (ks) { QISG_OCC(3) QISG_OCC(4) QISG_OCC(5) QISG_OCC(6) QISG_OCC(7) QISG_OCC(8) default: QISG_OCC(9) }
-#undef QISG_OCC
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock4, 0) != cudaSuccess || per_sm < 1) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)blue_kernel<Word>(ks, variant), kBlock4, 0) !=
+          cudaSuccess ||
+      per_sm < 1) {
     (void)cudaGetLastError();
     per_sm = 1;
   }
   return c = per_sm;
 }
 
-// Blocks of one (b, s, q) set for n_seg segments per column: a block per
-// (segment, 128 columns) when the plane is a multiple of 128 (walk lengths
-// may then differ between segments), else 128 consecutive (segment, column)
-// pairs per block (segments of one length).
-int64_t blocks_per_set4(int plane, int n_seg) {
-  return plane % kBlock4 == 0 ? (int64_t)(plane / kBlock4) * n_seg
-                              : ((int64_t)plane * n_seg + kBlock4 - 1) / kBlock4;
+// Blocks of one (b, s, q) set for n_seg segments per column and cols columns
+// per block: a block per (segment, cols columns) when the plane is a multiple
+// of cols (walk lengths may then differ between segments), else cols
+// consecutive (segment, column) pairs per block (segments of one length).
+int64_t blocks_per_set4(int plane, int n_seg, int cols) {
+  return plane % cols == 0 ? (int64_t)(plane / cols) * n_seg : ((int64_t)plane * n_seg + cols - 1) / cols;
 }
 
 // Segments per column of the blue pass when no tile is pinned: the count
 // that minimises (waves of blocks over the resident ones) x (work of one
 // block), a block's work being its threads' walks of G sites on average
 // (about 490 instructions a site for the four replica words) plus its
-// counter tree (about 32 instructions per counter plane and level): the
+// counter tree (about 14 instructions per counter plane and level): the
 // pass is latency-bound, so a block takes about the same time whatever the
 // blocks beside it on the SM.  Walks of at most max_walk sites; counts that
 // leave segments of unequal length are candidates only when a block holds
 // one segment.  resident(ks) gives the resident blocks for ks counter
 // planes.
 template <typename Resident>
-int wave_fill_segments(int64_t sets, int plane, int half_col, int max_walk, Resident resident) {
+int wave_fill_segments(int64_t sets, int plane, int half_col, int max_walk, int cols, Resident resident) {
   int best = half_col;
   double best_cost = -1.0;
   for (int ns = std::max(1, (half_col + max_walk - 1) / max_walk); ns <= half_col; ++ns) {
-    if (plane % kBlock4 != 0 && half_col % ns != 0) continue;
+    if (plane % cols != 0 && half_col % ns != 0) continue;
     const int gmax = (half_col + ns - 1) / ns;
     const int ks = counter_planes(gmax);
     const int64_t R = std::max<int64_t>(1, resident(ks));
-    const int64_t blocks = sets * blocks_per_set4(plane, ns);
+    const int64_t blocks = sets * blocks_per_set4(plane, ns, cols);
     const int64_t waves = (blocks + R - 1) / R;
-    const double cost = (double)waves * (490.0 * half_col / ns + 32.0 * (2 * ks + 13));
+    const double cost = (double)waves * (490.0 * half_col / ns + 14.0 * (2 * ks + 13));
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
       best = ns;
@@ -1762,75 +1835,44 @@ int wave_fill_segments(int64_t sets, int plane, int half_col, int max_walk, Resi
   return best;
 }
 
-// W = 32 kernel: one thread per column segment.  A pinned tile G gives
-// ceil((L_tau / 2) / G) segments of at most G sites (planes that are not a
-// multiple of 128: the largest divisor of L_tau / 2 not above G); the
-// default gives the
-// blue pass the wave-filling count above (resident_blocks: the launch's
-// resident blocks, 0 = those of the blue kernel itself; walks of at most
-// max_walk sites) and the red pass as many sites per thread as keep about
-// half the old kernel's thread count.
-SamplesArgs<uint32_t> make_args4(qisg_handle *h, int colour, SlotThresholds &th, int64_t resident_blocks = 0,
-                                 int max_walk = 64) {
-  SamplesArgs<uint32_t> p = make_args<uint32_t>(h, colour);
+// Blue pass: one thread (W = 64: two) per column segment and replica quad.  A
+// pinned tile G gives ceil((L_tau / 2) / G) segments of at most G sites (4 G,
+// at most 64, for 64-bit words; planes that are not a multiple of the block's
+// columns: the largest divisor of L_tau / 2 not above it); the default is the
+// wave-filling count above (resident_blocks: the launch's resident blocks, 0 =
+// those of the blue kernel itself; walks of at most max_walk sites).
+template <typename Word>
+SamplesArgs<Word> make_args4(qisg_handle *h, SlotThresholds &th, int64_t resident_blocks = 0, int max_walk = 64) {
+  SamplesArgs<Word> p = make_args<Word>(h, 1);
+  constexpr int cols = kBlock4 / ((int)sizeof(Word) / 4);
   const int half_col = h->Lt / 2;
   const int64_t sets = h->n_b * h->n_slots * h->n_q;
-  const int tile = std::min(h->sweep_tile[colour], half_col);
+  const int sites = sizeof(Word) == 8 ? std::min(4 * h->sweep_tile[1], 64) : h->sweep_tile[1];
+  const int tile = std::min(sites, half_col);
   int n_seg;
-  if (tile > 0 && p.plane % kBlock4 == 0) {
+  if (tile > 0 && p.plane % cols == 0) {
     n_seg = (half_col + tile - 1) / tile;
   } else if (tile > 0) {
     int G = tile;
     while (G > 1 && half_col % G) --G;
     n_seg = half_col / G;
-  } else if (colour == 1) {
-    const int variant = h->sweep_variant[1];
-    n_seg = wave_fill_segments(sets, p.plane, half_col, max_walk, [&](int ks) -> int64_t {
-      return resident_blocks > 0 ? resident_blocks : (int64_t)blue_blocks_per_sm(h, ks, variant) * std::max(1, h->n_sm);
-    });
   } else {
-    const int64_t want_threads = (int64_t)h->sweep_min_blocks_per_sm * std::max(1, h->n_sm) * kBlock / 2;
-    int G = 64;
-    while (G > 1 && sets * p.plane * (int64_t)(half_col / std::min(G, half_col)) < want_threads) G >>= 1;
-    if (G > half_col) G = half_col;
-    while (G > 1 && half_col % G) --G;
-    n_seg = half_col / G;
+    const int variant = h->sweep_variant[1];
+    n_seg = wave_fill_segments(sets, p.plane, half_col, max_walk, cols, [&](int ks) -> int64_t {
+      return resident_blocks > 0 ? resident_blocks
+                                 : (int64_t)blue_blocks_per_sm<Word>(h, ks, variant) * std::max(1, h->n_sm);
+    });
   }
   p.n_seg = n_seg;
   p.seg_base = half_col / n_seg;
   p.seg_rem = half_col % n_seg;
   p.seg_sites = p.seg_base + (p.seg_rem > 0 ? 1 : 0);
-  p.seg_blocks = p.plane % kBlock4 == 0 ? p.plane / kBlock4 : 0;
+  p.seg_blocks = p.plane % cols == 0 ? p.plane / cols : 0;
   p.fd_sb = FastDiv((uint32_t)std::max(1, p.seg_blocks));
-  p.blocks_per_set = (int)blocks_per_set4(p.plane, n_seg);
+  p.blocks_per_set = (int)blocks_per_set4(p.plane, n_seg, cols);
   p.fd_bps = FastDiv((uint32_t)p.blocks_per_set);
   fill_thresholds(h, th);
   return p;
-}
-
-// MINB > 0: the kernel's registers are bounded so that MINB blocks fit on an
-// SM (variant 2 of the blue pass: more resident warps, no prefetch).
-template <bool BLUE, bool PF, int MINB = 0>
-void launch_sweep4(bool pdl, const SamplesArgs<uint32_t> &p, const SlotThresholds &th, unsigned blocks, cudaStream_t st,
-                   int colour, int count_only, const PTFold &f = PTFold{}) {
-  if constexpr (!BLUE) {   // the red pass keeps no counters
-    launch_kernel(pdl, samples_sweep4_kernel<false, 3, PF>, dim3(blocks), dim3(kBlock4), 0, st, p, th, colour,
-                  count_only, f);
-  } else {
-    switch (counter_planes(p.seg_sites)) {   // walks of at most 64 sites: 3 .. 9 planes
-#define QISG_CASE(n)                                                                                         \
-  case n:                                                                                                    \
-    launch_kernel(pdl, samples_sweep4_kernel<true, n, PF, blue_min_blocks<PF, MINB, n>()>, dim3(blocks),      \
-                  dim3(kBlock4), 0, st, p, th, colour, count_only, f);                                       \
-    break;
-      QISG_CASE(3) QISG_CASE(4) QISG_CASE(5) QISG_CASE(6) QISG_CASE(7) QISG_CASE(8)
-      default:
-        launch_kernel(pdl, samples_sweep4_kernel<true, 9, PF, blue_min_blocks<PF, MINB, 9>()>, dim3(blocks),
-                      dim3(kBlock4), 0, st, p, th, colour, count_only, f);
-        break;
-#undef QISG_CASE
-    }
-  }
 }
 
 // Arguments of the fused red pass (and its threads per site, from the red
@@ -1847,7 +1889,7 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
   p.acc = reinterpret_cast<const Word *>(h->d_acc);
   p.d_t = h->d_t;
   p.zero_U = h->d_U;
-  p.n_zero_U = a.n_zero_U;
+  p.n_zero_U = h->n_a_pad * h->n_rep * h->n_slots * 2;
   p.key = a.key;
   p.N = h->N;
   p.L = h->L;
@@ -1912,21 +1954,20 @@ int fused_red(qisg_handle *h) {
 
 template <typename Word>
 int half_sweep_t(qisg_handle *h, int colour, int count_only) {
-  if (h->fused && colour == 0 && !count_only) return fused_red<Word>(h);
-  // W = 32, blue variants 0 and 2 (and the counting red pass): a thread per
-  // (column segment, replica quad), variant 2 with its registers bounded to
-  // four blocks per SM; otherwise the column walk, a thread per (column
-  // segment, replica)
-  if (sizeof(Word) == 4 && !(colour == 1 && h->sweep_variant[1] == 1)) {
+  if (colour == 0 && !count_only) return fused_red<Word>(h);
+  if (colour == 0) {   // energies of the stored state: the blue pass counts them
+    int rc = cuda_check(cudaMemsetAsync(h->d_U, 0, (size_t)h->n_a_pad * h->n_rep * h->n_slots * 16, h->stream), "clear counters");
+    if (!rc) rc = cuda_check(cudaMemsetAsync(h->d_acc, 0, (size_t)h->n_b * h->n_rep * h->n_slots * sizeof(Word), h->stream),
+                             "clear PT masks");
+    return rc;
+  }
+  // blue: a thread per (column segment, replica quad or half of it); variant 2
+  // of 32-bit words with its registers bounded to four blocks per SM, variant
+  // 1 the column walk, a thread per (column segment, replica)
+  if (sizeof(Word) == 8 || h->sweep_variant[1] != 1) {
     SlotThresholds th;
-    SamplesArgs<uint32_t> p = make_args4(h, colour, th);
-    if (h->fused && colour == 1) {   // the fused red pass read the masks: clear them here
-      p.n_zero_U = 0;
-      if (!count_only) p.t_copy = h->d_t + 1;
-    } else if (colour == 1) {
-      p.n_zero_U = 0;
-      p.n_zero_acc = 0;
-    }
+    SamplesArgs<Word> p = make_args4<Word>(h, th);
+    if (!count_only) p.t_copy = h->d_t + 1;   // the fused red pass read the masks: they are cleared here
     const int64_t blocks = h->n_b * h->n_slots * h->n_q * p.blocks_per_set;
     if (blocks > 0x7FFFFFFF || (int64_t)p.blocks_per_set * kBlock4 > 0x7FFFFFFF)
       return fail(QISG_EINVAL, "lattice too large for one launch");
@@ -1935,11 +1976,11 @@ int half_sweep_t(qisg_handle *h, int colour, int count_only) {
     // blocks, energy differences fit 32 bits and the sweep's PT is due
     PTFold f{};
     h->pt_folded = false;
-    if (colour == 1 && h->fused && !count_only && h->pt_in_blue && h->pt_every > 0 &&
+    if (sizeof(Word) == 4 && !count_only && h->pt_in_blue && h->pt_every > 0 &&
         (h->t + 1) % (uint64_t)h->pt_every == 0 && 2 * h->N < (int64_t(1) << 30) && h->n_slots <= kMaxSlotsPT) {
       const int64_t chains = h->n_samples * h->n_rep;
       const int64_t P = (chains + kBlock4 / 32 - 1) / (kBlock4 / 32);
-      const int64_t resident = (int64_t)blue_blocks_per_sm(h, counter_planes(p.seg_sites), h->sweep_variant[1]) *
+      const int64_t resident = (int64_t)blue_blocks_per_sm<Word>(h, counter_planes(p.seg_sites), h->sweep_variant[1]) *
                                std::max(1, h->n_sm);
       if (P >= 1 && 2 * P <= blocks && 2 * P <= resident) {
         f.P = (int)P;
@@ -1960,41 +2001,27 @@ int half_sweep_t(qisg_handle *h, int colour, int count_only) {
       }
     }
     const int tok = prof_begin(h, sweep_kind(colour));
-    // the blue pass loads the next site of its walk while it updates the
-    // current one (measured: 4% off the production sweep, with the tuner then
-    // taking walks of 4 sites)
-    if (colour == 1 && h->sweep_variant[1] == 2)
-      launch_sweep4<true, false, 4>(h->pdl, p, th, (unsigned)blocks, h->stream, 1, count_only, f);
-    else if (colour == 1)
-      launch_sweep4<true, true>(h->pdl, p, th, (unsigned)blocks, h->stream, 1, count_only, f);
-    else
-      launch_sweep4<false, false>(h->pdl, p, th, (unsigned)blocks, h->stream, 0, count_only);
+    // walks of at most 64 sites: 3 .. 9 counter planes
+    launch_kernel(h->pdl, blue_kernel<Word>(counter_planes(p.seg_sites), h->sweep_variant[1]), dim3((unsigned)blocks),
+                  dim3(kBlock4), 0, h->stream, p, th, count_only, f);
     prof_end(h, sweep_kind(colour), tok);
     h->launches++;
     return cuda_check(cudaGetLastError(), "samples half sweep");
   }
-  SamplesArgs<Word> p = make_args<Word>(h, colour);
-  SlotThresholds th;
-  fill_thresholds(h, th);
-  if (colour == 1) {
-    p.n_zero_U = 0;
-    if (h->fused) {   // masks read by the fused red pass: clear them here
-      if (!count_only) p.t_copy = h->d_t + 1;
-    } else {
-      p.n_zero_acc = 0;
-    }
+  if constexpr (sizeof(Word) == 4) {
+    SamplesArgs<Word> p = make_args<Word>(h, colour);
+    SlotThresholds th;
+    fill_thresholds(h, th);
+    if (!count_only) p.t_copy = h->d_t + 1;
+    const int64_t sets = h->n_b * h->n_slots * h->n_q;
+    const int64_t blocks = sets * p.blocks_per_set;
+    if (blocks > 0x7FFFFFFF || (int64_t)p.blocks_per_set * kQuads > 0x7FFFFFFF)
+      return fail(QISG_EINVAL, "lattice too large for one launch");
+    const int tok = prof_begin(h, sweep_kind(colour));
+    launch_sweep_g(h->pdl, p, th, (unsigned)blocks, h->stream, count_only);
+    prof_end(h, sweep_kind(colour), tok);
+    h->launches++;
   }
-  const int64_t sets = h->n_b * h->n_slots * h->n_q;
-  const int64_t blocks = sets * p.blocks_per_set;
-  if (blocks > 0x7FFFFFFF || (int64_t)p.blocks_per_set * kQuads > 0x7FFFFFFF)
-    return fail(QISG_EINVAL, "lattice too large for one launch");
-  const int tok = prof_begin(h, sweep_kind(colour));
-  if (colour == 1)
-    launch_sweep_g<Word, true>(h->pdl, p, th, (unsigned)blocks, h->stream, 1, count_only);
-  else
-    launch_sweep<Word, false, 0>(h->pdl, p, th, (unsigned)blocks, h->stream, 0, count_only);
-  prof_end(h, sweep_kind(colour), tok);
-  h->launches++;
   return cuda_check(cudaGetLastError(), "samples half sweep");
 }
 
@@ -2316,8 +2343,7 @@ int samples_persistent(qisg_handle *h, int n_sweeps) {
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, samples_persistent_kernel<1, 5>, kBlock4, 0),
                   "occupancy");
   if (rc) return rc;
-  a.blue = make_args4(h, 1, th_blue, (int64_t)std::max(1, per_sm0) * std::max(1, h->n_sm), 32);
-  a.blue.n_zero_U = 0;
+  a.blue = make_args4<uint32_t>(h, th_blue, (int64_t)std::max(1, per_sm0) * std::max(1, h->n_sm), 32);
   a.blue.n_zero_acc = 0;
   a.blue.t_copy = nullptr;
   const int64_t blue_blocks = h->n_b * h->n_slots * h->n_q * a.blue.blocks_per_set;

@@ -426,3 +426,23 @@ def test_spins_of_sample_ranges(qisg, W):
         S = inst.spins()
         for lo, n in ((0, 1), (31, 2), (30, 70), (63, 1), (65, 85), (149, 1)):
             assert np.array_equal(inst.spins(lo, n), S[lo:lo + n]), (lo, n)
+
+
+@pytest.mark.parametrize("L,Lt,n_rep,n_a,tile,ap", [
+    (8, 14, 4, 70, 0, 0),      # a block per segment of 64 columns, seven sites a column
+    (8, 14, 3, 64, 1, 1),      # walks of four and three sites, a replica missing, antiperiodic
+    (6, 10, 5, 65, 16, 0),     # a plane that no block divides, a second replica quad, one walk of five sites
+    (16, 6, 2, 33, 1, 1),      # four blocks per plane, half a quad, a group of lanes empty
+])
+def test_blue_walks_of_64_bit_words(qisg, L, Lt, n_rep, n_a, tile, ap):
+    inst, ladder = make(qisg, L, Lt, 0.2, 0.5, 4, 0.9, n_rep, n_a, 17 + L, layout=qisg.QISG_LAYOUT_SAMPLES, word_bits=64,
+                        tau_antiperiodic=ap, measure_every=2)
+    st = oracle_state(ladder, L, Lt, n_rep, 17 + L, 0, n_a, tau_ap=bool(ap))
+    with inst:
+        inst.set_tiles((0, tile))
+        inst.sweep(6)
+        oracle.run(st, 6, measure_every=2)
+        assert_same_state(inst, st, what=f"L={L} Lt={Lt} tile {tile}")
+        sums = inst.measurements()
+    assert np.array_equal(sums[0], st.sumA) and np.array_equal(sums[1], st.sumB)
+    assert np.array_equal(sums[2], st.sumq) and np.array_equal(sums[3], st.sumq2)
