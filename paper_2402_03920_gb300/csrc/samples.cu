@@ -385,7 +385,6 @@ __device__ __forceinline__ uint32_t *addr_mad(const uint32_t *base, uint32_t i, 
 
 __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const FusedRedArgs p,
                                                                      const __grid_constant__ SlotThresholds th) {
-  pdl_begin();
   __shared__ uint32_t msk[4][kMaxSlotsPT];
   __shared__ unsigned long long thr[kMaxSlotsPT][9];
   __shared__ uint4 rnd[kBlock4];   // per warp: [slot in group][quad][replica]
@@ -395,12 +394,6 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
   const uint32_t b = p.fd_nq.div(set);
   const int q = (int)(set - b * (uint32_t)p.n_q);
   const int n = p.n_slots;
-  {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_U; i += stride) p.zero_U[i] = 0;
-    if (p.ticket && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0u;
-  }
-
   const uint32_t tid = chunk * (uint32_t)kBlock4 + threadIdx.x;
   const int j = (int)(tid & 3u);
   const uint32_t quad = tid >> 2;
@@ -431,6 +424,25 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
   uint32_t zo[7];
   const uint32_t *Jb = p.J + (int64_t)b * P * 2;
   uint32_t Jxp = 0, Jxm = 0, Jyp = 0, Jym = 0;
+  if (live) {
+    Jxp = Jb[2 * i2];
+    Jxm = Jb[2 * ixm];
+    Jyp = Jb[2 * i2 + 1];
+    Jym = Jb[2 * iym + 1];
+  }
+  // the slots' threshold constants through shared memory, so that the
+  // accept flags take them from ordinary registers: measured 6 fewer
+  // logic-pipe and 9 more multiply-add-pipe instructions per word, 2.1% off
+  // the L=16, L_tau=256 sweep (the replica-quad red and the blue kernels,
+  // which would hold them across their sites, lost by it)
+  for (int i = threadIdx.x; i < n * 9; i += blockDim.x) thr[i / 9][i % 9] = th.v[i / 9][i % 9];
+  // what came so far depends on no other kernel of the sweep
+  pdl_begin();
+  {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_U; i += stride) p.zero_U[i] = 0;
+    if (p.ticket && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0u;
+  }
   const unsigned long long t = *p.d_t;
   const uint32_t ctr_w = (DOM_SWEEP << 28) | ((b * 32u) >> 6);
   uint32_t cw[7], n1[7];   // carried words at the current slot; words of the next slot
@@ -439,10 +451,6 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
   const uint32_t *sb = p.src + base;
   uint32_t *db = p.dst + base;
   if (live) {
-    Jxp = Jb[2 * i2];
-    Jxm = Jb[2 * ixm];
-    Jyp = Jb[2 * i2 + 1];
-    Jym = Jb[2 * iym + 1];
 #pragma unroll
     for (int k = 0; k < 7; ++k) cw[k] = sb[zo[k]];
     if (n > 1)
@@ -515,12 +523,6 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
     const int rr = 4 * q + jj;
     msk[jj][sl] = (rr < p.n_rep && sl + 1 < n) ? p.acc[((int64_t)b * p.n_rep + rr) * n + sl] : 0u;
   }
-  // the slots' threshold constants through shared memory, so that the
-  // accept flags take them from ordinary registers: measured 6 fewer
-  // logic-pipe and 9 more multiply-add-pipe instructions per word, 2.1% off
-  // the L=16, L_tau=256 sweep (the replica-quad red and the blue kernels,
-  // which would hold them across their sites, lost by it)
-  for (int i = threadIdx.x; i < n * 9; i += blockDim.x) thr[i / 9][i % 9] = th.v[i / 9][i % 9];
   __syncthreads();
   for (; 4 * g + 6 <= n; ++g) {
     if (live) *reinterpret_cast<uint4 *>(rw + ((j * 8 + ql) << 2)) = r4;
@@ -897,9 +899,11 @@ __device__ __forceinline__ void planes_lane_sums(const uint32_t *buf, int pr, in
 // replica w (W = 32) or 2 h + w / 2.
 // KS: counter planes of a thread's u_s sum (at most 4 G, so KS =
 // counter_planes(G)); the u_t sum (at most 2 G) takes one plane less.
-template <typename Word, int KS, bool PF, bool CG>
+// begin() returns the sweep t; what comes before it depends on no other kernel
+// of the sweep.
+template <typename Word, int KS, bool PF, bool CG, typename Begin>
 __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const SlotThresholds &th, uint32_t bid,
-                                            unsigned long long t, int count_only) {
+                                            Begin begin, int count_only) {
   constexpr int KT = KS - 1, TPQ = (int)sizeof(Word) / 4;
   constexpr uint32_t kCols = kBlock4 / TPQ;   // columns per block
   __shared__ uint32_t buf[4 * (KS + KT) * kBlock4];   // u_s counters, then u_t
@@ -958,16 +962,17 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
 
   [[maybe_unused]] const unsigned walkers = TPQ == 1 ? 0u : __ballot_sync(0xffffffffu, live);   // whole sites
   if (live) {
-    {
-      const Word jxp = Jb[2 * i2], jxm = Jb[2 * ixm], jyp = Jb[2 * i2 + 1], jym = Jb[2 * iym + 1];
+    const Word jxp = Jb[2 * i2], jxm = Jb[2 * ixm], jyp = Jb[2 * i2 + 1], jym = Jb[2 * iym + 1];
 #pragma unroll
-      for (int k = 0; k < TPQ; ++k) {
-        Jxp[k] = (uint32_t)(jxp >> (32 * k));
-        Jxm[k] = (uint32_t)(jxm >> (32 * k));
-        Jyp[k] = (uint32_t)(jyp >> (32 * k));
-        Jym[k] = (uint32_t)(jym >> (32 * k));
-      }
+    for (int k = 0; k < TPQ; ++k) {
+      Jxp[k] = (uint32_t)(jxp >> (32 * k));
+      Jxm[k] = (uint32_t)(jxm >> (32 * k));
+      Jyp[k] = (uint32_t)(jyp >> (32 * k));
+      Jym[k] = (uint32_t)(jym >> (32 * k));
     }
+  }
+  const unsigned long long t = begin();
+  if (live) {
     const uint32_t PS = P * TPQ;   // 16-byte words per plane
     uint32_t off = tau0 * PS;      // of the current site's plane
     const uint32_t anti = ones_if<uint32_t>(p.tau_ap);   // the antiperiodic wrap bond is unsatisfied when its spins agree
@@ -1170,6 +1175,9 @@ __device__ __forceinline__ void pt_in_blue_tail(const PTFold &f, uint2 key, unsi
   }
   __syncthreads();
   const unsigned nb = gridDim.x, tk = s_tk;
+  // every block triggers the red pass once its own work is done, so that its
+  // blocks start (and get as far as their wait) beside the PT chains
+  pdl_trigger();
   if (tk + (unsigned)f.P < nb) return;   // not among the last P blocks
   if (threadIdx.x == 0) {
     int go = 1;
@@ -1209,15 +1217,18 @@ template <typename Word, int KS, bool PF, int MINB = 0>
 __global__ void __launch_bounds__(kBlock4, MINB) samples_sweep4_kernel(const SamplesArgs<Word> p,
                                                                   const __grid_constant__ SlotThresholds th,
                                                                   int count_only, const PTFold f) {
-  pdl_begin();
-  {   // masks the host asked this pass to clear (nothing reads them before the next pass)
+  unsigned long long t = 0;
+  auto begin = [&]() {
+    pdl_begin();
+    // masks the host asked this pass to clear (nothing reads them before the next pass)
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_acc; i += stride)
       p.zero_acc[i] = 0;
-  }
-  const unsigned long long t = *p.d_t;
-  if (p.t_copy && blockIdx.x == 0 && threadIdx.x == 0) *p.t_copy = t;
-  sweep4_body<Word, KS, PF, false>(p, th, blockIdx.x, t, count_only);
+    t = *p.d_t;
+    if (p.t_copy && blockIdx.x == 0 && threadIdx.x == 0) *p.t_copy = t;
+    return t;
+  };
+  sweep4_body<Word, KS, PF, false>(p, th, blockIdx.x, begin, count_only);
   if (sizeof(Word) == 4 && f.P > 0) pt_in_blue_tail(f, p.key, t);
 }
 
@@ -1643,7 +1654,7 @@ __global__ void __launch_bounds__(kBlock4, 3) samples_persistent_kernel(const Pe
     SamplesArgs<uint32_t> bp = a.blue;
     bp.spins = a.buf[cur ^ 1];
     for (int vb = blockIdx.x; vb < a.blue_blocks; vb += gridDim.x)
-      sweep4_body<uint32_t, KS, true, true>(bp, th, vb, t, 0);
+      sweep4_body<uint32_t, KS, true, true>(bp, th, vb, [t]() { return t; }, 0);
     if (!grid_barrier(a.bar, a.err, a.wait_ns)) return;
     for (int64_t c = gwarp; c < n_chains; c += warps) {   // whole warps: c is uniform over the warp
       const int64_t sa = c / a.n_rep;
