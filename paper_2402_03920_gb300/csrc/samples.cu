@@ -46,7 +46,7 @@ struct SamplesArgs {
                          // multiple of 128), so a block's walks have one length; 0: a block takes
                          // 128 consecutive (segment, column) pairs and seg_rem = 0
   int blocks_per_set;    // blocks per (b, s, q) word set
-  uint32_t one;          // 1 as a runtime value (accept_flag)
+  uint32_t one;          // 1 as a runtime value (take_if_less)
   unsigned long long *t_copy;   // blue pass, fused mode: copy t here for the PT pass
   int tau_ap;                   // antiperiodic along tau: the wrap tau bond flips sign
   // division by the invariants of the index decomposition (32-bit indices)
@@ -55,36 +55,55 @@ struct SamplesArgs {
   int64_t n_zero_acc;
 };
 
-// Accept constants per slot for the classes (u_t = 0: u_s = 0..4),
-// (u_t = 1: u_s = 0, 1), (u_t = 2: u_s = 0, 1); the classes u_t >= 1,
-// u_s >= 2 always accept.  A class with table entry T accepts a draw R iff
-// R < T', T' = T for a finite entry (T = 0: never) and T' = 2^32 for the
-// always-accept sentinel.  The slot holds C = 2^64 - T' (mod 2^64): R + C
-// stays below 2^64 iff R < T', and then its high word is 0xFFFFFFFF (R + C
-// >= 2^64 - 2^32), else 0.  So one 64-bit multiply-add, R * 1 + C, gives the
-// class's accept mask in its high word, on the integer multiply-add pipe
-// (leaving the logic pipe to the bit-sliced arithmetic).
+// Thresholds per slot of the classes (u_t = 0: u_s = 0..4), (u_t = 1: u_s = 0,
+// 1), (u_t = 2: u_s = 0, 1); the classes u_t >= 1, u_s >= 2 always accept.
 struct SlotThresholds {
-  unsigned long long v[kMaxSlotsPT][9];
+  uint32_t v[kMaxSlotsPT][9];
 };
 
-// one is the runtime value 1 (a kernel parameter, so the compiler keeps the
-// multiply-add rather than splitting it into two additions)
-__device__ __forceinline__ uint32_t accept_flag(uint32_t R, unsigned long long C, uint32_t one) {
-  unsigned long long v;
-  asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(v) : "r"(R), "r"(one), "l"(C));
-  return (uint32_t)(v >> 32);
+// v = R < T ? x : v by a predicated multiply-add (one is the runtime value 1):
+// the comparison is the only operation on the logic pipe, which binds the
+// passes, and the move runs on the multiply-add pipe.
+template <typename Word>
+__device__ __forceinline__ void take_if_less(Word &v, uint32_t R, uint32_t T, Word x, uint32_t one) {
+  if constexpr (sizeof(Word) == 4) {
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p mad.lo.u32 %0, %3, %4, 0;\n\t}"
+        : "+r"(v)
+        : "r"(R), "r"(T), "r"(x), "r"(one));
+  } else {
+    uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %2, %3;\n\t@p mad.lo.u32 %0, %4, %6, 0;\n\t@p mad.lo.u32 %1, %5, %6, 0;\n\t}"
+        : "+r"(lo), "+r"(hi)
+        : "r"(R), "r"(T), "r"((uint32_t)x), "r"((uint32_t)(x >> 32)), "r"(one));
+    v = ((Word)hi << 32) | lo;
+  }
 }
 
-// Accept mask of one 32-bit word: a mux tree over the class planes (u_s in
-// us2 us1 us0, u_t in ut1 ut0) of the per-class accept masks.  nz = ut0 | ut1.
-__device__ __forceinline__ uint32_t accept_mask(uint32_t R, const unsigned long long *C, uint32_t us0, uint32_t us1,
-                                                uint32_t us2, uint32_t nz, uint32_t ut1, uint32_t one) {
-#define QISG_A(c) accept_flag(R, C[c], one)
-  const uint32_t row0 = mux(us2, QISG_A(4), mux(us1, mux(us0, QISG_A(3), QISG_A(2)), mux(us0, QISG_A(1), QISG_A(0))));
-  const uint32_t low = mux(us0, mux(ut1, QISG_A(8), QISG_A(6)), mux(ut1, QISG_A(7), QISG_A(5)));   // u_t > 0, u_s < 2
-#undef QISG_A
-  return mux(nz, us1 | us2 | low, row0);
+// Accept mask of one word of draw R, T the slot's nine thresholds: a lane
+// accepts iff T of its class is 2^32 - 1 or R < T, and with R cut to 2^32 - 2
+// (no finite threshold exceeds that) both are R < T.  At fixed u_t the
+// threshold does not decrease with u_s (k >= 0), so the accepted lanes of a
+// row are those with u_s >= some l(R): a plane of the thermometer of u_s,
+// chosen by comparisons of the word's one draw.  Masks of each class (a 64-bit
+// addition each) and a mux tree over them took 28 logic operations per word:
+// the red pass with a thread per replica went from 483 to 424 us at 128
+// samples, L = 24, L_tau = 512, the production sweep from 35.0 to 32.8 us.
+template <typename Word>
+__device__ __forceinline__ Word accept_word(uint32_t R, const uint32_t *T, Word us0, Word us1, Word us2, Word ut0,
+                                            Word ut1, uint32_t one) {
+  const uint32_t r = min(R, 0xFFFFFFFEu);
+  const Word ge1 = us0 | us1 | us2, ge2 = us1 | us2, ge3 = us2 | (us1 & us0), all = ~Word(0);
+  Word m0 = 0, m1 = ge2, m2 = ge2;   // u_t = 0, 1, 2
+  take_if_less(m0, r, T[4], us2, one);
+  take_if_less(m0, r, T[3], ge3, one);
+  take_if_less(m0, r, T[2], ge2, one);
+  take_if_less(m0, r, T[1], ge1, one);
+  take_if_less(m0, r, T[0], all, one);
+  take_if_less(m1, r, T[6], ge1, one);
+  take_if_less(m1, r, T[5], all, one);
+  take_if_less(m2, r, T[8], ge1, one);
+  take_if_less(m2, r, T[7], all, one);
+  return mux(ut1, m2, mux(ut0, m1, m0));
 }
 
 // Per-replica-class sum of the block's counters: thread (quad, j) holds
@@ -128,24 +147,6 @@ __device__ __forceinline__ void quad_sum_counters(const VCount<Word, K> &c, Word
   __syncthreads();   // buf is reused by the caller
 }
 
-// Accept mask of one word for class planes (us, ut): the class masks are 32
-// bits wide (accept_flag), doubled for 64-bit words.
-template <typename Word>
-__device__ __forceinline__ Word accept_word(uint32_t R, const unsigned long long *C, Word us0, Word us1, Word us2,
-                                            Word nz, Word ut1, uint32_t one) {
-  if constexpr (sizeof(Word) == 4) {
-    return accept_mask(R, C, us0, us1, us2, nz, ut1, one);
-  } else {
-    auto f = [&](int c) -> Word {
-      const uint32_t m = accept_flag(R, C[c], one);
-      return ((Word)m << 32) | (Word)m;
-    };
-    const Word row0 = mux(us2, f(4), mux(us1, mux(us0, f(3), f(2)), mux(us0, f(1), f(0))));
-    const Word low = mux(us0, mux(ut1, f(8), f(6)), mux(ut1, f(7), f(5)));
-    return mux(nz, us1 | us2 | low, row0);
-  }
-}
-
 // Blue half sweep, column walk (32-bit words, variant 1).  Block: one (b, s, q) word set; quad thread j
 // owns replica r = 4q + j.  Quad k owns one (x, y) column and a segment of
 // G sites of the colour along tau (tau = tau0, tau0 + 2, ...; tau0 = 2 G seg
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_acc; i += stride)
       p.zero_acc[i] = 0;
   }
-  const unsigned long long *C = th.v[s];
+  const uint32_t *T = th.v[s];
 
   const int L = p.L, plane = p.plane, G = p.seg_sites;
   const uint32_t Lt = (uint32_t)p.Lt;
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
         const Word ut1 = t1 & t2;
         // accept mask: mux tree over (u_t, u_s) of the per-class masks
         const Word nz = t1 | t2;
-        const Word flip = count_only ? Word(0) : accept_mask(R, C, us0, us1, us2, nz, ut1, p.one);
+        const Word flip = count_only ? Word(0) : accept_word<Word>(R, T, us0, us1, us2, ut0, ut1, p.one);
         if (!count_only) base[(size_t)site * 4] = sc ^ flip;
         // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
         const Word vs1 = us1 ^ (flip & us0);
@@ -386,7 +387,6 @@ __device__ __forceinline__ uint32_t *addr_mad(const uint32_t *base, uint32_t i, 
 __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const FusedRedArgs p,
                                                                      const __grid_constant__ SlotThresholds th) {
   __shared__ uint32_t msk[4][kMaxSlotsPT];
-  __shared__ unsigned long long thr[kMaxSlotsPT][9];
   __shared__ uint4 rnd[kBlock4];   // per warp: [slot in group][quad][replica]
   const uint32_t bid = blockIdx.x;
   const uint32_t set = p.fd_bps.div(bid);   // (b, q)
@@ -430,12 +430,6 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
     Jyp = Jb[2 * i2 + 1];
     Jym = Jb[2 * iym + 1];
   }
-  // the slots' threshold constants through shared memory, so that the
-  // accept flags take them from ordinary registers: measured 6 fewer
-  // logic-pipe and 9 more multiply-add-pipe instructions per word, 2.1% off
-  // the L=16, L_tau=256 sweep (the replica-quad red and the blue kernels,
-  // which would hold them across their sites, lost by it)
-  for (int i = threadIdx.x; i < n * 9; i += blockDim.x) thr[i / 9][i % 9] = th.v[i / 9][i % 9];
   // what came so far depends on no other kernel of the sweep
   pdl_begin();
   {
@@ -490,7 +484,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
       for (int k = 0; k < 7; ++k) fw[k] = cw[k];
     }
     const uint32_t R = rw[((i * 8 + ql) << 2) + j];
-    const unsigned long long *C = thr[sl];
+    const uint32_t *T = th.v[sl];
     const uint32_t sc = fw[0];
     const uint32_t b1 = sc ^ fw[3] ^ Jxp;
     const uint32_t b2 = sc ^ fw[4] ^ Jxm;
@@ -504,7 +498,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
     const uint32_t c2 = s1 & b4;
     const uint32_t us1 = c1 ^ c2;
     const uint32_t us2 = c1 & c2;
-    const uint32_t acc = accept_mask(R, C, us0, us1, us2, t1 | t2, t1 & t2, p.one);
+    const uint32_t acc = accept_word<uint32_t>(R, T, us0, us1, us2, t1 ^ t2, t1 & t2, p.one);
     *addr_mad(pd, zo[0], four) = sc ^ acc;
     *addr_mad(pd, zo[1], four) = fw[1];
     ps2 += SS;
@@ -589,7 +583,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
           for (int k = 0; k < 7; ++k) fw[k] = cw[k];
         }
         const uint32_t R = rw[((i * 8 + ql) << 2) + j];
-        const unsigned long long *C = thr[sl];
+        const uint32_t *T = th.v[sl];
         const uint32_t sc = fw[0];
         const uint32_t b1 = sc ^ fw[3] ^ Jxp;
         const uint32_t b2 = sc ^ fw[4] ^ Jxm;
@@ -603,7 +597,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
         const uint32_t c2 = s1 & b4;
         const uint32_t us1 = c1 ^ c2;
         const uint32_t us2 = c1 & c2;
-        const uint32_t acc = accept_mask(R, C, us0, us1, us2, t1 | t2, t1 & t2, p.one);
+        const uint32_t acc = accept_word<uint32_t>(R, T, us0, us1, us2, t1 ^ t2, t1 & t2, p.one);
         uint32_t *pd = db + (int64_t)sl * SS;
         pd[zo[0]] = sc ^ acc;
         pd[zo[1]] = fw[1];
@@ -778,7 +772,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
 #pragma unroll
         for (int jj = 0; jj < RP; ++jj) fw[k][jj] = cw[k][jj];
     }
-    const unsigned long long *C = th.v[sl];
+    const uint32_t *T = th.v[sl];
     Word out[RP];
 #pragma unroll
     for (int jj = 0; jj < RP; ++jj) {
@@ -795,7 +789,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
       const Word c2 = s1 & b4;
       const Word us1 = c1 ^ c2;
       const Word us2 = c1 & c2;
-      out[jj] = sc ^ accept_word<Word>(Rj[jj], C, us0, us1, us2, t1 | t2, t1 & t2, p.one);
+      out[jj] = sc ^ accept_word<Word>(Rj[jj], T, us0, us1, us2, t1 ^ t2, t1 & t2, p.one);
     }
     Word *pd = db + (int64_t)sl * SS;
     st_rp<Word, RP>(addr_scaled(pd, zo[0], wbytes), out);
@@ -915,7 +909,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
   const int q = (int)(set - bs * (uint32_t)p.n_q);
   const uint32_t b = p.fd_ns.div(bs);
   const int s = (int)(bs - b * (uint32_t)p.n_slots);
-  const unsigned long long *C = th.v[s];
+  const uint32_t *T = th.v[s];
   const int L = p.L, plane = p.plane;
   const uint32_t Lt = (uint32_t)p.Lt, P = (uint32_t)plane;
   const uint32_t h = TPQ == 1 ? 0u : threadIdx.x & 1u, col = threadIdx.x / TPQ;
@@ -1061,7 +1055,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
         const uint32_t ut0 = t1 ^ t2;
         const uint32_t ut1 = t1 & t2;
         const uint32_t nz = t1 | t2;
-        const uint32_t flip = count_only ? 0u : accept_mask(R[j], C, us0, us1, us2, nz, ut1, p.one);
+        const uint32_t flip = count_only ? 0u : accept_word<uint32_t>(R[j], T, us0, us1, us2, ut0, ut1, p.one);
         f[j] = flip;
         // unsatisfied counts after the flip: u -> 4 - u (spatial), 2 - u (tau)
         const uint32_t vs1 = us1 ^ (flip & us0);
@@ -1750,17 +1744,12 @@ void launch_sweep_g(bool pdl, const SamplesArgs<uint32_t> &p, const SlotThreshol
   }
 }
 
-// The 9 classes' accept constants C = 2^64 - T' of every slot, in the form
-// accept_flag reads them (T' = T, or 2^32 for the always-accept sentinel).
+// The thresholds of the nine classes of every slot, in the order of SlotThresholds.
 void fill_thresholds(const qisg_handle *h, SlotThresholds &th) {
   std::memset(&th, 0, sizeof(th));
   static const int cls[9] = {0, 3, 6, 9, 12, 1, 4, 2, 5};   // us * 3 + ut of the 9 classes
   for (int sl = 0; sl < h->n_slots; ++sl)
-    for (int c = 0; c < 9; ++c) {
-      const uint32_t T = h->T[(size_t)sl * 15 + cls[c]];
-      const unsigned long long Tp = T == 0xFFFFFFFFu ? (1ull << 32) : (unsigned long long)T;
-      th.v[sl][c] = 0ull - Tp;
-    }
+    for (int c = 0; c < 9; ++c) th.v[sl][c] = h->T[(size_t)sl * 15 + cls[c]];
 }
 
 // Blocks per SM the blue kernel's registers are bounded to: MINB when the
