@@ -638,15 +638,14 @@ struct qisg_handle {
   int device = 0;
   int n_sm = 0;
   // SAMPLES sweep schedule per colour (red, blue); none of it changes results.
-  // tile: W = 64 and the W = 32 column walk: site groups of 4 per thread
-  // quad; W = 32 replica-quad kernel: at most this many sites per thread
-  // along tau; W = 32 red pass: threads per site (1: four, 2: two, else
-  // one; by default four for lattices with few sites per launch); 0 =
-  // default.
+  // red tile: threads per site (1: four, 2: two, else one, or two for 64-bit
+  // words; 0: by the number of sites).  blue tile: at most this many sites per
+  // thread along tau (W = 64 and the W = 32 column walk: site groups of 4);
+  // 0 = default.
   // variant (W = 32 blue pass): 0 the replica-quad kernel, 1 the column walk,
   // 2 the replica-quad kernel bounded to four blocks per SM (no prefetch).
-  // The default grid aims at sweep_min_blocks_per_sm blocks of 256 threads
-  // per SM.
+  // The column walk's default grid aims at sweep_min_blocks_per_sm blocks of
+  // 256 threads per SM.
   int sweep_tile[2] = {0, 0};
   int sweep_variant[2] = {0, 0};
   int blue_occ[3][7] = {};   // resident blocks per SM of the blue kernel (W = 32 variant 0 | 2, W = 64; 3 .. 9 counter planes)

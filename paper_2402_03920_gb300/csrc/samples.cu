@@ -1876,9 +1876,8 @@ SamplesArgs<Word> make_args4(qisg_handle *h, SlotThresholds &th, int64_t residen
 }
 
 // Arguments of the fused red pass (and its threads per site, from the red
-// tile: 1 -> four, 2 -> two, else one, 0 -> four for lattices with few sites
-// per launch; 64-bit words: at most two replicas per thread) and its block
-// count.
+// tile: 1 -> four, 2 -> two, else one, 0 -> by the number of sites; 64-bit
+// words: at most two replicas per thread) and its block count.
 template <typename Word>
 int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, int &tpsite, int64_t &blocks) {
   const SamplesArgs<Word> a = make_args<Word>(h, 0);
@@ -1902,10 +1901,18 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
   p.tau_ap = h->tau_ap;
   p.ticket = h->d_bar ? h->d_bar + 2 : nullptr;
   if (h->sweep_tile[0] == 0) {
-    // default: a thread per site and replica unless one thread per site
-    // already gives a few waves of full SMs (2048 threads each)
-    const int64_t site_threads = h->n_b * h->n_q * (int64_t)a.plane * (h->Lt / 2);
-    tpsite = site_threads < (int64_t)4 * 2048 * std::max(1, h->n_sm) ? 4 : 1;
+    // default, by the red sites of the launch (us per sweep with a thread per
+    // replica | pair | quad).  32-bit words: 32768 sites 32.8 | 32.9 | 34.9,
+    // 65536: 55.5 | 53.9 | 51.4, 147456: 114 | 118 | 104, 589824: 435 | 459 |
+    // 392; persistent form: 6480: 23.0 | 24.7 | 30.9, 32768: 48.7 | 47.7 |
+    // 51.3, 147456: 197 | 166 | 199, 589824: 735 | 593 | 641 (its grid is one
+    // wave of 168-register blocks).  64-bit words, replica | pair: 6480: 18.5 |
+    // 18.5, 32768: 50.2 | 48.3, 294912: 408 | 340
+    const int64_t sites = h->n_b * h->n_q * (int64_t)a.plane * (h->Lt / 2);
+    const int64_t sm = std::max(1, h->n_sm);
+    if (sizeof(Word) == 8) tpsite = sites < 128 * sm ? 4 : 2;
+    else if (h->persistent) tpsite = sites < 128 * sm ? 4 : 2;
+    else tpsite = sites < 320 * sm ? 4 : 1;
   } else {
     tpsite = h->sweep_tile[0] == 1 ? 4 : h->sweep_tile[0] == 2 ? 2 : 1;
   }
