@@ -36,6 +36,7 @@ struct SamplesArgs {
   unsigned long long *U;
   const unsigned long long *d_t;
   uint2 key;
+  PhiloxKeys rk;         // its round keys
   int64_t N, half_N;
   int L, Lt, plane, half_plane, n_slots, n_rep, n_q, W;
   int seg_sites;         // G: sites of one colour each quad walks along tau (the most of any thread)
@@ -357,6 +358,7 @@ struct FusedRedArgsT {
   unsigned long long *zero_U;
   int64_t n_zero_U;
   uint2 key;
+  PhiloxKeys rk;         // its round keys
   int64_t N;
   int L, Lt, plane, n_slots, n_q, n_rep, blocks_per_set;
   uint32_t one;
@@ -509,7 +511,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
   // groups of four slots that all have two successors; this thread's Philox
   // call of the group (slot 4 g + j), the next group's call made while this
   // group's slots are updated
-  if (live && 6 <= n) r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)j | ((uint32_t)q << 16), ctr_w), p.key);
+  if (live && 6 <= n) r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)j | ((uint32_t)q << 16), ctr_w), p.rk);
   // the PT masks of the (b, q) set, staged after the first slots' loads and
   // draw are issued, so the two round trips to L2 overlap
   for (int i = threadIdx.x; i < 4 * kMaxSlotsPT; i += blockDim.x) {
@@ -522,7 +524,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
     if (live) *reinterpret_cast<uint4 *>(rw + ((j * 8 + ql) << 2)) = r4;
     __syncwarp();
     if (live && 4 * (g + 1) + j < n)
-      r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)(4 * (g + 1) + j) | ((uint32_t)q << 16), ctr_w), p.key);
+      r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)(4 * (g + 1) + j) | ((uint32_t)q << 16), ctr_w), p.rk);
     if (live) {
 #pragma unroll 2   // two slots' loads in flight: 72 registers, seven blocks per SM
       for (int i = 0; i < 4; ++i) update_slot(i, 4 * g + i, yes, yes);
@@ -534,7 +536,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
   if (n % 4 == 0 && 4 * g < n) {
     if (live) {
       if (g == 0)
-        r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)(4 * g + j) | ((uint32_t)q << 16), ctr_w), p.key);
+        r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)(4 * g + j) | ((uint32_t)q << 16), ctr_w), p.rk);
       *reinterpret_cast<uint4 *>(rw + ((j * 8 + ql) << 2)) = r4;
     }
     __syncwarp();
@@ -552,7 +554,7 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
   for (bool made = g > 0; 4 * g < n; ++g, made = false) {
     if (live && 4 * g + j < n) {
       if (!made)
-        r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)(4 * g + j) | ((uint32_t)q << 16), ctr_w), p.key);
+        r4 = philox(make_uint4(z[0], (uint32_t)t, (uint32_t)(4 * g + j) | ((uint32_t)q << 16), ctr_w), p.rk);
       *reinterpret_cast<uint4 *>(rw + ((j * 8 + ql) << 2)) = r4;
     }
     __syncwarp();
@@ -613,16 +615,16 @@ __global__ void __launch_bounds__(kBlock4, 7) samples_red_fused_kernel(const Fus
 // shuffle: the even thread draws even slots, the odd thread odd ones).
 // Fewer threads and instructions per word than the per-replica form; the
 // autotuner picks the form (results are identical).
-template <typename Word, int RP, bool CG = false>
+template <typename Word, int RP>
 __device__ __forceinline__ void ld_rp(Word (&d)[RP], const Word *p) {
   if constexpr (RP * sizeof(Word) == 16) {
-    const uint4 v = ld_g<CG>(reinterpret_cast<const uint4 *>(p));
+    const uint4 v = *reinterpret_cast<const uint4 *>(p);
     memcpy(d, &v, 16);
   } else if constexpr (RP * sizeof(Word) == 8) {
-    const uint2 v = ld_g<CG>(reinterpret_cast<const uint2 *>(p));
+    const uint2 v = *reinterpret_cast<const uint2 *>(p);
     memcpy(d, &v, 8);
   } else {
-    d[0] = ld_g<CG>(p);
+    d[0] = *p;
   }
 }
 template <typename Word, int RP>
@@ -645,9 +647,8 @@ __device__ __forceinline__ void st_rp(Word *p, const Word (&d)[RP]) {
 // per site, consecutive lanes).  The site's Philox calls (one per slot, four
 // draws) are spread over its threads: thread h makes the call of slot
 // TPS g + h and the draws are passed on by shuffles.
-// Body of the pass for (virtual) block bid of sweep t; CG: read what other
-// blocks of a persistent launch wrote (spins, masks) through L2 only.
-template <typename Word, int RP, bool CG>
+// Body of the pass for (virtual) block bid of sweep t.
+template <typename Word, int RP>
 __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, const SlotThresholds &th, uint32_t bid,
                                                 unsigned long long t) {
   constexpr int TPS = 4 / RP;
@@ -703,17 +704,17 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
     Jyp = Jb[2 * i2 + 1];
     Jym = Jb[2 * iym + 1];
 #pragma unroll
-    for (int k = 0; k < 7; ++k) ld_rp<Word, RP, CG>(cw[k], sb + zo[k]);
+    for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(cw[k], sb + zo[k]);
     if (n > 1)
 #pragma unroll
-      for (int k = 0; k < 7; ++k) ld_rp<Word, RP, CG>(n1[k], sb + SS + zo[k]);
+      for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n1[k], sb + SS + zo[k]);
   }
   // the PT masks of the (b, q) set, staged after the first slots' loads are
   // issued, so the two round trips to L2 overlap
   for (int i = threadIdx.x; i < 4 * kMaxSlotsPT; i += blockDim.x) {
     const int sl = i >> 2, jj = i & 3;
     const int rr = 4 * q + jj;
-    msk[sl][jj] = (rr < p.n_rep && sl + 1 < n) ? ld_g<CG>(p.acc + ((int64_t)b * p.n_rep + rr) * n + sl) : Word(0);
+    msk[sl][jj] = (rr < p.n_rep && sl + 1 < n) ? p.acc[((int64_t)b * p.n_rep + rr) * n + sl] : Word(0);
   }
   __syncthreads();
   uint4 R4 = make_uint4(0, 0, 0, 0);
@@ -726,7 +727,13 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
     const int i = sl % TPS;   // thread i of the site holds slot sl's call
     if (i == 0) {
       const int sm = sl + h;
-      if (live && sm < n) R4 = philox(make_uint4(site, (uint32_t)t, (uint32_t)sm | ((uint32_t)q << 16), ctr_w), p.key);
+      if (live && sm < n) {
+        const uint4 ctr = make_uint4(site, (uint32_t)t, (uint32_t)sm | ((uint32_t)q << 16), ctr_w);
+        // round keys as operands cost the 16-byte forms registers (24 bytes of
+        // spills, 1% off the passes' gain)
+        if constexpr (RP * sizeof(Word) == 16) R4 = philox(ctr, p.key);
+        else R4 = philox(ctr, p.rk);
+      }
     }
     uint32_t Rj[RP];
     if constexpr (TPS == 1) {
@@ -753,7 +760,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
       if constexpr (H2) {
         const Word *ps = sb + (int64_t)(sl + 2) * SS;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) ld_rp<Word, RP, CG>(n2[k], addr_scaled(ps, zo[k], wbytes));
+        for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n2[k], addr_scaled(ps, zo[k], wbytes));
       }
       Word m[RP];
 #pragma unroll
@@ -803,8 +810,11 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
   if (sl < n) step(sl, no, no);
 }
 
+// 16-byte forms bounded to four blocks per SM (three where the registers are
+// left free: 122.5 against 114.9 ms for 20 sweeps of 1024 samples at L = 24,
+// L_tau = 512).
 template <typename Word, int RP>
-__global__ void __launch_bounds__(kBlock4) samples_red_fusedq_kernel(const FusedRedArgsT<Word> p,
+__global__ void __launch_bounds__(kBlock4, RP * sizeof(Word) == 16 ? 4 : 0) samples_red_fusedq_kernel(const FusedRedArgsT<Word> p,
                                                                       const __grid_constant__ SlotThresholds th) {
   pdl_begin();
   {
@@ -812,7 +822,7 @@ __global__ void __launch_bounds__(kBlock4) samples_red_fusedq_kernel(const Fused
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_U; i += stride) p.zero_U[i] = 0;
     if (p.ticket && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0u;
   }
-  red_fusedq_body<Word, RP, false>(p, th, blockIdx.x, *p.d_t);
+  red_fusedq_body<Word, RP>(p, th, blockIdx.x, *p.d_t);
 }
 
 // ---- per-lane sums of the block's bit-sliced counters ----
@@ -885,8 +895,8 @@ __device__ __forceinline__ void planes_lane_sums(const uint32_t *buf, int pr, in
   }
 }
 
-// Body of the blue pass for (virtual) block bid of sweep t; CG: read the
-// spins through L2 only (a persistent launch, where other blocks wrote them).
+// Body of the blue pass for (virtual) block bid of sweep t; LOOP: one of
+// several virtual blocks of a persistent launch.
 // A thread holds 16 bytes of a site: the four replicas' words (W = 32) or two
 // replicas' words (W = 64: TPQ = 2 threads per site, thread h with replicas
 // 2 h and 2 h + 1), four 32-bit words w in any case; word w has the draw of
@@ -895,7 +905,7 @@ __device__ __forceinline__ void planes_lane_sums(const uint32_t *buf, int pr, in
 // counter_planes(G)); the u_t sum (at most 2 G) takes one plane less.
 // begin() returns the sweep t; what comes before it depends on no other kernel
 // of the sweep.
-template <typename Word, int KS, bool PF, bool CG, typename Begin>
+template <typename Word, int KS, bool PF, bool LOOP, typename Begin>
 __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const SlotThresholds &th, uint32_t bid,
                                             Begin begin, int count_only) {
   constexpr int KT = KS - 1, TPQ = (int)sizeof(Word) / 4;
@@ -970,7 +980,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
     const uint32_t PS = P * TPQ;   // 16-byte words per plane
     uint32_t off = tau0 * PS;      // of the current site's plane
     const uint32_t anti = ones_if<uint32_t>(p.tau_ap);   // the antiperiodic wrap bond is unsatisfied when its spins agree
-    uint4 dn = ld_g<CG>(pc + (size_t)(tau0 == 0 ? (Lt - 1) * PS : off - PS));
+    uint4 dn = *(pc + (size_t)(tau0 == 0 ? (Lt - 1) * PS : off - PS));
     if (tau0 == 0) {
       dn.x ^= anti;
       dn.y ^= anti;
@@ -978,18 +988,18 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
       dn.w ^= anti;
     }
     Quad4 cur;
-    cur.c = ld_g<CG>(pc + off);
-    cur.up = ld_g<CG>(pc + (size_t)(tau0 + 1 == Lt ? 0u : off + PS));
-    cur.xp = ld_g<CG>(pxp + off);
-    cur.xm = ld_g<CG>(pxm + off);
-    cur.yp = ld_g<CG>(pyp + off);
-    cur.ym = ld_g<CG>(pym + off);
+    cur.c = *(pc + off);
+    cur.up = *(pc + (size_t)(tau0 + 1 == Lt ? 0u : off + PS));
+    cur.xp = *(pxp + off);
+    cur.xm = *(pxm + off);
+    cur.yp = *(pyp + off);
+    cur.ym = *(pym + off);
     // the draws of a site: one Philox call.  W = 64: two sites' calls are
     // made by the two threads of the site, thread h the one of site k + h (k
     // even), and each passes the other the two draws it needs
     uint32_t zsite = (uint32_t)i2 + tau0 * P + (TPQ == 1 ? 0u : h * 2 * P);   // of the next call
     auto call = [&]() {
-      const uint4 v = philox(make_uint4(zsite, (uint32_t)t, ctr_z, ctr_w), p.key);
+      const uint4 v = philox(make_uint4(zsite, (uint32_t)t, ctr_z, ctr_w), p.rk);
       zsite += 2 * P * TPQ;
       return v;
     };
@@ -1027,12 +1037,12 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
       }
       auto load_next = [&](Quad4 &q) {
         const uint32_t offn = off + 2 * PS;
-        q.c = ld_g<CG>(pc + offn);
-        q.up = ld_g<CG>(pc + (size_t)(tau + 3 == Lt ? 0u : offn + PS));
-        q.xp = ld_g<CG>(pxp + offn);
-        q.xm = ld_g<CG>(pxm + offn);
-        q.yp = ld_g<CG>(pyp + offn);
-        q.ym = ld_g<CG>(pym + offn);
+        q.c = *(pc + offn);
+        q.up = *(pc + (size_t)(tau + 3 == Lt ? 0u : offn + PS));
+        q.xp = *(pxp + offn);
+        q.xm = *(pxm + offn);
+        q.yp = *(pyp + offn);
+        q.ym = *(pym + offn);
       };
       if (PF && k + 1 < G) load_next(nx);
       const uint32_t gtp = tau + 1 == Lt ? anti : 0u;
@@ -1084,7 +1094,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
     using Hold = std::integral_constant<int, 0>;
     using Pair = std::integral_constant<int, 1>;
     using One = std::integral_constant<int, 2>;
-    if constexpr (PF && !CG) {
+    if constexpr (PF && !LOOP) {
       // two sites per iteration: the current and next sites' words swap
       // registers instead of being copied, and their counts enter the
       // counters together (not in the persistent kernel, whose register
@@ -1109,7 +1119,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
     }
   }
 
-  if (CG) __syncthreads();   // the previous virtual block's sums are read
+  if (LOOP) __syncthreads();   // the previous virtual block's sums are read
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
 #pragma unroll
@@ -1602,7 +1612,10 @@ __global__ void samples_pack_kernel(Word *spins, const int8_t *stage, const int3
 // warp per chain, accepted pairs OR-ed into the masks the next red pass
 // applies), a barrier.  Blocks take the passes' blocks in turn (block b does
 // b, b + grid, ...), so a pass's work split is the one its own kernel has;
-// anything another block wrote earlier in the launch is read through L2.
+// what another block wrote in an earlier phase is read after a grid barrier,
+// whose release and acquire fences order the phases' plain accesses, so the
+// neighbour loads hit L1 (through L2 only: 46.2 against 44.5 ms for 20 sweeps of
+// 256 samples at L = 24, L_tau = 512).
 // The barriers' waits are bounded (error flag -> QISG_ETIMEOUT).
 struct PersistArgs {
   FusedRedArgsT<uint32_t> red;    // src/dst set per sweep from buf
@@ -1642,7 +1655,7 @@ __global__ void __launch_bounds__(kBlock4, 3) samples_persistent_kernel(const Pe
     rp.src = a.buf[cur];
     rp.dst = a.buf[cur ^ 1];
     for (int64_t i = gtid; i < a.n_U; i += gstride) a.U[i] = 0;
-    for (int vb = blockIdx.x; vb < a.red_blocks; vb += gridDim.x) red_fusedq_body<uint32_t, RP, true>(rp, th, vb, t);
+    for (int vb = blockIdx.x; vb < a.red_blocks; vb += gridDim.x) red_fusedq_body<uint32_t, RP>(rp, th, vb, t);
     if (!grid_barrier(a.bar, a.err, a.wait_ns)) return;
     for (int64_t i = gtid; i < a.n_acc; i += gstride) a.acc[i] = 0;
     SamplesArgs<uint32_t> bp = a.blue;
@@ -1672,6 +1685,7 @@ SamplesArgs<Word> make_args(qisg_handle *h, int colour) {
   p.U = h->d_U;
   p.d_t = h->d_t;
   p.key = make_uint2((uint32_t)h->seed, (uint32_t)(h->seed >> 32));
+  p.rk = PhiloxKeys(p.key);
   p.N = h->N;
   p.half_N = h->N / 2;
   p.L = h->L;
@@ -1890,6 +1904,7 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
   p.zero_U = h->d_U;
   p.n_zero_U = h->n_a_pad * h->n_rep * h->n_slots * 2;
   p.key = a.key;
+  p.rk = a.rk;
   p.N = h->N;
   p.L = h->L;
   p.Lt = h->Lt;
@@ -2315,6 +2330,14 @@ int set_couplings_t(qisg_handle *h, const int8_t *J) {
 int samples_init(qisg_handle *h) {
   if (h->n_slots > kMaxSlotsPermute) return fail(QISG_EINVAL, "SAMPLES packing supports up to 32 slots");
   if (h->L > 1024) return fail(QISG_EINVAL, "SAMPLES packing supports L <= 1024");
+  // accept_word relies on thresholds that do not decrease with u_s (k >= 0
+  // makes the exponents so, and exp keeps their order)
+  for (int sl = 0; sl < h->n_slots; ++sl)
+    for (int us = 0; us < 4; ++us)
+      for (int ut = 0; ut < 3; ++ut) {
+        const uint32_t *T = &h->T[(size_t)sl * 15 + ut];
+        if (T[us * 3] > T[us * 3 + 3]) return fail(QISG_EINVAL, "thresholds are not ordered by u_s");
+      }
   return h->W == 64 ? init_t<unsigned long long>(h) : init_t<unsigned int>(h);
 }
 int samples_materialize(qisg_handle *h) {
