@@ -311,18 +311,35 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
   }
 }
 
-// ---- W = 32: one thread per (column segment, 4 replicas) ----
+// ---- one thread per (column segment, 16 bytes of replica words) ----
 //
-// The 4 replica words of a site are adjacent ([site][4] x 32 bits), so one
-// 16-byte load brings a site's replica quad and one Philox call gives the
-// quad's four draws.  A thread walks G sites of the colour along tau in one
-// (x, y) column, loading the next site while it updates the current one
-// (the steps touch disjoint words: centres of this colour, neighbours of the
-// other).  The 9 thresholds that can reject come from the parameter bank,
-// uniform over the block.  In the blue pass each thread keeps bit-sliced
-// counters per replica; the block then sums them with a tree in shared
-// memory (vertical adds, 32 lanes per operation) instead of warp shuffles.
+// The 4 replica words of a site are adjacent ([site][4]): 16 bytes hold the
+// quad of 32-bit words, or two replicas of 64-bit ones, and one Philox call
+// gives the quad's four draws.  A thread walks G sites of the colour along tau
+// in one (x, y) column, the next site's words on their way to shared memory
+// while it updates the current one (the steps touch disjoint words: centres of
+// this colour, neighbours of the other).  The nine thresholds that can reject
+// come from the parameter bank, uniform over the block.  Each thread keeps
+// bit-sliced counters per word; the block then sums them (below).
+//
+// What bounds it: the latency of the instruction chains at three blocks (12
+// warps) per SM, the registers being the counters', the held counts' and the
+// words'; the logic pipe is 70% busy.  1024 samples at L = 24, L_tau = 512: the
+// next site's words in shared memory instead of registers took 20 sweeps from
+// 116.3 to 109.3 ms; four blocks per SM spill (113 ms), two stages ahead gain
+// nothing more.
 constexpr int kBlock4 = 128;
+
+// Asynchronous 16-byte copies of this thread from global to shared memory.
+__device__ __forceinline__ void async_copy16(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void async_wait() {   // all but the last N groups are complete
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 
 struct Quad4 {
   uint4 c, up, xp, xm, yp, ym;
@@ -910,7 +927,11 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
                                             Begin begin, int count_only) {
   constexpr int KT = KS - 1, TPQ = (int)sizeof(Word) / 4;
   constexpr uint32_t kCols = kBlock4 / TPQ;   // columns per block
-  __shared__ uint32_t buf[4 * (KS + KT) * kBlock4];   // u_s counters, then u_t
+  constexpr bool SPF = PF && !LOOP;   // the walk's words are staged in shared memory
+  // staged words (two sites of 24 words of 4 bytes per thread), then the counters
+  // (u_s, then u_t)
+  constexpr int kBuf = SPF && 48 > 4 * (KS + KT) ? 48 : 4 * (KS + KT);
+  __shared__ __align__(16) uint32_t buf[kBuf * kBlock4];
 
   // block -> (b, s, q, chunk) and thread -> (segment, column) in 32 bits
   const uint32_t set = p.fd_bps.div(bid);
@@ -988,12 +1009,14 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
       dn.w ^= anti;
     }
     Quad4 cur;
-    cur.c = *(pc + off);
-    cur.up = *(pc + (size_t)(tau0 + 1 == Lt ? 0u : off + PS));
-    cur.xp = *(pxp + off);
-    cur.xm = *(pxm + off);
-    cur.yp = *(pyp + off);
-    cur.ym = *(pym + off);
+    if constexpr (!SPF) {
+      cur.c = *(pc + off);
+      cur.up = *(pc + (size_t)(tau0 + 1 == Lt ? 0u : off + PS));
+      cur.xp = *(pxp + off);
+      cur.xm = *(pxm + off);
+      cur.yp = *(pyp + off);
+      cur.ym = *(pym + off);
+    }
     // the draws of a site: one Philox call.  W = 64: two sites' calls are
     // made by the two threads of the site, thread h the one of site k + h (k
     // even), and each passes the other the two draws it needs
@@ -1008,9 +1031,10 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
     // the even site's post-flip counts, held until the odd site's are added
     // with them (the prefetching walk of the per-pass launch)
     uint32_t h0[4], h1[4], h2[4], g0[4], g1[4];
-    // site k of the walk, its words in cu; with the prefetch the next site's
-    // words go to nx while this one is updated, else to cu after it.  PH: 0
-    // hold this site's counts, 1 add them with the held ones, 2 add them
+    // site k of the walk, its words in cu; the next site's words come through
+    // shared memory (SPF), go to nx while this one is updated (the persistent
+    // kernel) or to cu after it.  PH: 0 hold this site's counts, 1 add them
+    // with the held ones, 2 add them
     auto site = [&](int k, Quad4 &cu, Quad4 &nx, auto phase) {
       constexpr int PH = decltype(phase)::value;
       const uint32_t tau = tau0 + 2u * (uint32_t)k;
@@ -1044,7 +1068,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
         q.yp = *(pyp + offn);
         q.ym = *(pym + offn);
       };
-      if (PF && k + 1 < G) load_next(nx);
+      if (PF && LOOP && k + 1 < G) load_next(nx);
       const uint32_t gtp = tau + 1 == Lt ? anti : 0u;
       uint32_t f[4];
 #pragma unroll
@@ -1094,18 +1118,47 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
     using Hold = std::integral_constant<int, 0>;
     using Pair = std::integral_constant<int, 1>;
     using One = std::integral_constant<int, 2>;
-    if constexpr (PF && !LOOP) {
-      // two sites per iteration: the current and next sites' words swap
-      // registers instead of being copied, and their counts enter the
-      // counters together (not in the persistent kernel, whose register
-      // bound would make this walk spill)
-      Quad4 nxt;
+    if constexpr (SPF) {
+      // the next site's words are copied to shared memory while this one is
+      // updated: the copies in flight hold no registers (24 of the prefetch in
+      // registers).  Two sites per iteration: their counts enter the counters
+      // together (not in the persistent kernel, whose register bound would make
+      // this walk spill)
+      uint4 *ring = reinterpret_cast<uint4 *>(buf) + threadIdx.x;   // [2][6][thread]
+      auto copy_in = [&](int st, uint32_t o, bool wrap) {
+        const uint4 *g[6] = {pc + o, pc + (size_t)(wrap ? 0u : o + PS), pxp + o, pxm + o, pyp + o, pym + o};
+#pragma unroll
+        for (int m = 0; m < 6; ++m) async_copy16(ring + (st * 6 + m) * kBlock4, g[m]);
+        async_commit();
+      };
+      auto fetch = [&](int k) {
+        if (k + 1 < G) {
+          copy_in((k + 1) & 1, off + 2 * PS, tau0 + 2u * (uint32_t)k + 3 == Lt);
+          async_wait<1>();   // site k's words are here
+        } else {
+          async_wait<0>();
+        }
+        const uint4 *r = ring + (k & 1) * 6 * kBlock4;
+        cur.c = r[0];
+        cur.up = r[kBlock4];
+        cur.xp = r[2 * kBlock4];
+        cur.xm = r[3 * kBlock4];
+        cur.yp = r[4 * kBlock4];
+        cur.ym = r[5 * kBlock4];
+      };
+      copy_in(0, off, tau0 + 1 == Lt);
       int k = 0;
+#pragma unroll 1
       for (; k + 1 < G; k += 2) {
-        site(k, cur, nxt, Hold{});
-        site(k + 1, nxt, cur, Pair{});
+        fetch(k);
+        site(k, cur, cur, Hold{});
+        fetch(k + 1);
+        site(k + 1, cur, cur, Pair{});
       }
-      if (k < G) site(k, cur, nxt, One{});
+      if (k < G) {
+        fetch(k);
+        site(k, cur, cur, One{});
+      }
     } else if constexpr (PF) {
       Quad4 nxt;
 #pragma unroll 1
@@ -1119,7 +1172,7 @@ __device__ __forceinline__ void sweep4_body(const SamplesArgs<Word> &p, const Sl
     }
   }
 
-  if (LOOP) __syncthreads();   // the previous virtual block's sums are read
+  __syncthreads();   // the staged words, or the previous virtual block's sums, are read
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
 #pragma unroll
@@ -1772,7 +1825,7 @@ void fill_thresholds(const qisg_handle *h, SlotThresholds &th) {
 // blocks), none beyond (the bound would spill).
 template <bool PF, int MINB, int KS>
 constexpr int blue_min_blocks() {
-  return MINB > 0 ? MINB : (PF && KS <= 7) ? 3 : 0;
+  return MINB > 0 ? MINB : (PF && KS <= 7) ? (3) : 0;
 }
 
 // The blue kernel for ks = 3 .. 9 counter planes (variant 0 or 2; 64-bit words
