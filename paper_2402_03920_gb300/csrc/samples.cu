@@ -330,17 +330,6 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
 // nothing more.
 constexpr int kBlock4 = 128;
 
-// Asynchronous 16-byte copies of this thread from global to shared memory.
-__device__ __forceinline__ void async_copy16(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void async_wait() {   // all but the last N groups are complete
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 struct Quad4 {
   uint4 c, up, xp, xm, yp, ym;
 };
@@ -659,15 +648,29 @@ __device__ __forceinline__ void st_rp(Word *p, const Word (&d)[RP]) {
   }
 }
 
+// Asynchronous 16-byte copies of this thread from global to shared memory.
+__device__ __forceinline__ void async_copy16(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void async_wait() {   // all but the last N groups are complete
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Red pass with the pending PT exchanges (as above) for either word width,
 // one thread per red site and RP of its four replicas (TPS = 4 / RP threads
 // per site, consecutive lanes).  The site's Philox calls (one per slot, four
 // draws) are spread over its threads: thread h makes the call of slot
 // TPS g + h and the draws are passed on by shuffles.
-// Body of the pass for (virtual) block bid of sweep t.
-template <typename Word, int RP>
+// Body of the pass for (virtual) block bid of sweep t.  NS > 0 (16 bytes per
+// thread and site): the words of the next NS slots are copied to shared memory
+// (ring, [NS][7][kBlock4]) while a slot is updated, so the copies in flight
+// hold no registers; else the next two slots' words are held.
+template <typename Word, int RP, int NS>
 __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, const SlotThresholds &th, uint32_t bid,
-                                                unsigned long long t) {
+                                                unsigned long long t, uint4 *ring) {
   constexpr int TPS = 4 / RP;
   constexpr int W = (int)sizeof(Word) * 8;
   __shared__ __align__(16) Word msk[kMaxSlotsPT][4];
@@ -715,6 +718,18 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
   const uint32_t site = i2 + off;
   const int lane = (int)(threadIdx.x & 31), lane0 = lane & ~(TPS - 1);
   Word cw[7][RP], n1[7][RP];
+  static_assert(NS == 0 || RP * sizeof(Word) == 16, "the ring holds 16-byte words");
+  [[maybe_unused]] uint4 *rg = NS ? ring + threadIdx.x : nullptr;
+  [[maybe_unused]] auto copy_in = [&](int slot) {
+    if constexpr (NS > 0) {
+      if (live && slot < n) {
+        const Word *ps = sb + (int64_t)slot * SS;
+#pragma unroll
+        for (int k = 0; k < 7; ++k) async_copy16(rg + ((slot % NS) * 7 + k) * kBlock4, ps + zo[k]);
+      }
+      async_commit();   // a group per slot, empty past the ladder
+    }
+  };
   if (live) {
     Jxp = Jb[2 * i2];
     Jxm = Jb[2 * ixm];
@@ -722,10 +737,12 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
     Jym = Jb[2 * iym + 1];
 #pragma unroll
     for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(cw[k], sb + zo[k]);
-    if (n > 1)
+    if (NS == 0 && n > 1)
 #pragma unroll
       for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n1[k], sb + SS + zo[k]);
   }
+#pragma unroll
+  for (int k = 1; k < NS; ++k) copy_in(k);
   // the PT masks of the (b, q) set, staged after the first slots' loads are
   // issued, so the two round trips to L2 overlap
   for (int i = threadIdx.x; i < 4 * kMaxSlotsPT; i += blockDim.x) {
@@ -774,7 +791,16 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
     Word fw[7][RP];
     if constexpr (H1) {
       Word n2[7][RP];
-      if constexpr (H2) {
+      if constexpr (NS > 0) {
+        copy_in(sl + NS);
+        async_wait<NS - 1>();   // slot sl + 1 is complete
+        const uint4 *r = rg + ((sl + 1) % NS) * 7 * kBlock4;
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+          const uint4 v = r[k * kBlock4];
+          memcpy(n1[k], &v, 16);
+        }
+      } else if constexpr (H2) {
         const Word *ps = sb + (int64_t)(sl + 2) * SS;
 #pragma unroll
         for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n2[k], addr_scaled(ps, zo[k], wbytes));
@@ -788,7 +814,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
         for (int jj = 0; jj < RP; ++jj) {   // lanes of m exchange pair (sl, sl + 1)
           fw[k][jj] = mux(m[jj], n1[k][jj], cw[k][jj]);
           cw[k][jj] = mux(m[jj], cw[k][jj], n1[k][jj]);
-          if constexpr (H2) n1[k][jj] = n2[k][jj];
+          if constexpr (H2 && NS == 0) n1[k][jj] = n2[k][jj];
         }
     } else {
 #pragma unroll
@@ -827,19 +853,24 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
   if (sl < n) step(sl, no, no);
 }
 
-// 16-byte forms bounded to four blocks per SM (three where the registers are
-// left free: 122.5 against 114.9 ms for 20 sweeps of 1024 samples at L = 24,
-// L_tau = 512).
+// Slots staged ahead by the 16-byte forms (the quads of 32-bit words, the
+// pairs of 64-bit ones), and their bound of blocks per SM.  They waited on
+// their neighbour loads (3.2 to 3.5 warps per issue on the long scoreboard)
+// with two slots' words in 56 registers; 1024 samples at L = 24, L_tau = 512,
+// 20 sweeps: 109.3 -> 100.8 ms (three stages 104, five blocks 102 to 116: the
+// stages take the room of L1).
+constexpr int kRedStages = 2, kRedBlocks = 4;
 template <typename Word, int RP>
-__global__ void __launch_bounds__(kBlock4, RP * sizeof(Word) == 16 ? 4 : 0) samples_red_fusedq_kernel(const FusedRedArgsT<Word> p,
-                                                                      const __grid_constant__ SlotThresholds th) {
+__global__ void __launch_bounds__(kBlock4, RP * sizeof(Word) == 16 ? kRedBlocks : 0)
+    samples_red_fusedq_kernel(const FusedRedArgsT<Word> p, const __grid_constant__ SlotThresholds th) {
+  extern __shared__ uint4 ring[];
   pdl_begin();
   {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < p.n_zero_U; i += stride) p.zero_U[i] = 0;
     if (p.ticket && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0u;
   }
-  red_fusedq_body<Word, RP>(p, th, blockIdx.x, *p.d_t);
+  red_fusedq_body<Word, RP, RP * sizeof(Word) == 16 ? kRedStages : 0>(p, th, blockIdx.x, *p.d_t, ring);
 }
 
 // ---- per-lane sums of the block's bit-sliced counters ----
@@ -1708,7 +1739,7 @@ __global__ void __launch_bounds__(kBlock4, 3) samples_persistent_kernel(const Pe
     rp.src = a.buf[cur];
     rp.dst = a.buf[cur ^ 1];
     for (int64_t i = gtid; i < a.n_U; i += gstride) a.U[i] = 0;
-    for (int vb = blockIdx.x; vb < a.red_blocks; vb += gridDim.x) red_fusedq_body<uint32_t, RP>(rp, th, vb, t);
+    for (int vb = blockIdx.x; vb < a.red_blocks; vb += gridDim.x) red_fusedq_body<uint32_t, RP, 0>(rp, th, vb, t, nullptr);
     if (!grid_barrier(a.bar, a.err, a.wait_ns)) return;
     for (int64_t i = gtid; i < a.n_acc; i += gstride) a.acc[i] = 0;
     SamplesArgs<uint32_t> bp = a.blue;
@@ -1970,12 +2001,12 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
   p.ticket = h->d_bar ? h->d_bar + 2 : nullptr;
   if (h->sweep_tile[0] == 0) {
     // default, by the red sites of the launch (us per sweep with a thread per
-    // replica | pair | quad).  32-bit words: 32768 sites 32.8 | 32.9 | 34.9,
-    // 65536: 55.5 | 53.9 | 51.4, 147456: 114 | 118 | 104, 589824: 435 | 459 |
-    // 392; persistent form: 6480: 23.0 | 24.7 | 30.9, 32768: 48.7 | 47.7 |
-    // 51.3, 147456: 197 | 166 | 199, 589824: 735 | 593 | 641 (its grid is one
+    // replica | pair | quad).  32-bit words: 32768 sites 32.6 | 32.9 | 32.8,
+    // 65536: 54.4 | 51.8 | 49.3, 147456: 112 | 110 | 97, 589824: 426 | 414 |
+    // 364; persistent form: 6480: 22.8 | 24.6 | 30.4, 32768: 47.6 | 46.5 |
+    // 49.0, 147456: 187 | 158 | 182, 589824: 725 | 567 | 604 (its grid is one
     // wave of 168-register blocks).  64-bit words, replica | pair: 6480: 18.5 |
-    // 18.5, 32768: 50.2 | 48.3, 294912: 408 | 340
+    // 17.8, 32768: 48.2 | 47.2, 294912: 365 | 319
     const int64_t sites = h->n_b * h->n_q * (int64_t)a.plane * (h->Lt / 2);
     const int64_t sm = std::max(1, h->n_sm);
     if (sizeof(Word) == 8) tpsite = sites < 128 * sm ? 4 : 2;
@@ -2005,6 +2036,7 @@ int fused_red(qisg_handle *h) {
   int64_t blocks = 0;
   const int rc = make_red_args<Word>(h, th, p, tpsite, blocks);
   if (rc) return rc;
+  constexpr size_t ring_bytes = (size_t)kRedStages * 7 * kBlock4 * 16;
   const int tok = prof_begin(h, QISG_KERNEL_SWEEP);
   if constexpr (sizeof(Word) == 4) {
     const FusedRedArgs &p32 = p;
@@ -2013,12 +2045,12 @@ int fused_red(qisg_handle *h) {
     else if (tpsite == 2)
       launch_kernel(h->pdl, samples_red_fusedq_kernel<uint32_t, 2>, dim3((unsigned)blocks), dim3(kBlock4), 0, h->stream, p, th);
     else
-      launch_kernel(h->pdl, samples_red_fusedq_kernel<uint32_t, 4>, dim3((unsigned)blocks), dim3(kBlock4), 0, h->stream, p, th);
+      launch_kernel(h->pdl, samples_red_fusedq_kernel<uint32_t, 4>, dim3((unsigned)blocks), dim3(kBlock4), ring_bytes, h->stream, p, th);
   } else {
     if (tpsite == 4)
       launch_kernel(h->pdl, samples_red_fusedq_kernel<Word, 1>, dim3((unsigned)blocks), dim3(kBlock4), 0, h->stream, p, th);
     else
-      launch_kernel(h->pdl, samples_red_fusedq_kernel<Word, 2>, dim3((unsigned)blocks), dim3(kBlock4), 0, h->stream, p, th);
+      launch_kernel(h->pdl, samples_red_fusedq_kernel<Word, 2>, dim3((unsigned)blocks), dim3(kBlock4), ring_bytes, h->stream, p, th);
   }
   prof_end(h, QISG_KERNEL_SWEEP, tok);
   h->launches++;
