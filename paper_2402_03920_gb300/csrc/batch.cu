@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <map>
 #include <vector>
 
@@ -257,6 +258,7 @@ struct qisg_batch {
   int n_chains = 0;
   unsigned *d_bar = nullptr;
   int *d_err = nullptr;
+  unsigned char *pin = nullptr;   // pinned host memory of the read-outs (read_back)
   bool dirty = true;
   int tile_rows = 0;      // rows of 256 sites per tile; 0: chosen for the batch (build_tables)
   int schedule = 0;       // 0: instance order; 1: largest instances first
@@ -465,15 +467,14 @@ int check_desc(const qisg_instance_desc *d) {
   return QISG_OK;
 }
 
-int sync_batch(qisg_batch *B) {
-  int rc = cuda_check(cudaStreamSynchronize(B->stream), "stream synchronize");
-  if (rc) return rc;
+int read_batch(qisg_batch *B, std::initializer_list<ReadBack> c) {
   int err = 0;
-  rc = cuda_check(cudaMemcpy(&err, B->d_err, sizeof(int), cudaMemcpyDeviceToHost), "error flag");
-  if (rc) return rc;
-  if (err) return fail(QISG_ETIMEOUT, "a grid barrier of the batch kernel timed out");
-  return QISG_OK;
+  const int rc = read_back(B->stream, B->pin, B->d_err, c.begin(), (int)c.size(), &err);
+  if (!rc && err) return fail(QISG_ETIMEOUT, "a grid barrier of the batch kernel timed out");
+  return rc;
 }
+
+int sync_batch(qisg_batch *B) { return read_batch(B, {}); }
 
 }  // namespace
 
@@ -499,6 +500,10 @@ int qisg_batch_create(qisg_batch **out, int capacity, size_t mem_budget, void *c
       mem_budget = fr / 2;
     }
     B->budget = mem_budget;
+  }
+  if (!rc && cudaMallocHost((void **)&B->pin, kPinBytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    B->pin = nullptr;   // read-outs then copy straight to host memory
   }
   if (!rc) rc = cuda_check(cudaMalloc(&B->arena, B->budget), "arena");
   if (!rc) rc = cuda_check(cudaMalloc(&B->d_inst, sizeof(InstDev) * (size_t)capacity), "descriptors");
@@ -651,15 +656,12 @@ int qisg_batch_status(qisg_batch *B, int slot, uint64_t *sweeps_done, int *done)
 
 int qisg_batch_results(qisg_batch *B, int slot, int64_t *A, int64_t *Bt, int32_t *walker_at, int8_t *S_out) {
   if (!B || slot < 0 || slot >= B->capacity || !B->slots[slot].used) return fail(QISG_EINVAL, "bad slot");
-  int rc = sync_batch(B);
-  if (rc) return rc;
   const Slot &S = B->slots[slot];
   const InstDev &I = S.dev;
   const int n = I.n_slots, nr = I.n_rep;
   std::vector<int32_t> wa((size_t)nr * n);
   std::vector<unsigned long long> U((size_t)nr * n * 2);
-  rc = cuda_check(cudaMemcpy(wa.data(), I.walker, wa.size() * 4, cudaMemcpyDeviceToHost), "walker");
-  if (!rc) rc = cuda_check(cudaMemcpy(U.data(), I.U, U.size() * 8, cudaMemcpyDeviceToHost), "U");
+  int rc = read_batch(B, {{wa.data(), I.walker, wa.size() * 4}, {U.data(), I.U, U.size() * 8}});
   if (rc) return rc;
   if (walker_at) std::memcpy(walker_at, wa.data(), wa.size() * 4);
   for (int r = 0; r < nr; ++r)
@@ -720,6 +722,7 @@ void qisg_batch_destroy(qisg_batch *B) {
   if (B->d_chains) cudaFree(B->d_chains);
   if (B->d_bar) cudaFree(B->d_bar);
   if (B->d_err) cudaFree(B->d_err);
+  if (B->pin) cudaFreeHost(B->pin);
   delete B;
 }
 

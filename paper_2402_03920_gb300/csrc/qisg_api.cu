@@ -185,20 +185,46 @@ int recompute_energies(qisg_handle *h) {
   return samples_half_sweep(h, 1, 1);
 }
 
-int sync_handle(qisg_handle *h) {
-  int rc = cuda_check(cudaStreamSynchronize(h->stream), "stream synchronize");
-  if (rc) return rc;
-  int err = 0;
-  rc = cuda_check(cudaMemcpy(&err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost), "read error flag");
-  if (rc) return rc;
-  if (err) return fail(QISG_ETIMEOUT, "a bounded device wait expired");
-  return QISG_OK;
-}
+int sync_handle(qisg_handle *h) { return read_back(h, {}); }
 
 }  // namespace
 
 namespace qisg {
 int handle_sync(qisg_handle *h) { return sync_handle(h); }
+
+int read_back(cudaStream_t st, unsigned char *pin, const int *d_err, const ReadBack *c, int n, int *err) {
+  size_t total = 16;
+  for (int i = 0; i < n; ++i) total += (c[i].bytes + 15) & ~size_t(15);
+  const bool staged = pin && total <= kPinBytes;
+  size_t at = 16;
+  int rc = QISG_OK;
+  for (int i = 0; i < n && !rc; ++i) {
+    if (!c[i].bytes) continue;
+    rc = cuda_check(cudaMemcpyAsync(staged ? pin + at : c[i].dst, c[i].src, c[i].bytes, cudaMemcpyDeviceToHost, st), "copy");
+    at += (c[i].bytes + 15) & ~size_t(15);
+  }
+  *err = 0;
+  if (!rc && pin) rc = cuda_check(cudaMemcpyAsync(pin, d_err, sizeof(int), cudaMemcpyDeviceToHost, st), "read error flag");
+  const int rc_sync = cuda_check(cudaStreamSynchronize(st), "stream synchronize");
+  if (!rc) rc = rc_sync;
+  if (!rc && !pin) rc = cuda_check(cudaMemcpy(err, d_err, sizeof(int), cudaMemcpyDeviceToHost), "read error flag");
+  if (rc) return rc;
+  if (pin) std::memcpy(err, pin, sizeof(int));
+  at = 16;
+  for (int i = 0; i < n && staged; ++i) {
+    if (!c[i].bytes) continue;
+    std::memcpy(c[i].dst, pin + at, c[i].bytes);
+    at += (c[i].bytes + 15) & ~size_t(15);
+  }
+  return QISG_OK;
+}
+
+int read_back(qisg_handle *h, std::initializer_list<ReadBack> c) {
+  int err = 0;
+  const int rc = read_back(h->stream, h->pin, h->d_err, c.begin(), (int)c.size(), &err);
+  if (!rc && err) return fail(QISG_ETIMEOUT, "a bounded device wait expired");
+  return rc;
+}
 }  // namespace qisg
 
 extern "C" {
@@ -314,6 +340,10 @@ int qisg_create(qisg_handle **out, int L, int L_tau, const qisg_slot *ladder, in
   build_bases(h);
 
   int rc = cuda_check(cudaGetDevice(&h->device), "cudaGetDevice");
+  if (!rc && cudaMallocHost((void **)&h->pin, kPinBytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    h->pin = nullptr;   // read-outs then copy straight to the caller's memory
+  }
   if (!rc) rc = cuda_check(cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, h->device),
                            "device attribute");
   const int64_t n_chain_slots = h->n_a_pad * n_replicas * n_slots;
@@ -844,11 +874,7 @@ int qisg_energies(qisg_handle *h, int64_t *A, int64_t *B) {
   if (rc) return rc;
   const size_t n = (size_t)h->n_samples * h->n_rep * h->n_slots;
   const size_t stride = (size_t)h->n_a_pad * h->n_rep * h->n_slots;
-  rc = cuda_check(cudaMemcpyAsync(A, h->d_out, n * 8, cudaMemcpyDeviceToHost, h->stream), "copy A");
-  if (!rc) rc = cuda_check(cudaMemcpyAsync(B, h->d_out + stride, n * 8, cudaMemcpyDeviceToHost, h->stream),
-                           "copy B");
-  if (!rc) rc = sync_handle(h);
-  return rc;
+  return read_back(h, {{A, h->d_out, n * 8}, {B, h->d_out + stride, n * 8}});
 }
 
 int qisg_overlaps(qisg_handle *h, int64_t *q) {
@@ -860,20 +886,16 @@ int qisg_overlaps(qisg_handle *h, int64_t *q) {
                                              : samples_measure(h, 1);
   if (rc) return rc;
   const size_t n = (size_t)h->n_samples * h->n_slots * n_pairs;
-  rc = cuda_check(cudaMemcpyAsync(q, h->d_q, n * 8, cudaMemcpyDeviceToHost, h->stream), "copy q");
+  rc = read_back(h, {{q, h->d_q, n * 8}});
   if (!rc) rc = cuda_check(cudaMemsetAsync(h->d_q, 0, (size_t)h->n_a_pad * h->n_slots * n_pairs * 8, h->stream),
                            "memset");
-  if (!rc) rc = sync_handle(h);
   return rc;
 }
 
 int qisg_permutation(qisg_handle *h, int32_t *walker_at) {
   if (!h || !walker_at) return fail(QISG_EINVAL, "NULL argument");
   const size_t n = (size_t)h->n_samples * h->n_rep * h->n_slots;
-  int rc = cuda_check(cudaMemcpyAsync(walker_at, h->d_walker, n * 4, cudaMemcpyDeviceToHost, h->stream),
-                      "copy walker");
-  if (!rc) rc = sync_handle(h);
-  return rc;
+  return read_back(h, {{walker_at, h->d_walker, n * 4}});
 }
 
 int qisg_get_spins(qisg_handle *h, int64_t a_lo, int64_t n_a, int8_t *S) {
@@ -1039,14 +1061,12 @@ int qisg_pt_given(qisg_handle *h, const int64_t *U, int32_t *walker_at, uint64_t
 int qisg_measurements(qisg_handle *h, int64_t *sumA, int64_t *sumB, int64_t *sumq, int64_t *sumq2,
                       int64_t *n_meas) {
   if (!h) return fail(QISG_EINVAL, "NULL handle");
-  int rc = QISG_OK;
   const size_t ncs = (size_t)h->n_samples * h->n_rep * h->n_slots;
   const size_t nq = (size_t)h->n_samples * h->n_slots * h->n_pairs();
-  if (sumA) rc = cuda_check(cudaMemcpyAsync(sumA, h->d_sumA, ncs * 8, cudaMemcpyDeviceToHost, h->stream), "copy");
-  if (!rc && sumB) rc = cuda_check(cudaMemcpyAsync(sumB, h->d_sumB, ncs * 8, cudaMemcpyDeviceToHost, h->stream), "copy");
-  if (!rc && sumq && nq) rc = cuda_check(cudaMemcpyAsync(sumq, h->d_sumq, nq * 8, cudaMemcpyDeviceToHost, h->stream), "copy");
-  if (!rc && sumq2 && nq) rc = cuda_check(cudaMemcpyAsync(sumq2, h->d_sumq2, nq * 8, cudaMemcpyDeviceToHost, h->stream), "copy");
-  if (!rc) rc = sync_handle(h);
+  const int rc = read_back(h, {{sumA, h->d_sumA, sumA ? ncs * 8 : 0},
+                               {sumB, h->d_sumB, sumB ? ncs * 8 : 0},
+                               {sumq, h->d_sumq, sumq ? nq * 8 : 0},
+                               {sumq2, h->d_sumq2, sumq2 ? nq * 8 : 0}});
   if (!rc && n_meas) *n_meas = h->n_meas;
   return rc;
 }
@@ -1155,6 +1175,7 @@ void qisg_destroy(qisg_handle *h) {
   for (void *p : ptrs)
     if (p) cudaFree(p);
   drop_cycle(h);
+  if (h->pin) cudaFreeHost(h->pin);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   for (int b = 0; b < kLanesBranches; ++b) {
     if (h->branch[b]) cudaStreamDestroy(h->branch[b]);

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <map>
 #include <string>
 #include <utility>
@@ -716,6 +717,8 @@ struct qisg_handle {
   unsigned long long *d_dcum = nullptr;   // SITES: cumulative tables [n_slots][256]
   uint32_t *d_dlut = nullptr;             // SITES: prefix index [n_slots][kDaemonLutWords]
   int *d_err = nullptr;
+  // pinned host memory the small read-outs go through (read_back)
+  unsigned char *pin = nullptr;
   // records at every measurement (Appendix A): PT walk history and maxit block sums
   int hist_len = 0, maxit = 0, blk_len = 0;
   unsigned long long *d_meas = nullptr;   // measurements taken (device copy of n_meas)
@@ -800,6 +803,19 @@ int samples_stage_spins(qisg_handle *h, int64_t a_lo, int64_t n_a, int8_t *d);
 // persistent form: n sweeps (red, blue, PT) in one cooperative launch
 bool samples_persistent_ok(const qisg_handle *h);
 int samples_persistent(qisg_handle *h, int n_sweeps);
+
+// Device to host copies of a read-out, with the error flag and one
+// synchronisation of the handle's stream.  Up to kPinBytes in all go through
+// the handle's pinned buffer: a copy to pageable memory waits for the device by
+// itself, about 8 us each.
+constexpr size_t kPinBytes = 256 << 10;
+struct ReadBack {
+  void *dst;
+  const void *src;
+  size_t bytes;
+};
+int read_back(cudaStream_t st, unsigned char *pin, const int *d_err, const ReadBack *c, int n, int *err);
+int read_back(qisg_handle *h, std::initializer_list<ReadBack> c);
 
 // common small kernels (qisg_api.cu)
 int advance_counter(qisg_handle *h);
