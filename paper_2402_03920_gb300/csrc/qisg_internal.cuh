@@ -420,6 +420,13 @@ __device__ __forceinline__ T ld_g(const T *p) {
     return *p;
 }
 
+// v += R < T ? x : 0 by a predicated multiply-add (one is the runtime value 1).
+__device__ __forceinline__ void add_if_less(uint32_t &v, uint32_t R, uint32_t T, uint32_t x, uint32_t one) {
+  asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p mad.lo.u32 %0, %3, %4, %0;\n\t}"
+      : "+r"(v)
+      : "r"(R), "r"(T), "r"(x), "r"(one));
+}
+
 // ---- bit-sliced helpers shared by the sweep kernels ----
 
 template <typename Word>

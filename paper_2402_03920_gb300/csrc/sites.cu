@@ -38,10 +38,12 @@
 //     with the site alone, and those with the system are the block's;
 //   * a thread walks up the tau' of one column (x, y), two planes a step, so
 //     the couplings and neighbour offsets are fixed, and the word above is
-//     the next step's word below.
+//     the next step's word below;
+//   * the comparison adds its byte's one by a predicated multiply-add and the
+//     round keys are parameters: the logic pipe (62% busy) binds the kernel.
 // 423 instructions per word of 32 updates (555 with 8-byte entries, a branch
 // per look-up, whole Philox calls and index arithmetic per word): 10 sweeps at
-// L = 16, L_tau = 8192, 16 samples 14.25 -> 11.5 ms.
+// L = 16, L_tau = 8192, 16 samples 14.25 -> 10.7 ms (11.2 without the last point).
 //
 // Device arrays (systems walker-major; PT exchanges slot labels only):
 //   spins  u32 [a][r][w][L^2 M]       bit = 1 <=> spin -1
@@ -74,11 +76,13 @@ struct SitesArgs {
   const unsigned long long *d_t;
   unsigned long long *t_copy;  // blue pass: copy t here for the PT pass that advances it (or null)
   uint2 key;
+  PhiloxKeys rk;               // its round keys
   FastDiv plane_div, L_div, bps_div, ns_div, nr_div;
   int L, M, plane, n_words;
   int n_slots, n_rep;
   int n_seg, walk;             // segments per column and words of the colour in one (at most)
   int tau_ap;
+  uint32_t one;                // 1 as a runtime value (add_if_less)
 };
 
 // xoroshiro128++ state step (Blackman and Vigna, 2019) on the 128 bits of a
@@ -112,15 +116,15 @@ static __device__ __noinline__ uint32_t daemon_exact(uint4 x, const uint32_t *lu
 }
 
 // One daemon word: byte i is n* of the 64-bit word whose upper half is Philox
-// output i.  c: the Philox state after two rounds; k: the third round's key.
-__device__ __forceinline__ uint32_t daemon_word(uint4 c, uint2 k, const uint32_t *lut, const unsigned long long *cum) {
+// output i.  c: the Philox state after two rounds; k: the round keys.
+__device__ __forceinline__ uint32_t daemon_word(uint4 c, const PhiloxKeys &k, const uint32_t *lut,
+                                                const unsigned long long *cum, uint32_t one) {
 #pragma unroll
   for (int i = 2; i < 10; ++i) {   // one wide product per half round: measured faster here than two halves
     const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c.x;
     const unsigned long long p1 = (unsigned long long)kPhiloxM1 * c.z;
-    c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k.y, (uint32_t)p0);
-    k.x += kPhiloxW0;
-    k.y += kPhiloxW1;
+    c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.k[i].x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k.k[i].y,
+                   (uint32_t)p0);
   }
   uint32_t e0 = lut[c.x >> (32 - kDaemonLutBits)], e1 = lut[c.y >> (32 - kDaemonLutBits)];
   uint32_t e2 = lut[c.z >> (32 - kDaemonLutBits)], e3 = lut[c.w >> (32 - kDaemonLutBits)];
@@ -139,10 +143,10 @@ __device__ __forceinline__ uint32_t daemon_word(uint4 c, uint2 k, const uint32_t
   // (the entry's low bits do not reach the next cut value: x > e iff the
   // fields compare so)
   uint32_t b = __byte_perm(__byte_perm(e0, e1, 0x0040), __byte_perm(e2, e3, 0x0040), 0x5410);
-  b += x0 > e0 ? 1u : 0u;
-  b += x1 > e1 ? 1u << 8 : 0u;
-  b += x2 > e2 ? 1u << 16 : 0u;
-  b += x3 > e3 ? 1u << 24 : 0u;
+  add_if_less(b, e0, x0, 1u, one);
+  add_if_less(b, e1, x1, 1u << 8, one);
+  add_if_less(b, e2, x2, 1u << 16, one);
+  add_if_less(b, e3, x3, 1u << 24, one);
   const uint32_t tie = min(min(x0 ^ e0, x1 ^ e1), min(x2 ^ e2, x3 ^ e3));   // < 2^bits: equal fields
   if ((tie >> kDaemonLutBits) == 0u || ((e0 | e1 | e2 | e3) & kSpanFlag)) b = daemon_exact(c, lut, cum);
   return b;
@@ -221,12 +225,12 @@ __global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(const SitesArg
         // rounds 1 and 2, the products of the word-site; the three words
         // differ in the last counter word
         const uint32_t zs = __umulhi(kPhiloxM0, ws) ^ p.key.y ^ c3, z2 = (kPhiloxM0 * ws) ^ X;
-        const uint2 k3 = make_uint2(p.key.x + 2 * kPhiloxW0, p.key.y + 2 * kPhiloxW1);
         // b4, b8, b12 in a rolled loop (one copy of the look-up code)
 #pragma unroll 1
         for (uint32_t which = 0; which < 3; ++which) {
           const uint32_t z1 = zs ^ (which << 24);
-          const uint32_t dw = daemon_word(make_uint4(__umulhi(kPhiloxM1, z1) ^ y1, kPhiloxM1 * z1, z2, w2), k3, lut_s, cum_s);
+          const uint32_t dw =
+              daemon_word(make_uint4(__umulhi(kPhiloxM1, z1) ^ y1, kPhiloxM1 * z1, z2, w2), p.rk, lut_s, cum_s, p.one);
           b4 = b8;
           b8 = b12;
           b12 = dw;
@@ -364,6 +368,7 @@ SitesArgs make_args(qisg_handle *h) {
   p.d_t = h->d_t;
   p.t_copy = nullptr;
   p.key = make_uint2((uint32_t)h->seed, (uint32_t)(h->seed >> 32));
+  p.rk = PhiloxKeys(p.key);
   p.L = h->L;
   p.M = h->Lt / 32;
   p.plane = h->L * h->L;
@@ -375,6 +380,7 @@ SitesArgs make_args(qisg_handle *h) {
   p.ns_div = FastDiv((uint32_t)h->n_slots);
   p.nr_div = FastDiv((uint32_t)h->n_rep);
   p.tau_ap = h->tau_ap;
+  p.one = 1u;
   // words per walk: up to 16 (a block stages 40 KB of tables for its 256
   // walks; ms per sweep at 8 | 16 | 32 words: L = 16, L_tau = 8192 1.119 | 1.100
   // | 1.096, L = 24, L_tau = 2048 0.641 | 0.643 | 0.701) while the grid keeps 8
