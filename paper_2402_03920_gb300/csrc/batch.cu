@@ -57,7 +57,7 @@ struct ChainRef {
 
 // One tile of a half sweep of instance I (sample 0, 64-bit LANES words).
 template <bool BLUE>
-__device__ void batch_tile(const InstDev &I, uint32_t t, int colour, int j0, int n, unsigned char *smem) {
+__device__ void batch_tile(const InstDev &I, uint32_t t, uint32_t one, int colour, int j0, int n, unsigned char *smem) {
   LanesSample<unsigned long long> S;
   S.spins = I.spins;
   S.T = I.T;
@@ -79,6 +79,7 @@ __device__ void batch_tile(const InstDev &I, uint32_t t, int colour, int j0, int
   S.rpw = I.rpw;
   S.n_groups = I.n_groups;
   S.tau_ap = I.tau_ap;
+  S.one = one;
   // four replicas (every uneven-batch and serving instance): one quad and
   // the registers of the word groups there are
   if (I.n_rep == 4 && I.n_groups == 1)
@@ -110,7 +111,8 @@ __device__ __forceinline__ bool live(const InstDev &I, int sw) {
 // two or four blocks are within 2% of it.
 __global__ void __launch_bounds__(kBatchBlock, 3) batch_kernel(InstDev *insts, int n_inst, const Tile *tiles,
                                                             int n_tiles, const ChainRef *chains, int n_chains,
-                                                            int n_sweeps, unsigned *bar, int *err, long long wait_ns) {
+                                                            int n_sweeps, unsigned *bar, int *err, long long wait_ns,
+                                                            uint32_t one) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_next[2];
   unsigned *taken = bar + 2;   // [colour]: tiles taken beyond the first of each block
@@ -126,9 +128,9 @@ __global__ void __launch_bounds__(kBatchBlock, 3) batch_kernel(InstDev *insts, i
         if (live(I, sw)) {
           const uint32_t t = (uint32_t)__ldcg(&I.t) + (uint32_t)sw;
           if (colour == 0)
-            batch_tile<false>(I, t, 0, tl.j0, tl.n, smem);
+            batch_tile<false>(I, t, one, 0, tl.j0, tl.n, smem);
           else
-            batch_tile<true>(I, t, 1, tl.j0, tl.n, smem);
+            batch_tile<true>(I, t, one, 1, tl.j0, tl.n, smem);
         }
         __syncthreads();   // s_next is written; the other entry is free again
         k = s_next[buf];
@@ -575,8 +577,9 @@ int qisg_batch_run(qisg_batch *B, int64_t n_sweeps) {
   int64_t left = n_sweeps;
   while (left > 0 && !rc) {
     int ns = (int)std::min<int64_t>(left, chunk);
+    uint32_t one = 1;
     void *args[] = {&B->d_inst, &B->capacity, &B->d_tiles, &B->n_tiles, &B->d_chains, &B->n_chains,
-                    &ns, &B->d_bar, &B->d_err, &B->wait_ns};
+                    &ns, &B->d_bar, &B->d_err, &B->wait_ns, &one};
     rc = cuda_check(cudaMemsetAsync(B->d_bar, 0, 4 * sizeof(unsigned), B->stream), "reset barrier");
     if (rc) break;
     rc = cuda_check(cudaLaunchCooperativeKernel((const void *)batch_kernel, dim3((unsigned)B->grid),

@@ -35,6 +35,7 @@ struct LanesArgs {
   FastDiv half_plane_div, half_L_div;
   int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, sites_per_block;
   int tau_ap;
+  uint32_t one;
   unsigned long long *t_copy;   // blue pass: copy t here for the PT pass that advances it (or null)
 };
 
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(kBlock) lanes_half_sweep_kernel(LanesArgs<Word
   S.rpw = p.rpw;
   S.n_groups = p.n_groups;
   S.tau_ap = p.tau_ap;
+  S.one = p.one;
   const int64_t j0 = (int64_t)blockIdx.x * tile_sites;
   const int n = (int)(p.half_N - j0 < tile_sites ? p.half_N - j0 : tile_sites);
   lanes_tile<Word, false, BLUE, NREP, NGC, TPS>(S, colour, (int)j0, n, count_only, colour == 0 && blockIdx.x == 0, smem_raw);
@@ -269,6 +271,7 @@ LanesArgs<Word> make_args(qisg_handle *h) {
   p.n_groups = h->n_groups;
   p.sites_per_block = kBlock / h->n_slots;
   p.tau_ap = h->tau_ap;
+  p.one = 1u;
   p.t_copy = nullptr;
   return p;
 }
