@@ -306,13 +306,12 @@ def kernel_shares(kern):
 
 
 def red_threads_per_site(w, wb, t_red, n_sm):
-    """Threads per red site of the fused red pass: the library's rule (tile
-    1 -> four, 2 -> two, 0 -> four while one thread per site would fill fewer
-    than four waves of 2048 threads per SM, else one; 64-bit words at most
-    two replicas per thread)."""
+    """Threads per red site of the fused red pass: the library's rule for
+    separate launches (tile 1 -> four, 2 -> two, 0 -> four below 320 red sites
+    per SM, else one; 64-bit words at most two replicas per thread)."""
     if t_red == 0:
         site_threads = (-(-w.n_samples // wb)) * (-(-w.n_replicas // 4)) * w.L * w.L * (w.L_tau // 2)
-        tps = 4 if site_threads < 4 * 2048 * max(1, n_sm) else 1
+        tps = 4 if site_threads < 320 * max(1, n_sm) else 1
     else:
         tps = {1: 4, 2: 2}.get(t_red, 1)
     return 2 if (wb == 64 and tps == 1) else tps
@@ -330,7 +329,7 @@ def kernel_names(layout, wb, tiles, w, n_sm):
         blue = {0: "samples_sweep4_kernel", 2: "samples_sweep4_kernel<min 4 blocks>"}.get(v_blue, "samples_half_sweep_kernel")
     else:
         red = "samples_red_fusedq_kernel<u64, 1>" if tps == 4 else "samples_red_fusedq_kernel<u64, 2>"
-        blue = "samples_half_sweep_kernel"
+        blue = "samples_sweep4_kernel<u64>"
     return {"red": red, "blue": blue}
 
 

@@ -42,7 +42,7 @@ struct InstDev {
   long long remaining;         // sweeps left; < 0: no limit (mutable)
   uint2 key;
   FastDiv hpd, hld;
-  int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, spb, N;
+  int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, N;
   int tau_ap;   // antiperiodic along tau: the wrap tau bond flips sign
   int active;
 };
@@ -266,7 +266,7 @@ struct qisg_batch {
   int schedule = 0;       // 0: instance order; 1: largest instances first
   int grid = 0;
   size_t smem = 0;
-  int max_plane = 4, max_slots = 1, max_rep = 1, max_spb_groups = 1;
+  int max_plane = 4, max_slots = 1, max_rep = 1;
   int64_t launches = 0;
   long long wait_ns = qisg::kBarrierTimeoutNs;   // bound of each grid-barrier wait
 };
@@ -297,7 +297,7 @@ int build_tables(qisg_batch *B) {
     while (rows > 1 && total < (int64_t)8 * rows * 3 * B->n_sm) rows >>= 1;   // three blocks per SM
   }
   B->max_plane = 4;
-  B->max_slots = B->max_rep = B->max_spb_groups = 1;
+  B->max_slots = B->max_rep = 1;
   B->smem = 0;
   for (int i : order) {
     const InstDev &I = B->slots[i].dev;
@@ -309,7 +309,6 @@ int build_tables(qisg_batch *B) {
     B->max_slots = std::max(B->max_slots, I.n_slots);
     B->max_rep = std::max(B->max_rep, I.n_rep);
     B->smem = std::max(B->smem, lanes_tile_smem(I.n_slots, I.n_rep));
-    B->max_spb_groups = std::max(B->max_spb_groups, I.spb * I.n_groups);
   }
   int rc = QISG_OK;
   if (tiles.size() > B->tiles_cap) {
@@ -427,7 +426,6 @@ int setup_slot(qisg_batch *B, int i) {
   I.n_rep = d.n_replicas;
   I.rpw = rpw;
   I.n_groups = n_groups;
-  I.spb = kBatchBlock / n;
   I.N = (int)N;
   I.tau_ap = d.tau_antiperiodic;
   I.active = 1;

@@ -33,21 +33,11 @@ struct LanesArgs {
   uint2 key;
   int64_t N, half_N;
   FastDiv half_plane_div, half_L_div;
-  int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups, sites_per_block;
+  int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups;
   int tau_ap;
-  uint32_t one;
+  uint32_t one;                 // 1 as a runtime value (add_if_less)
   unsigned long long *t_copy;   // blue pass: copy t here for the PT pass that advances it (or null)
 };
-
-template <typename Word>
-__device__ __forceinline__ Word all_ones_if(bool b) {
-  return b ? ~Word(0) : Word(0);
-}
-
-template <typename Word>
-__device__ __forceinline__ uint32_t bit_at(Word w, int lane) {
-  return (uint32_t)(w >> lane) & 1u;
-}
 
 // One half sweep (colour 0 = red, 1 = blue) of samples a0 + blockIdx.y:
 // block x is the tile of colour sites [x * tile_sites, (x+1) * tile_sites),
@@ -269,7 +259,6 @@ LanesArgs<Word> make_args(qisg_handle *h) {
   p.n_rep = h->n_rep;
   p.rpw = h->rpw;
   p.n_groups = h->n_groups;
-  p.sites_per_block = kBlock / h->n_slots;
   p.tau_ap = h->tau_ap;
   p.one = 1u;
   p.t_copy = nullptr;

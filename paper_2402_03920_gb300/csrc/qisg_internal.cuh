@@ -410,16 +410,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, long long 
   return *(volatile int *)err == 0;
 }
 
-// Load through L2 only (CG) where other blocks of the same persistent launch
-// wrote the data in an earlier phase (L1 is not coherent across SMs).
-template <bool CG, typename T>
-__device__ __forceinline__ T ld_g(const T *p) {
-  if constexpr (CG)
-    return __ldcg(p);
-  else
-    return *p;
-}
-
 // v += R < T ? x : 0 by a predicated multiply-add (one is the runtime value 1).
 __device__ __forceinline__ void add_if_less(uint32_t &v, uint32_t R, uint32_t T, uint32_t x, uint32_t one) {
   asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p mad.lo.u32 %0, %3, %4, %0;\n\t}"
@@ -615,22 +605,6 @@ __device__ __forceinline__ void flush_counter(const VCount<Word, K> &c, int *acc
     for (int i = 0; i < KT; ++i) v |= (int)((mine[i] >> lane) & 1u) << i;
     if (v) atomicAdd(&acc[key * W + lane], v);
   }
-}
-
-
-// Sites of one colour: j in [0, N/2) -> site.  Each (y, tau) row holds L/2
-// sites of each colour (L even).
-struct SiteXYT {
-  int x, y, tau;
-};
-__device__ __forceinline__ SiteXYT site_of_colour(int64_t j, int L, int colour) {
-  const int half_L = L >> 1;
-  const int64_t row = j / half_L;
-  SiteXYT s;
-  s.y = (int)(row % L);
-  s.tau = (int)(row / L);
-  s.x = 2 * (int)(j - row * half_L) + ((s.y + s.tau + colour) & 1);
-  return s;
 }
 
 }  // namespace qisg

@@ -1907,7 +1907,7 @@ int64_t blocks_per_set4(int plane, int n_seg, int cols) {
 // that minimises (waves of blocks over the resident ones) x (work of one
 // block), a block's work being its threads' walks of G sites on average
 // (about 490 instructions a site for the four replica words) plus its
-// counter tree (about 14 instructions per counter plane and level): the
+// counter sums (about 14 (2 ks + 13) instructions, ks counter planes): the
 // pass is latency-bound, so a block takes about the same time whatever the
 // blocks beside it on the SM.  Walks of at most max_walk sites; counts that
 // leave segments of unequal length are candidates only when a block holds
@@ -2006,11 +2006,10 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
     // 364; persistent form: 6480: 22.8 | 24.6 | 30.4, 32768: 47.6 | 46.5 |
     // 49.0, 147456: 187 | 158 | 182, 589824: 725 | 567 | 604 (its grid is one
     // wave of 168-register blocks).  64-bit words, replica | pair: 6480: 18.5 |
-    // 17.8, 32768: 48.2 | 47.2, 294912: 365 | 319
+    // 17.8, 32768: 48.2 | 47.2, 294912: 365 | 319 (one line for both words)
     const int64_t sites = h->n_b * h->n_q * (int64_t)a.plane * (h->Lt / 2);
     const int64_t sm = std::max(1, h->n_sm);
-    if (sizeof(Word) == 8) tpsite = sites < 128 * sm ? 4 : 2;
-    else if (h->persistent) tpsite = sites < 128 * sm ? 4 : 2;
+    if (h->persistent) tpsite = sites < 128 * sm ? 4 : 2;
     else tpsite = sites < 320 * sm ? 4 : 1;
   } else {
     tpsite = h->sweep_tile[0] == 1 ? 4 : h->sweep_tile[0] == 2 ? 2 : 1;

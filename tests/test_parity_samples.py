@@ -446,3 +446,22 @@ def test_blue_walks_of_64_bit_words(qisg, L, Lt, n_rep, n_a, tile, ap):
         sums = inst.measurements()
     assert np.array_equal(sums[0], st.sumA) and np.array_equal(sums[1], st.sumB)
     assert np.array_equal(sums[2], st.sumq) and np.array_equal(sums[3], st.sumq2)
+
+
+@pytest.mark.parametrize("W,tile", [(32, 4), (64, 2)])
+@pytest.mark.parametrize("n_slots,L,Lt,n_rep,n_a", [
+    (1, 4, 6, 4, 33),      # no next slot to copy in
+    (2, 6, 4, 3, 65),      # as many slots as the ring has stages, a replica missing
+    (3, 4, 10, 5, 40),     # the ring wraps; a second replica quad
+    (5, 8, 4, 4, 32),      # a block of one plane and a whole number of waves
+])
+def test_red_ring_at_ladder_edges(qisg, W, tile, n_slots, L, Lt, n_rep, n_a):
+    """The red pass's 16-byte forms copy the next slots' words ahead of use."""
+    inst, ladder = make(qisg, L, Lt, 0.2, 0.5, n_slots, 0.9, n_rep, n_a, 29 + n_slots,
+                        layout=qisg.QISG_LAYOUT_SAMPLES, word_bits=W)
+    st = oracle_state(ladder, L, Lt, n_rep, 29 + n_slots, 0, n_a)
+    with inst:
+        inst.set_tiles((tile, 0))
+        inst.sweep(5)
+        oracle.run(st, 5)
+        assert_same_state(inst, st, what=f"W={W} slots {n_slots}")
