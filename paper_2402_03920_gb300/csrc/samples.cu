@@ -4,7 +4,7 @@
 // word see the same ladder slot, so they share one Metropolis table row and
 // one draw R (the draw is keyed on the 64-sample block a >> 6).  The local
 // energy class (u_s, u_t) of every lane is computed with bit-sliced adders;
-// a mux tree over the class bits selects the per-class reject flags.
+// comparisons of the one draw pick the accepting lanes (accept_word).
 //
 // Because a word is one slot, a PT exchange between slots s and s+1 of a
 // sample (Sec. 2.1) moves that sample's bits between the two slot words; the
