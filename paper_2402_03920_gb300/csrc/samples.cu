@@ -860,6 +860,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
 // 20 sweeps: 109.3 -> 100.8 ms (three stages 104, five blocks 102 to 116: the
 // stages take the room of L1).
 constexpr int kRedStages = 2, kRedBlocks = 4;
+constexpr size_t kRedRingBytes = (size_t)kRedStages * 7 * kBlock4 * 16;
 template <typename Word, int RP>
 __global__ void __launch_bounds__(kBlock4, RP * sizeof(Word) == 16 ? kRedBlocks : 0)
     samples_red_fusedq_kernel(const FusedRedArgsT<Word> p, const __grid_constant__ SlotThresholds th) {
@@ -1699,7 +1700,9 @@ __global__ void samples_pack_kernel(Word *spins, const int8_t *stage, const int3
 // what another block wrote in an earlier phase is read after a grid barrier,
 // whose release and acquire fences order the phases' plain accesses, so the
 // neighbour loads hit L1 (through L2 only: 46.2 against 44.5 ms for 20 sweeps of
-// 256 samples at L = 24, L_tau = 512).
+// 256 samples at L = 24, L_tau = 512).  With the red phase's next slots copied to
+// shared memory (a thread per replica quad, whose registers had spilled) and
+// walks of six counter planes that case takes 38.3 ms.
 // The barriers' waits are bounded (error flag -> QISG_ETIMEOUT).
 struct PersistArgs {
   FusedRedArgsT<uint32_t> red;    // src/dst set per sweep from buf
@@ -1725,6 +1728,7 @@ struct PersistArgs {
 template <int RP, int KS>
 __global__ void __launch_bounds__(kBlock4, 3) samples_persistent_kernel(const PersistArgs a,
                                                                       const __grid_constant__ SlotThresholds th) {
+  extern __shared__ uint4 ring[];
   const unsigned long long t0 = __ldcg(a.d_t);
   const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t gstride = (int64_t)gridDim.x * blockDim.x;
@@ -1739,7 +1743,7 @@ __global__ void __launch_bounds__(kBlock4, 3) samples_persistent_kernel(const Pe
     rp.src = a.buf[cur];
     rp.dst = a.buf[cur ^ 1];
     for (int64_t i = gtid; i < a.n_U; i += gstride) a.U[i] = 0;
-    for (int vb = blockIdx.x; vb < a.red_blocks; vb += gridDim.x) red_fusedq_body<uint32_t, RP, 0>(rp, th, vb, t, nullptr);
+    for (int vb = blockIdx.x; vb < a.red_blocks; vb += gridDim.x) red_fusedq_body<uint32_t, RP, RP == 4 ? kRedStages : 0>(rp, th, vb, t, ring);
     if (!grid_barrier(a.bar, a.err, a.wait_ns)) return;
     for (int64_t i = gtid; i < a.n_acc; i += gstride) a.acc[i] = 0;
     SamplesArgs<uint32_t> bp = a.blue;
@@ -1912,9 +1916,10 @@ int64_t blocks_per_set4(int plane, int n_seg, int cols) {
 // blocks beside it on the SM.  Walks of at most max_walk sites; counts that
 // leave segments of unequal length are candidates only when a block holds
 // one segment.  resident(ks) gives the resident blocks for ks counter
-// planes.
+// planes; spill the cost of each plane above six in a kernel that spills there.
 template <typename Resident>
-int wave_fill_segments(int64_t sets, int plane, int half_col, int max_walk, int cols, Resident resident) {
+int wave_fill_segments(int64_t sets, int plane, int half_col, int max_walk, int cols, double spill,
+                       Resident resident) {
   int best = half_col;
   double best_cost = -1.0;
   for (int ns = std::max(1, (half_col + max_walk - 1) / max_walk); ns <= half_col; ++ns) {
@@ -1924,7 +1929,8 @@ int wave_fill_segments(int64_t sets, int plane, int half_col, int max_walk, int 
     const int64_t R = std::max<int64_t>(1, resident(ks));
     const int64_t blocks = sets * blocks_per_set4(plane, ns, cols);
     const int64_t waves = (blocks + R - 1) / R;
-    const double cost = (double)waves * (490.0 * half_col / ns + 14.0 * (2 * ks + 13));
+    const double cost =
+        (double)waves * (490.0 * half_col / ns + 14.0 * (2 * ks + 13)) * (1.0 + spill * std::max(0, ks - 6));
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
       best = ns;
@@ -1956,7 +1962,7 @@ SamplesArgs<Word> make_args4(qisg_handle *h, SlotThresholds &th, int64_t residen
     n_seg = half_col / G;
   } else {
     const int variant = h->sweep_variant[1];
-    n_seg = wave_fill_segments(sets, p.plane, half_col, max_walk, cols, [&](int ks) -> int64_t {
+    n_seg = wave_fill_segments(sets, p.plane, half_col, max_walk, cols, resident_blocks > 0 ? 0.2 : 0.0, [&](int ks) -> int64_t {
       return resident_blocks > 0 ? resident_blocks
                                  : (int64_t)blue_blocks_per_sm<Word>(h, ks, variant) * std::max(1, h->n_sm);
     });
@@ -2003,14 +2009,13 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
     // default, by the red sites of the launch (us per sweep with a thread per
     // replica | pair | quad).  32-bit words: 32768 sites 32.6 | 32.9 | 32.8,
     // 65536: 54.4 | 51.8 | 49.3, 147456: 112 | 110 | 97, 589824: 426 | 414 |
-    // 364; persistent form: 6480: 22.8 | 24.6 | 30.4, 32768: 47.6 | 46.5 |
-    // 49.0, 147456: 187 | 158 | 182, 589824: 725 | 567 | 604 (its grid is one
-    // wave of 168-register blocks).  64-bit words, replica | pair: 6480: 18.5 |
+    // 364; persistent form, whole sweeps: 6480: 25.7 | 28.0 | 34.9,
+    // 32768: 47.7 | 46.7 | 43.4, 147456: 382 | 312 | 267, 589824: 1426 | 1119 |
+    // 1046 (its grid is one wave of 168-register blocks).  64-bit words, replica | pair: 6480: 18.5 |
     // 17.8, 32768: 48.2 | 47.2, 294912: 365 | 319 (one line for both words)
     const int64_t sites = h->n_b * h->n_q * (int64_t)a.plane * (h->Lt / 2);
     const int64_t sm = std::max(1, h->n_sm);
-    if (h->persistent) tpsite = sites < 128 * sm ? 4 : 2;
-    else tpsite = sites < 320 * sm ? 4 : 1;
+    tpsite = sites < (h->persistent ? 128 : 320) * sm ? 4 : 1;
   } else {
     tpsite = h->sweep_tile[0] == 1 ? 4 : h->sweep_tile[0] == 2 ? 2 : 1;
   }
@@ -2035,7 +2040,6 @@ int fused_red(qisg_handle *h) {
   int64_t blocks = 0;
   const int rc = make_red_args<Word>(h, th, p, tpsite, blocks);
   if (rc) return rc;
-  constexpr size_t ring_bytes = (size_t)kRedStages * 7 * kBlock4 * 16;
   const int tok = prof_begin(h, QISG_KERNEL_SWEEP);
   if constexpr (sizeof(Word) == 4) {
     const FusedRedArgs &p32 = p;
@@ -2044,12 +2048,12 @@ int fused_red(qisg_handle *h) {
     else if (tpsite == 2)
       launch_kernel(h->pdl, samples_red_fusedq_kernel<uint32_t, 2>, dim3((unsigned)blocks), dim3(kBlock4), 0, h->stream, p, th);
     else
-      launch_kernel(h->pdl, samples_red_fusedq_kernel<uint32_t, 4>, dim3((unsigned)blocks), dim3(kBlock4), ring_bytes, h->stream, p, th);
+      launch_kernel(h->pdl, samples_red_fusedq_kernel<uint32_t, 4>, dim3((unsigned)blocks), dim3(kBlock4), kRedRingBytes, h->stream, p, th);
   } else {
     if (tpsite == 4)
       launch_kernel(h->pdl, samples_red_fusedq_kernel<Word, 1>, dim3((unsigned)blocks), dim3(kBlock4), 0, h->stream, p, th);
     else
-      launch_kernel(h->pdl, samples_red_fusedq_kernel<Word, 2>, dim3((unsigned)blocks), dim3(kBlock4), ring_bytes, h->stream, p, th);
+      launch_kernel(h->pdl, samples_red_fusedq_kernel<Word, 2>, dim3((unsigned)blocks), dim3(kBlock4), kRedRingBytes, h->stream, p, th);
   }
   prof_end(h, QISG_KERNEL_SWEEP, tok);
   h->launches++;
@@ -2452,7 +2456,9 @@ int samples_persistent(qisg_handle *h, int n_sweeps) {
   a.red.n_zero_U = 0;
   // the blue phase's default segmentation fills the persistent grid (every
   // form of the kernel is bounded to the same residency), walks of at most
-  // 32 sites
+  // 32 sites, above 15 (seven counter planes, with which the kernel spills more)
+  // at a cost (us a sweep, 256 samples at L = 24, L_tau = 512, walks of 4 | 8 |
+  // 16 | 32 sites: 1954 | 1873 | 1995 | 2228)
   int per_sm0 = 0;
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, samples_persistent_kernel<1, 5>, kBlock4, 0),
                   "occupancy");
@@ -2493,7 +2499,12 @@ int samples_persistent(qisg_handle *h, int n_sweeps) {
   QISG_PK(4, 3) QISG_PK(4, 4) QISG_PK(4, 5) QISG_PK(4, 6) QISG_PK(4, 7) QISG_PK(4, 8)
 #undef QISG_PK
   int per_sm = 0;
-  rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock4, 0), "occupancy");
+  const size_t smem = rp == 4 ? kRedRingBytes : 0;
+  if (smem) {   // with the blue phase's shared memory above the default limit
+    rc = cuda_check(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "shared memory");
+    if (rc) return rc;
+  }
+  rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock4, smem), "occupancy");
   if (rc) return rc;
   if (per_sm < 1) return fail(QISG_ECUDA, "persistent kernel does not fit on an SM");
   const int grid = per_sm * std::max(1, h->n_sm);
@@ -2502,7 +2513,7 @@ int samples_persistent(qisg_handle *h, int n_sweeps) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kBlock4);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = h->stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
