@@ -381,9 +381,12 @@ __device__ __forceinline__ unsigned long long gtime() {
 // Grid-wide barrier of a cooperative launch with a bounded wait: bar[0]
 // counts arrivals, bar[1] is the generation.  A wait that exceeds wait_ns
 // sets *err and gives up; every block checks *err after each barrier and
-// leaves (returns false), so the launch always ends.  bar must be zero at
-// launch.
+// leaves (returns false), so the launch always ends.  The verdict is thread
+// 0's, taken once: another block may set *err at any time, and a block must
+// leave or go on as a whole (the phases share tables and indexes through
+// shared memory).  bar must be zero at launch.
 __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, long long wait_ns) {
+  int bad = 0;
   __syncthreads();
   if (threadIdx.x == 0) {
     volatile unsigned *gen = bar + 1;
@@ -405,9 +408,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, long long 
       }
     }
     __threadfence();
+    bad = *(volatile int *)err;
   }
-  __syncthreads();
-  return *(volatile int *)err == 0;
+  return !__syncthreads_or(bad);
 }
 
 // v += R < T ? x : 0 by a predicated multiply-add (one is the runtime value 1).
