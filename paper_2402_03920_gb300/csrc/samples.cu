@@ -695,7 +695,10 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
   const uint32_t off = tau * P;
   // the antiperiodic wrap bond is unsatisfied when its spins agree
   const Word gtp = ones_if<Word>(p.tau_ap && tau + 1 == Lt), gtm = ones_if<Word>(p.tau_ap && tau == 0);
-  uint32_t zo[7];   // word offsets of the seven sites' replica groups
+  // places of the seven sites' replica groups, in groups of RP words (word
+  // offsets would pass 32 bits above 2^30 sites; these hold 2^31 at RP >= 2, and
+  // RP = 1 takes fewer than 2^30, make_red_args)
+  uint32_t zo[7];
   {
     uint32_t z[7];
     z[0] = i2 + off;
@@ -706,7 +709,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
     z[5] = iyp + off;
     z[6] = iym + off;
 #pragma unroll
-    for (int k = 0; k < 7; ++k) zo[k] = 4 * z[k] + (uint32_t)(RP * h);
+    for (int k = 0; k < 7; ++k) zo[k] = (uint32_t)TPS * z[k] + (uint32_t)h;
   }
   const int64_t base = (((int64_t)b * n * p.n_q + q) * p.N) * 4;
   const int64_t SS = (int64_t)p.n_q * p.N * 4;
@@ -725,7 +728,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
       if (live && slot < n) {
         const Word *ps = sb + (int64_t)slot * SS;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) async_copy16(rg + ((slot % NS) * 7 + k) * kBlock4, ps + zo[k]);
+        for (int k = 0; k < 7; ++k) async_copy16(rg + ((slot % NS) * 7 + k) * kBlock4, ps + (size_t)zo[k] * RP);
       }
       async_commit();   // a group per slot, empty past the ladder
     }
@@ -736,10 +739,10 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
     Jyp = Jb[2 * i2 + 1];
     Jym = Jb[2 * iym + 1];
 #pragma unroll
-    for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(cw[k], sb + zo[k]);
+    for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(cw[k], sb + (size_t)zo[k] * RP);
     if (NS == 0 && n > 1)
 #pragma unroll
-      for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n1[k], sb + SS + zo[k]);
+      for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n1[k], sb + SS + (size_t)zo[k] * RP);
   }
 #pragma unroll
   for (int k = 1; k < NS; ++k) copy_in(k);
@@ -752,7 +755,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
   }
   __syncthreads();
   uint4 R4 = make_uint4(0, 0, 0, 0);
-  const uint32_t wbytes = p.one * (uint32_t)sizeof(Word);   // the runtime element size (addr_scaled)
+  const uint32_t gbytes = p.one * (uint32_t)(RP * sizeof(Word));   // a group's bytes as a runtime value (addr_scaled)
   // slot sl: its draws, the words of slot sl after the exchanges of pairs
   // 0 .. sl, the update of the red site and the stores; H1 / H2: slot sl + 1
   // / sl + 2 exists (known at compile time, so the slot has no checks)
@@ -803,7 +806,7 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
       } else if constexpr (H2) {
         const Word *ps = sb + (int64_t)(sl + 2) * SS;
 #pragma unroll
-        for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n2[k], addr_scaled(ps, zo[k], wbytes));
+        for (int k = 0; k < 7; ++k) ld_rp<Word, RP>(n2[k], addr_scaled(ps, zo[k], gbytes));
       }
       Word m[RP];
 #pragma unroll
@@ -842,8 +845,8 @@ __device__ __forceinline__ void red_fusedq_body(const FusedRedArgsT<Word> &p, co
       out[jj] = sc ^ accept_word<Word>(Rj[jj], T, us0, us1, us2, t1 ^ t2, t1 & t2, p.one);
     }
     Word *pd = db + (int64_t)sl * SS;
-    st_rp<Word, RP>(addr_scaled(pd, zo[0], wbytes), out);
-    st_rp<Word, RP>(addr_scaled(pd, zo[1], wbytes), fw[1]);
+    st_rp<Word, RP>(addr_scaled(pd, zo[0], gbytes), out);
+    st_rp<Word, RP>(addr_scaled(pd, zo[1], gbytes), fw[1]);
   };
   const std::integral_constant<bool, true> yes;
   const std::integral_constant<bool, false> no;
@@ -2021,6 +2024,7 @@ int make_red_args(qisg_handle *h, SlotThresholds &th, FusedRedArgsT<Word> &p, in
   }
   if (sizeof(Word) == 8 && tpsite == 1) tpsite = 2;
   const int64_t threads_per_set = (int64_t)a.plane * (h->Lt / 2) * tpsite;
+  // (also what keeps four threads per site, whose word offsets have 32 bits, below 2^30 sites)
   if (threads_per_set + kBlock4 > 0x7FFFFFFF) return fail(QISG_EINVAL, "lattice too large for one launch");
   p.blocks_per_set = (int)((threads_per_set + kBlock4 - 1) / kBlock4);
   p.fd_bps = FastDiv((uint32_t)p.blocks_per_set);
