@@ -73,7 +73,7 @@ __device__ void batch_tile(const InstDev &I, uint32_t t, uint32_t one, int colou
   S.Lt = I.Lt;
   S.plane = I.plane;
   S.half_plane = I.half_plane;
-  S.N = I.N;
+  S.N = (uint32_t)I.N;
   S.n_slots = I.n_slots;
   S.n_rep = I.n_rep;
   S.rpw = I.rpw;

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kBlock) lanes_half_sweep_kernel(LanesArgs<Word
   S.Lt = p.Lt;
   S.plane = p.plane;
   S.half_plane = p.half_plane;
-  S.N = (int)p.N;
+  S.N = (uint32_t)p.N;
   S.n_slots = p.n_slots;
   S.n_rep = p.n_rep;
   S.rpw = p.rpw;

@@ -58,7 +58,8 @@ struct LanesSample {
   uint32_t ctr_w;                // (DOM_SWEEP << 28) | (a >> 6)
   uint32_t t;                    // sweep index
   FastDiv hpd, hld;              // by plane / 2 and by L / 2
-  int L, Lt, plane, half_plane, N, n_slots, n_rep, rpw, n_groups;
+  uint32_t N;                    // sites (up to 2^31)
+  int L, Lt, plane, half_plane, n_slots, n_rep, rpw, n_groups;
   uint32_t one;                  // 1 as a runtime value (add_if_less)
   int tau_ap;                    // antiperiodic along tau: the wrap tau bond flips sign
 };

@@ -40,3 +40,9 @@ def test_samples_above_2_30_sites(qisg, word_bits, slots, tile):
     L_tau = (1 << 16) + (1 << 12)
     _same(_run(qisg, L_tau, slots, qisg.QISG_LAYOUT_SAMPLES, word_bits, tile),
           _run(qisg, L_tau, slots, qisg.QISG_LAYOUT_LANES, 32))
+
+
+def test_lanes_at_2_31_sites(qisg):
+    """The largest lattice, in two word groups of 32 bits and in one of 64."""
+    a, b = (_run(qisg, 1 << 17, 17, qisg.QISG_LAYOUT_LANES, w) for w in (32, 64))
+    _same(a, b)
