@@ -1502,9 +1502,8 @@ __global__ void __launch_bounds__(kBlock4) samples_overlap4_kernel(const Word *s
 // Measurement sums (Appendix E.1): one thread per (sample, slot) and item,
 // items = the replicas' (A, B) then the pairs' q = N - 2 (differing sites);
 // to_q_only only converts the counts to q.
-__global__ void samples_finalize2_kernel(const unsigned long long *__restrict__ U, long long *__restrict__ qcnt,
-                                         long long *__restrict__ sumA, long long *__restrict__ sumB,
-                                         long long *__restrict__ sumq, long long *__restrict__ sumq2, int64_t n_a,
+__global__ void samples_finalize2_kernel(const unsigned long long *U, long long *qcnt, long long *sumA,
+                                         long long *sumB, long long *sumq, long long *sumq2, int64_t n_a,
                                          int n_rep, int n_slots, int64_t N, int to_q_only) {
   pdl_begin();
   const int n_pairs = n_rep * (n_rep - 1) / 2;

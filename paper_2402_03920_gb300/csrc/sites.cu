@@ -175,9 +175,10 @@ __global__ void __launch_bounds__(kBlock) sites_half_sweep_kernel(const SitesArg
   const uint32_t colour = BLUE ? 1u : 0u;
   if (!BLUE && chunk == 0 && threadIdx.x < 2) p.U[(size_t)sys * 2 + threadIdx.x] = 0;
   if (!BLUE && count_only) return;
-  // slot of walker w: lane l of every warp reads walker_at[a][r][l]
+  // slot of walker w: lane l of every warp reads walker_at[a][r][l] (a plain
+  // load: the PT pass before this kernel writes the labels)
   const int lane = threadIdx.x & 31;
-  const int32_t wl = lane < p.n_slots ? __ldg(p.walker + (size_t)ar * p.n_slots + lane) : -1;
+  const int32_t wl = lane < p.n_slots ? p.walker[(size_t)ar * p.n_slots + lane] : -1;
   const int s = max(__ffs(__ballot_sync(0xFFFFFFFFu, wl == (int32_t)w)) - 1, 0);   // rows are permutations
   // stage the slot's tables
   if (!count_only) {
