@@ -198,10 +198,13 @@ int read_back(cudaStream_t st, unsigned char *pin, const int *d_err, const ReadB
   const bool staged = pin && total <= kPinBytes;
   size_t at = 16;
   int rc = QISG_OK;
-  for (int i = 0; i < n && !rc; ++i) {
-    if (!c[i].bytes) continue;
-    rc = cuda_check(cudaMemcpyAsync(staged ? pin + at : c[i].dst, c[i].src, c[i].bytes, cudaMemcpyDeviceToHost, st), "copy");
+  for (int i = 0; i < n; ++i) {
+    if (!rc && c[i].bytes)
+      rc = cuda_check(cudaMemcpyAsync(staged ? pin + at : c[i].dst, c[i].src, c[i].bytes, cudaMemcpyDeviceToHost, st), "copy");
     at += (c[i].bytes + 15) & ~size_t(15);
+    if (!c[i].clear) continue;   // also after a failed copy
+    const int rc_clear = cuda_check(cudaMemsetAsync(const_cast<void *>(c[i].src), 0, c[i].clear, st), "memset");
+    if (!rc) rc = rc_clear;
   }
   *err = 0;
   if (!rc && pin) rc = cuda_check(cudaMemcpyAsync(pin, d_err, sizeof(int), cudaMemcpyDeviceToHost, st), "read error flag");
@@ -886,10 +889,8 @@ int qisg_overlaps(qisg_handle *h, int64_t *q) {
                                              : samples_measure(h, 1);
   if (rc) return rc;
   const size_t n = (size_t)h->n_samples * h->n_slots * n_pairs;
-  rc = read_back(h, {{q, h->d_q, n * 8}});
-  if (!rc) rc = cuda_check(cudaMemsetAsync(h->d_q, 0, (size_t)h->n_a_pad * h->n_slots * n_pairs * 8, h->stream),
-                           "memset");
-  return rc;
+  // the measurements add difference counts to d_q: no q value stays there
+  return read_back(h, {{q, h->d_q, n * 8, (size_t)h->n_a_pad * h->n_slots * n_pairs * 8}});
 }
 
 int qisg_permutation(qisg_handle *h, int32_t *walker_at) {

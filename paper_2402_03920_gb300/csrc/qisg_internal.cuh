@@ -797,6 +797,7 @@ struct ReadBack {
   void *dst;
   const void *src;
   size_t bytes;
+  size_t clear = 0;   // bytes at src zeroed once they are copied, before the synchronisation
 };
 int read_back(cudaStream_t st, unsigned char *pin, const int *d_err, const ReadBack *c, int n, int *err);
 int read_back(qisg_handle *h, std::initializer_list<ReadBack> c);
