@@ -425,6 +425,18 @@ int lanes_pt(qisg_handle *h, int explicit_pass) {
   return pt_pass(h, explicit_pass, 0, h->n_samples, !explicit_pass && lanes_pt_advances(h) ? h->d_t : nullptr);
 }
 
+// The streams and events of lanes_forked_sweep; what an earlier call could not
+// make is made now.
+static int lanes_make_branches(qisg_handle *h) {
+  int rc = QISG_OK;
+  if (!h->fork_ev) rc = cuda_check(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming), "event");
+  for (int b = 0; b < kLanesBranches && !rc; ++b) {
+    if (!h->branch[b]) rc = cuda_check(cudaStreamCreateWithFlags(&h->branch[b], cudaStreamNonBlocking), "branch stream");
+    if (!rc && !h->join_ev[b]) rc = cuda_check(cudaEventCreateWithFlags(&h->join_ev[b], cudaEventDisableTiming), "event");
+  }
+  return rc;
+}
+
 // One sweep of the per-instance form inside a stream capture: the launches of
 // different samples are independent (red, blue and PT of a sample follow one
 // another), so they are captured on kLanesBranches branches that fork from
@@ -433,15 +445,8 @@ int lanes_pt(qisg_handle *h, int explicit_pass) {
 // one waited for the one before it.  Production shape, 10 sweeps: 6.3 ms in a
 // chain, 2.57 | 2.28 | 2.27 on 4 | 8 | 16 branches.
 int lanes_forked_sweep(qisg_handle *h, int with_pt) {
-  int rc = QISG_OK;
-  if (!h->fork_ev) {
-    rc = cuda_check(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming), "event");
-    for (int b = 0; b < kLanesBranches && !rc; ++b) {
-      rc = cuda_check(cudaStreamCreateWithFlags(&h->branch[b], cudaStreamNonBlocking), "branch stream");
-      if (!rc) rc = cuda_check(cudaEventCreateWithFlags(&h->join_ev[b], cudaEventDisableTiming), "event");
-    }
-    if (rc) return rc;
-  }
+  int rc = lanes_make_branches(h);
+  if (rc) return rc;
   const int64_t in_flight = std::min<int64_t>(kLanesBranches, h->n_samples);
   cudaStream_t main = h->stream;
   const bool pdl = h->pdl;
