@@ -517,13 +517,16 @@ int qisg_batch_retire(qisg_batch *b, int slot);
 /* Advance every admitted instance by n_sweeps sweeps (an instance stops at
  * its target).  One cooperative persistent kernel runs all of them: red and
  * blue half sweeps over a work-list of (instance, site range) tiles, a PT
- * pass with one warp per (instance, replica) chain, and the counter advance,
- * separated by grid barriers whose waits are bounded (ETIMEOUT at the next
- * synchronising call if one gives up).  Asynchronous. */
+ * pass with one warp per (instance, replica) chain, separated by grid barriers
+ * whose waits are bounded (ETIMEOUT at the next synchronising call if one
+ * gives up); the sweep counters advance once, after the last sweep.
+ * Asynchronous. */
 int qisg_batch_run(qisg_batch *b, int64_t n_sweeps);
 
-/* Tile rows of 256 sites per work item (1..16) and tile order (0: admission order, 1:
- * largest instances first).  Results never depend on either. */
+/* Tile rows of 256 sites per work item (1..16; 0, the default: 8, 4, 2 or 1, by
+ * the sites of the instances admitted at the time) and tile order (0, the
+ * default: admission order, 1: largest instances first).  Results never
+ * depend on either.  EINVAL: rows or order outside these. */
 int qisg_batch_set_schedule(qisg_batch *b, int tile_rows, int schedule);
 
 /* Bound of each grid-barrier wait of the batch kernel, in nanoseconds (0:
@@ -534,8 +537,10 @@ int qisg_batch_set_schedule(qisg_batch *b, int tile_rows, int schedule);
  * EINVAL: wait_ns < 0. */
 int qisg_batch_set_wait_limit(qisg_batch *b, int64_t wait_ns);
 
-/* Time sweeps_per_candidate sweeps of each (tile rows, order) candidate on the
- * live batch and keep the fastest; the batch advances meanwhile. */
+/* Time sweeps_per_candidate sweeps of each (tile rows 1, 2, 4, 8, 16; order)
+ * candidate on the live batch and keep the fastest, also when instances come
+ * and go later (qisg_batch_set_schedule with 0 rows returns to the default);
+ * the batch advances meanwhile. */
 int qisg_batch_autotune(qisg_batch *b, int sweeps_per_candidate, int *tile_rows, int *schedule);
 
 /* Sweeps done by a slot and whether it reached its target. */

@@ -602,7 +602,7 @@ int qisg_batch_set_wait_limit(qisg_batch *B, int64_t wait_ns) {
 }
 
 int qisg_batch_set_schedule(qisg_batch *B, int tile_rows, int schedule) {
-  if (!B || tile_rows < 1 || tile_rows > kLanesMaxSitesPerThread || schedule < 0 || schedule > 1)
+  if (!B || tile_rows < 0 || tile_rows > kLanesMaxRows || schedule < 0 || schedule > 1)
     return fail(QISG_EINVAL, "bad schedule");
   B->tile_rows = tile_rows;
   B->schedule = schedule;

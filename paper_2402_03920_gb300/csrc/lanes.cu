@@ -299,10 +299,10 @@ int half_sweep_t(qisg_handle *h, int colour, int count_only, int64_t a_lo, int64
   // systems, four | one thread per site: 4096 sites a colour 12.4 | 16.5,
   // 16384: 14.4 | 16.5, 32768: 20.6 | 16.5, 147456: 49.1 | 35.4
   const int tps = p.half_N * in_flight < 160LL * h->n_sm ? 4 : 1;
-  // tiles of rows x (256 / tps) sites (rows <= 16, the counters' limit), as
-  // long as the grid keeps about four blocks per SM
+  // tiles of up to kLanesMaxRows x (256 / tps) sites, as long as the grid keeps
+  // about four blocks per SM
   const int per = kBlock / tps;
-  int rows = 16;
+  int rows = kLanesMaxRows;
   while (rows > 1 && ((p.half_N + per * (int64_t)rows - 1) / (per * (int64_t)rows)) * n_launch_samples < 4LL * h->n_sm) rows >>= 1;
   const int tile_sites = per * rows;
   const int64_t blocks = (p.half_N + tile_sites - 1) / tile_sites;

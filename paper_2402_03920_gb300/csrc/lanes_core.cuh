@@ -40,7 +40,7 @@
 namespace qisg {
 
 constexpr int kLanesMaxGroups = 2;    // word groups per site held in registers
-constexpr int kLanesMaxSitesPerThread = 16;   // tile rows
+constexpr int kLanesMaxRows = 16;     // rows of kLanesThreads sites in a tile (a choice: the counters are flushed every seven)
 constexpr int kLanesKs = 5;           // u_s counter planes: <= 4 x 7 sites per thread
 constexpr int kLanesKt = 4;           // u_t counter planes: <= 2 x 7 sites per thread
 constexpr int kLanesFlushSites = 7;   // sites per thread between flushes of the counters

@@ -186,3 +186,20 @@ def test_antiperiodic_instances_in_the_mix(qisg):
             A, B, wa, S = b.results(slot, spins=True)
             assert np.array_equal(S, st.S[0]) and np.array_equal(wa, st.walker_at[0]), slot
             assert np.array_equal(A, st.A[0]) and np.array_equal(B, st.B[0]), slot
+
+
+def test_default_rows_can_be_had_again(qisg):
+    """0 tile rows, the default, is a schedule like any other; what lies outside is refused."""
+    lad = qisg.ladder_linear(0.2, 0.5, 7, 1.0)
+    with qisg.Batch(2, 64 << 20) as b:
+        slot = b.admit(8, 16, lad, 4, 51)
+        b.set_schedule(16, 1)
+        b.run(3)
+        b.set_schedule(0, 0)
+        b.run(4)
+        for rows, order in ((-1, 0), (17, 0), (0, -1), (0, 2)):
+            with pytest.raises(qisg.QisgError):
+                b.set_schedule(rows, order)
+        _, _, wa, S = b.results(slot, spins=True)
+        st = _oracle_instance(8, 16, lad, 4, 51, 7)
+        assert np.array_equal(S, st.S[0]) and np.array_equal(wa, st.walker_at[0])
