@@ -138,9 +138,14 @@ int qisg_daemon_tables(double k, int lut_bits, uint64_t *cum, uint16_t *lut);
  *   ladder: host array of n_slots slots (copied).  opts may be NULL.
  * EINVAL: L odd or < 2; L_tau odd or < 2; n_slots < 1; n_replicas < 1;
  *   n_samples < 1; a k or k_tau negative or non-finite; a packing that cannot
- *   hold the systems (LANES needs n_slots <= word bits and n_replicas <=
- *   2 * (word bits / n_slots); SAMPLES needs n_slots <= 32).
- * ENOMEM: allocation failed or the state exceeds opts->mem_budget.        */
+ *   hold the systems (LANES needs n_slots <= word bits, n_replicas <=
+ *   2 * (word bits / n_slots) and 11 L^2 + 4 n_slots (32 + n_replicas) <=
+ *   198656, L <= 132 or 134; SAMPLES needs n_slots <= 32 and L <= 1024); more
+ *   than 2^31 sites.
+ * ENOMEM: allocation failed or the state exceeds opts->mem_budget.
+ * Beside its device memory each handle holds 256 KiB of pinned host memory,
+ * through which read-outs of up to that size pass (where none can be had they
+ * are copied straight to the caller's arrays). */
 int qisg_create(qisg_handle **out, int L, int L_tau, const qisg_slot *ladder, int n_slots,
                 int n_replicas, int64_t n_samples, uint64_t seed, const qisg_opts *opts);
 

@@ -266,7 +266,6 @@ struct qisg_batch {
   int schedule = 0;       // 0: instance order; 1: largest instances first
   int grid = 0;
   size_t smem = 0;
-  int max_plane = 4, max_slots = 1, max_rep = 1;
   int64_t launches = 0;
   long long wait_ns = qisg::kBarrierTimeoutNs;   // bound of each grid-barrier wait
 };
@@ -296,8 +295,6 @@ int build_tables(qisg_batch *B) {
     rows = 8;
     while (rows > 1 && total < (int64_t)8 * rows * 3 * B->n_sm) rows >>= 1;   // three blocks per SM
   }
-  B->max_plane = 4;
-  B->max_slots = B->max_rep = 1;
   B->smem = 0;
   for (int i : order) {
     const InstDev &I = B->slots[i].dev;
@@ -305,9 +302,6 @@ int build_tables(qisg_batch *B) {
     const int half = I.N / 2;
     for (int j0 = 0; j0 < half; j0 += per) tiles.push_back(Tile{i, j0, std::min(per, half - j0)});
     for (int r = 0; r < I.n_rep; ++r) chains.push_back(ChainRef{i, r});
-    B->max_plane = std::max(B->max_plane, I.plane);
-    B->max_slots = std::max(B->max_slots, I.n_slots);
-    B->max_rep = std::max(B->max_rep, I.n_rep);
     B->smem = std::max(B->smem, lanes_tile_smem(I.n_slots, I.n_rep));
   }
   int rc = QISG_OK;
@@ -334,7 +328,6 @@ int build_tables(qisg_batch *B) {
   if (rc) return rc;
   B->n_tiles = (int)tiles.size();
   B->n_chains = (int)chains.size();
-  if (!lanes_plane_fits(B->max_plane, B->max_slots, B->max_rep, 200 * 1024)) return fail(QISG_EINVAL, "instance too large for the batch kernel's shared memory");
   cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->smem);
   int per_sm = 0;
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kBatchBlock, B->smem),

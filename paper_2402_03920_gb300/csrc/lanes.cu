@@ -284,14 +284,22 @@ int set_smem_limits() {
   return QISG_OK;
 }
 
+// The planes the packing takes (L <= 132 for any ladder, 134 for short ones).
+// Nothing of the tile's depends on the plane: earlier tiles kept tables of 11
+// bytes per site beside 33792 fixed bytes in 227 KB, and handles beyond that
+// are refused as they were.
+bool lanes_plane_taken(int plane, int n_slots, int n_rep) {
+  return (int64_t)plane * 11 + 4LL * n_slots * (32 + n_rep) <= 227 * 1024 - 33792;
+}
+
 // One colour of samples a_lo .. a_lo + n_a - 1 on stream st, in_flight samples
 // running at a time.
 template <typename Word>
 int half_sweep_t(qisg_handle *h, int colour, int count_only, int64_t a_lo, int64_t n_a, int64_t in_flight, cudaStream_t st) {
   LanesArgs<Word> p = make_args<Word>(h);
   if (colour == 1 && !count_only && lanes_pt_advances(h)) p.t_copy = h->d_t + 1;
-  if (!lanes_plane_fits(p.plane, h->n_slots, h->n_rep, 227 * 1024))
-    return fail(QISG_EINVAL, "LANES plane tables exceed shared memory");
+  if (!lanes_plane_taken(p.plane, h->n_slots, h->n_rep))
+    return fail(QISG_EINVAL, "the LANES packing takes 11 L^2 + 4 n_slots (32 + n_replicas) <= 198656");
   const size_t smem = lanes_tile_smem(h->n_slots, h->n_rep);
   const int64_t n_launch_samples = h->per_sample_launch ? 1 : h->n_samples;
   // four threads per site where the sites in flight are few (one launch's, or

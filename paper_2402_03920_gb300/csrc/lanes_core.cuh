@@ -76,15 +76,6 @@ __host__ __device__ inline size_t lanes_tile_smem(int n_slots, int n_rep) {
   return (o + 15) & ~size_t(15);
 }
 
-// The largest planes the packing takes: 11 bytes per site of the plane
-// beside the fixed tables have to stay within `limit` bytes.
-inline bool lanes_plane_fits(int plane, int n_slots, int n_rep, size_t limit) {
-  size_t o = (size_t)(n_slots * 32 + n_rep * n_slots) * 4 + (size_t)2 * kLanesMaxGroups * 64 * 4 +
-             (size_t)kLanesCodeWords * kLanesThreads * 4;
-  o = ((o + 7) & ~size_t(7)) + (size_t)plane * 11;
-  return ((o + 15) & ~size_t(15)) <= limit;
-}
-
 template <bool CG, typename Word>
 __device__ __forceinline__ Word ld_word(const Word *p) {
   return CG ? __ldcg(p) : *p;

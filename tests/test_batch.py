@@ -203,3 +203,16 @@ def test_default_rows_can_be_had_again(qisg):
         _, _, wa, S = b.results(slot, spins=True)
         st = _oracle_instance(8, 16, lad, 4, 51, 7)
         assert np.array_equal(S, st.S[0]) and np.array_equal(wa, st.walker_at[0])
+
+
+def test_largest_lattice_side_runs(qisg):
+    """L = 128, the largest side an instance is admitted with, beside a small
+    instance with another ladder."""
+    specs = [(128, 4, 32, 61), (4, 6, 3, 62)]
+    with qisg.Batch(2, 64 << 20) as b:
+        slots = [b.admit(L, Lt, qisg.ladder_linear(0.2, 0.5, ns, 1.0), 4, seed) for (L, Lt, ns, seed) in specs]
+        b.run(2)
+        for slot, (L, Lt, ns, seed) in zip(slots, specs):
+            _, _, wa, S = b.results(slot, spins=True)
+            st = _oracle_instance(L, Lt, qisg.ladder_linear(0.2, 0.5, ns, 1.0), 4, seed, 2)
+            assert np.array_equal(S, st.S[0]) and np.array_equal(wa, st.walker_at[0]), L

@@ -244,3 +244,11 @@ def test_edge_cases_bit_exact(qisg, W, L, Lt, n_slots, n_rep, pt_every, measure_
         sA, sB, sq, sq2, nm = inst.measurements()
         assert nm == st.n_meas
         assert np.array_equal(sA, st.sumA) and np.array_equal(sB, st.sumB)
+
+
+@pytest.mark.parametrize("n_slots,n_rep,largest", [(1, 1, 134), (32, 4, 132)])
+def test_largest_lattice_side(qisg, n_slots, n_rep, largest):
+    """The side up to which the packing takes a lattice; beyond it the handle is refused."""
+    make(qisg, largest, 2, 0.2, 0.5, n_slots, 1.0, n_rep, 1, 3, layout=qisg.QISG_LAYOUT_LANES)[0].close()
+    with pytest.raises(qisg.QisgError):
+        make(qisg, largest + 2, 2, 0.2, 0.5, n_slots, 1.0, n_rep, 1, 3, layout=qisg.QISG_LAYOUT_LANES)
