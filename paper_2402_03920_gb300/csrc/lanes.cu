@@ -445,10 +445,10 @@ static int lanes_make_branches(qisg_handle *h) {
   return rc;
 }
 
-// One sweep of the per-instance form inside a stream capture: the launches of
-// different samples are independent (red, blue and PT of a sample follow one
-// another), so they are captured on kLanesBranches branches that fork from
-// h->stream and join it again.  One launch of the production lattice fills a
+// One sweep of the per-instance form: the launches of different samples are
+// independent (red, blue and PT of a sample follow one another), so they go to
+// kLanesBranches streams that fork from h->stream and join it again (in a
+// capture: branches of its graph).  One launch of the production lattice fills a
 // tenth of the GPU's threads and lasts a few microseconds; in a chain each
 // one waited for the one before it.  Production shape, 10 sweeps: 6.3 ms in a
 // chain, 2.57 | 2.28 | 2.27 on 4 | 8 | 16 branches.

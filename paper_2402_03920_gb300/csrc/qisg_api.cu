@@ -457,9 +457,9 @@ int one_sweep(qisg_handle *h, cudaEvent_t *ev = nullptr) {
   const bool sites = h->layout == QISG_LAYOUT_SITES;
   const uint64_t t = h->t;
   const bool pt_due = h->pt_every > 0 && (t + 1) % (uint64_t)h->pt_every == 0;
-  // the captured per-instance form runs its samples side by side (timed
-  // launches need the graph to be a chain)
-  const bool forked = lanes && !sites && h->per_sample_launch && h->stream == h->cap_stream && !h->prof;
+  // the per-instance form runs its samples side by side, captured or not
+  // (timed launches need the graph to be a chain)
+  const bool forked = lanes && !sites && h->per_sample_launch && h->n_samples > 1 && !h->prof;
   int rc = ev ? cuda_check(cudaEventRecord(ev[0], h->stream), "record") : QISG_OK;
   if (forked) rc = lanes_forked_sweep(h, pt_due);
   else if (!rc) rc = sites ? sites_half_sweep(h, 0, 0) : lanes ? lanes_half_sweep(h, 0, 0) : samples_half_sweep(h, 0, 0);

@@ -615,7 +615,7 @@ __device__ __forceinline__ void flush_counter(const VCount<Word, K> &c, int *acc
 // ----------------------------------------------------------------------------
 // The handle.
 // ----------------------------------------------------------------------------
-constexpr int kLanesBranches = 8;   // branches of the captured per-instance sweep
+constexpr int kLanesBranches = 8;   // branches of the per-instance sweep
 
 struct qisg_handle {
   // problem
@@ -720,7 +720,7 @@ struct qisg_handle {
   // captured on cap_stream and replayed on stream
   bool use_graphs = true;
   cudaStream_t cap_stream = nullptr;
-  cudaStream_t branch[kLanesBranches] = {};   // per-instance LANES: branches of the captured sweep
+  cudaStream_t branch[kLanesBranches] = {};   // per-instance LANES: branches of the sweep
   cudaEvent_t fork_ev = nullptr, join_ev[kLanesBranches] = {};
   cudaGraph_t cyc_graph = nullptr;
   cudaGraphExec_t cyc_exec = nullptr;

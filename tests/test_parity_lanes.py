@@ -252,3 +252,19 @@ def test_largest_lattice_side(qisg, n_slots, n_rep, largest):
     make(qisg, largest, 2, 0.2, 0.5, n_slots, 1.0, n_rep, 1, 3, layout=qisg.QISG_LAYOUT_LANES)[0].close()
     with pytest.raises(qisg.QisgError):
         make(qisg, largest + 2, 2, 0.2, 0.5, n_slots, 1.0, n_rep, 1, 3, layout=qisg.QISG_LAYOUT_LANES)
+
+
+@pytest.mark.parametrize("n_samples,graphs", [(1, True), (11, False)])
+def test_per_instance_on_a_stream_of_its_own(qisg, n_samples, graphs):
+    """One launch per sample, captured and launched directly, ordered on the caller's stream."""
+    torch = need_gpu()
+    lad = qisg.ladder_linear(0.2, 0.5, 6, 1.0)
+    cfg = qisg.Config(8, 16, lad, 3, n_samples, 19, per_sample_launch=1, layout=qisg.QISG_LAYOUT_LANES, measure_every=3)
+    st = oracle_state(lad, 8, 16, 3, 19, 0, n_samples)
+    stream = torch.cuda.Stream()
+    with qisg.Instance(cfg, stream=stream.cuda_stream) as inst:
+        inst.set_graphs(graphs)
+        for n in (2, 6, 5):   # with graphs: replays between direct launches
+            inst.sweep(n)
+            oracle.run(st, n, measure_every=3)
+            assert_same_state(inst, st, what=f"after {st.t}")
