@@ -26,7 +26,7 @@
 // Where the terms cancel (SF below 1/16 of the sum of their magnitudes, a
 // near-uniform q~; always at lag 0, whose SF the host computes) that lag is
 // evaluated as written above instead: rows and columns in order x = 0 .. L-1,
-// tau_1 in order, FP64 without contraction.
+// FP64 without contraction, a warp per lag with the tau_1 over its lanes.
 //
 // What bounds it: the population counts (16 lanes an SM) and integer issue,
 // about 140 instructions per pair of slices at L = 16.  A block takes one
@@ -104,12 +104,13 @@ struct TauPlane {
   }
 };
 
-// SF of one lag from its definition.
+// SF of one lag from its definition, by one warp: lane l takes the tau_1
+// congruent to l.  Every lane gets the sum.
 template <int L>
 __device__ __noinline__ double tau_sf_direct(const TauArgs &a, const uint32_t *W, int tau) {
   using P = TauPlane<L>;
   double sf = 0.0;
-  for (int t1 = 0; t1 < a.Lt; ++t1) {
+  for (int t1 = threadIdx.x & 31; t1 < a.Lt; t1 += 32) {
     const int t2 = t1 + tau < a.Lt ? t1 + tau : t1 + tau - a.Lt;
     const uint32_t *w1 = W + (size_t)t1 * a.pitch, *w2 = W + (size_t)t2 * a.pitch;
     double re1 = 0.0, im1 = 0.0, re2 = 0.0, im2 = 0.0;
@@ -125,6 +126,8 @@ __device__ __noinline__ double tau_sf_direct(const TauArgs &a, const uint32_t *W
     const double f2 = __dadd_rn(__dmul_rn(re2, re2), __dmul_rn(im2, im2));
     sf = __dadd_rn(sf, __dadd_rn(f1, f2));
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sf = __dadd_rn(sf, __shfl_xor_sync(0xffffffffu, sf, o));
   return sf;
 }
 
@@ -269,9 +272,18 @@ __global__ void __launch_bounds__(kTauBlock) tau_obs_kernel(const TauArgs a) {
         a.S1[o] = s1;
         a.S2[o] = (long long)s2;
         a.S4[o] = (long long)s4;
-        a.SF[o] = direct ? tau_sf_direct<L>(a, W, lag) : 4.0 * sf;
+        a.SF[o] = direct ? -1.0 : 4.0 * sf;   // -1 (no SF is negative): left to a warp below
       }
     }
+  }
+  __syncthreads();
+  // the lags whose terms cancel, a warp each; tau and L_tau - tau have the same terms
+  for (int tau = 1 + (int)(threadIdx.x >> 5); tau <= nl; tau += kTauBlock / 32) {
+    double *o = a.SF + c * Lt;
+    if (o[tau] >= 0.0) continue;   // the same in every lane
+    const double sf = tau_sf_direct<L>(a, W, tau);
+    __syncwarp();                  // every lane has read the mark
+    if ((threadIdx.x & 31) == 0) o[tau] = o[Lt - tau] = sf;
   }
   if (threadIdx.x == 0) {   // lag 0: q~ = 1 at every site
     const int64_t o = c * Lt;

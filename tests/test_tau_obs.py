@@ -78,3 +78,27 @@ def test_tau_observables_of_given_states(qisg, L, Lt, n_slots, n_rep, pattern):
     # the integer sums leave a few roundings at most 16 times enlarged by
     # cancellation (below 1e-13); other lags are the oracle's sums themselves
     assert np.allclose(got[3], want[3], rtol=1e-12, atol=0), "SF"
+
+
+@pytest.mark.parametrize("L,Lt", [(8, 2), (8, 6), (8, 70), (2, 600), (18, 34)])
+def test_cancelling_lags(qisg, L, Lt):
+    """Lags evaluated from the definition (a warp each, tau_1 over its lanes)
+    beside lags of the integer form: uniform layers, but for one replica with a
+    few layers of random spins."""
+    rng = np.random.default_rng(L * 1000 + Lt)
+    S = np.broadcast_to(rng.choice([-1, 1], size=(1, 3, 2, Lt, 1, 1)), (1, 3, 2, Lt, L, L)).copy()
+    S[:, 1, :, :1] = rng.choice([-1, 1], size=(1, 2, 1, L, L))
+    half = S[:, 2, :, :, :, : L // 2]   # q~ of period L / 2: no wave at the first wave number
+    half[:] = rng.choice([-1, 1], size=(1, 2, Lt, L, L // 2))
+    S[:, 2, :, :, :, L // 2:] = half
+    S = np.ascontiguousarray(S.reshape(1, 3, 2, Lt * L * L), dtype=np.int8)
+    wa = np.tile(np.arange(2, dtype=np.int32), (1, 3, 1))
+    inst, _ = make(qisg, L, Lt, 0.2, 0.5, 2, 1.0, 3, 1, 3, layout=qisg.QISG_LAYOUT_SAMPLES, word_bits=32)
+    with inst:
+        inst.set_state(S, wa, 0)
+        got = inst.tau_observables()
+    want = oracle.tau_observables(L, Lt, S, wa)
+    for name, g, w in zip(("S1", "S2", "S4"), got[:3], want[:3]):
+        assert np.array_equal(g, w), name
+    # sums of at most 600 terms that are not negative, in another order: below 1e-13
+    assert np.allclose(got[3], want[3], rtol=1e-12, atol=0), "SF"
