@@ -74,7 +74,7 @@ __device__ __forceinline__ int energy_index(const TransferArgs &a, uint32_t n) {
 // One pass: the tile's geometry and what the pass does besides its rounds.
 struct PassArgs {
   int c, lo, hi;      // tile bits: [0, c) and the rounds' bits [lo, hi)
-  int first, last;    // multiply by w on load / parity factor and w at the end
+  int first;          // multiply by w on load
   int nb;             // index bits
 };
 
@@ -109,7 +109,6 @@ __device__ __forceinline__ void rounds(double (&v)[1 << G], double r) {
 // G rounds on tile bits [tb, tb + G) of the whole tile (PAIR: of the tile and
 // its complement, element t of the one with element T - 1 - t of the other).
 // FROM / TO: elements come from src / go to dst instead of shared memory.
-// The tile of an unpaired last pass stays in shared memory (dst null).
 template <int G, bool PAIR, bool FROM, bool TO>
 __device__ __forceinline__ void stage(const double *src, double *dst, double *tile, const double *wt,
                                       const TransferArgs &a, const PassArgs &q, int T_log, uint32_t f, int tb) {
@@ -170,9 +169,8 @@ __device__ __forceinline__ void stage_g(int g, const double *src, double *dst, d
   }
 }
 
-// Block f takes the tile of fixed bits f (PAIR: and its complement, f below
-// half of them).  PAIR: the last pass with fixed bits; a last pass without
-// any holds the whole vector in one tile.  src and dst may be the same: every
+// Block f takes the tile of fixed bits f (PAIR, the last pass: and its
+// complement, f below half of them).  src and dst may be the same: every
 // element is read by the block that writes it, before it does.
 template <bool PAIR>
 __global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const double *src, double *dst,
@@ -189,7 +187,6 @@ __global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const dou
   __syncthreads();
   constexpr int GM = PAIR ? 3 : 4;
   int tb = q.c, left = q.hi - q.lo;
-  const bool to_mem = PAIR || !q.last;   // the last group writes HBM
   bool loaded = false;
   if (!PAIR && tb < 4) {   // consecutive elements per thread: load whole segments first
     for (uint32_t t = threadIdx.x; t < T; t += blockDim.x) {
@@ -202,7 +199,7 @@ __global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const dou
   }
   while (left > 0) {
     const int g = left < GM ? left : GM;
-    const bool end = left == g && to_mem;
+    const bool end = left == g;   // the last group writes HBM
     if (!loaded && end)
       stage_g<PAIR, true, true>(g, src, dst, tile, wt, a, q, T_log, f, tb);
     else if (!loaded)
@@ -216,12 +213,30 @@ __global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const dou
     left -= g;
     if (!end) __syncthreads();
   }
-  if (!PAIR && q.last)   // the whole vector in one tile: element t pairs with T-1-t
-    for (uint32_t t = threadIdx.x; t < T / 2; t += blockDim.x) {
-      const double x = tile[padded(t)], y = tile[padded(T - 1u - t)];
-      dst[t] = __dmul_rn(__fma_rn(a.pr, y, x), wt[64 + energy_index(a, t)]);
-      dst[T - 1u - t] = __dmul_rn(__fma_rn(a.pr, x, y), wt[64 + energy_index(a, T - 1u - t)]);
-    }
+}
+
+// L = 2 and 3, at most 256 elements: the product in one block, element n in
+// thread n, the rounds within a warp by shuffles.  Latency is all there is: the
+// kernel takes 2.6 and 3.5 us under ncu (6.2 and 11.2 in the tiled form, whose
+// groups of four rounds leave one and 16 threads at work); a call that is waited
+// for went from 25 and 28 us to 22 and 23.
+__global__ void __launch_bounds__(256) transfer_small_kernel(const double *in, double *out,
+                                                             const __grid_constant__ TransferArgs a, int nb) {
+  __shared__ double x[256];
+  const uint32_t n = threadIdx.x, T = 1u << nb;
+  const bool live = n < T;   // L = 2: 8 of a warp
+  const double w = live ? a.wtab[energy_index(a, n)] : 0.0;
+  double v = live ? __dmul_rn(in[n], __dmul_rn(w, a.jPn)) : 0.0;
+  for (int j = 0; j < min(nb, 5); ++j) v = __fma_rn(a.r, __shfl_xor_sync(0xffffffffu, v, 1 << j), v);
+  for (int j = 5; j < nb; ++j) {
+    x[n] = v;
+    __syncthreads();
+    v = __fma_rn(a.r, x[n ^ (1u << j)], v);
+    __syncthreads();
+  }
+  x[n] = v;
+  __syncthreads();
+  if (live) out[n] = __dmul_rn(__fma_rn(a.pr, x[T - 1u - n], v), w);
 }
 
 struct Pass {
@@ -280,17 +295,20 @@ extern "C" int qisg_transfer_matvec(const double *in, double *out, int L, double
       (jy > 0 ? a.jyp : a.jyn) |= 1u << i;
     }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+  if (L <= 3) {
+    transfer_small_kernel<<<1, std::max(32, 1 << nb), 0, st>>>(in, out, a, nb);
+    return cuda_check(cudaGetLastError(), "transfer matvec");
+  }
   const std::vector<Pass> plan = plan_passes(nb);
   int rc = QISG_OK;
   for (size_t p = 0; p < plan.size() && !rc; ++p) {
     const Pass &q = plan[p];
     const int width = q.c + (q.hi - q.lo);
     const int fixed = nb - width;
-    const bool last = p + 1 == plan.size();
-    const bool pair = last && fixed > 0;
+    const bool pair = p + 1 == plan.size();   // the last pass
     const unsigned blocks = pair ? 1u << (fixed - 1) : 1u << fixed;
     const size_t T = (size_t)1 << width, smem = (128 + (pair ? 2 * T + 2 * T / 16 : T + T / 16)) * sizeof(double);
-    const PassArgs pa{q.c, q.lo, q.hi, p == 0, last, nb};
+    const PassArgs pa{q.c, q.lo, q.hi, p == 0, nb};
     if (pair)
       transfer_pass_kernel<true><<<blocks, kTransferBlock / 2, smem, st>>>(p == 0 ? in : out, out, a, pa);
     else
