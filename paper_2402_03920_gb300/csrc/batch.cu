@@ -328,7 +328,6 @@ int build_tables(qisg_batch *B) {
   if (rc) return rc;
   B->n_tiles = (int)tiles.size();
   B->n_chains = (int)chains.size();
-  cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->smem);
   int per_sm = 0;
   rc = cuda_check(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kBatchBlock, B->smem),
                   "occupancy");

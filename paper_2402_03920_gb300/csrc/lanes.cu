@@ -272,18 +272,6 @@ void launch_half_sweep(bool pdl, const LanesArgs<Word> &p, dim3 grid, size_t sme
                 grid, dim3(kBlock), smem, st, p, BLUE ? 1 : 0, count_only, a0, tile_sites);
 }
 
-template <typename Word, bool BLUE>
-int set_smem_limits() {
-  const void *fns[] = {(const void *)lanes_half_sweep_kernel<Word, BLUE, 0, 0, 1>, (const void *)lanes_half_sweep_kernel<Word, BLUE, 0, 0, 4>,
-                       (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 1, 1>, (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 1, 4>,
-                       (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 0, 1>, (const void *)lanes_half_sweep_kernel<Word, BLUE, 4, 0, 4>};
-  for (const void *f : fns) {
-    const int rc = cuda_check(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024), "shared memory");
-    if (rc) return rc;
-  }
-  return QISG_OK;
-}
-
 // The planes the packing takes (L <= 132 for any ladder, 134 for short ones).
 // Nothing of the tile's depends on the plane: earlier tiles kept tables of 11
 // bytes per site beside 33792 fixed bytes in 227 KB, and handles beyond that
@@ -315,13 +303,6 @@ int half_sweep_t(qisg_handle *h, int colour, int count_only, int64_t a_lo, int64
   const int tile_sites = per * rows;
   const int64_t blocks = (p.half_N + tile_sites - 1) / tile_sites;
   if (blocks > 0x7FFFFFFF) return fail(QISG_EINVAL, "lattice too large for one launch");
-  static bool attr_set = false;
-  if (!attr_set) {
-    int rc = set_smem_limits<Word, false>();
-    if (!rc) rc = set_smem_limits<Word, true>();
-    if (rc) return rc;
-    attr_set = true;
-  }
   for (int64_t a0 = a_lo; a0 < a_lo + n_a; a0 += (h->per_sample_launch ? 1 : 65535)) {
     const int64_t na = h->per_sample_launch ? 1 : std::min<int64_t>(65535, a_lo + n_a - a0);
     const int tok = prof_begin(h, sweep_kind(colour));

@@ -66,7 +66,9 @@ struct LanesSample {
 
 // Shared memory of one tile: threshold rows by class code, the lane table,
 // the Philox words of each (slot, quad), counter sums, the flips that the
-// TPS = 4 form exchanges, and the class codes.
+// TPS = 4 form exchanges, and the class codes.  At most 41472 bytes (32 slots x
+// 4 replicas), so no kernel that runs tiles has to raise the 48 KB that a launch
+// may ask for.
 __host__ __device__ inline size_t lanes_tile_smem(int n_slots, int n_rep) {
   const size_t sq = (size_t)n_slots * ((n_rep + 3) / 4);
   size_t o = sq * 48 + (size_t)n_slots * 64;                  // lane table and Philox words, threshold rows

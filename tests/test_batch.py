@@ -216,3 +216,17 @@ def test_largest_lattice_side_runs(qisg):
             _, _, wa, S = b.results(slot, spins=True)
             st = _oracle_instance(L, Lt, qisg.ladder_linear(0.2, 0.5, ns, 1.0), 4, seed, 2)
             assert np.array_equal(S, st.S[0]) and np.array_equal(wa, st.walker_at[0]), L
+
+
+def test_two_batches_take_turns(qisg):
+    """A batch whose tiles need more shared memory runs again after one that needs less."""
+    lads = [qisg.ladder_linear(0.2, 0.5, ns, 1.0) for ns in (32, 1)]
+    with qisg.Batch(1, 16 << 20) as a, qisg.Batch(1, 16 << 20) as b:
+        sa, sb = a.admit(8, 16, lads[0], 4, 81), b.admit(8, 16, lads[1], 1, 82)
+        for _ in range(2):
+            a.run(2)
+            b.run(2)
+        for batch, slot, lad, n_rep, seed in ((a, sa, lads[0], 4, 81), (b, sb, lads[1], 1, 82)):
+            _, _, wa, S = batch.results(slot, spins=True)
+            st = _oracle_instance(8, 16, lad, n_rep, seed, 4)
+            assert np.array_equal(S, st.S[0]) and np.array_equal(wa, st.walker_at[0])
