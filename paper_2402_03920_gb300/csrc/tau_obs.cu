@@ -312,9 +312,9 @@ int launch_tau(int l, const TauArgs &a, unsigned blocks, cudaStream_t st) {
     size_t smem = (size_t)b.pitch * 4 * a.Lt;
     constexpr size_t kRed = ((P::H + 1) / 2 + 2) * kTauBlock * 4 + kTauBlock * 8;
     if (b.parts > 1) smem += kRed;   // L_tau <= 256: fits
-    if (smem > 48 * 1024) {
+    if (smem > 48 * 1024) {   // one limit for all callers: threads with other L_tau may be between this and their launch
       const int rc = cuda_check(cudaFuncSetAttribute(tau_obs_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)smem),
+                                                     (int)kTauSmemMax),
                                 "shared memory");
       if (rc) return rc;
     }

@@ -102,3 +102,28 @@ def test_cancelling_lags(qisg, L, Lt):
         assert np.array_equal(g, w), name
     # sums of at most 600 terms that are not negative, in another order: below 1e-13
     assert np.allclose(got[3], want[3], rtol=1e-12, atol=0), "SF"
+
+
+def test_two_threads(qisg):
+    """Handles of one L and two L_tau, with different needs of shared memory, in two threads."""
+    import threading
+    insts = [make(qisg, 16, Lt, 0.2, 0.5, 2, 1.0, 1, 1, 3, layout=qisg.QISG_LAYOUT_LANES)[0] for Lt in (1024, 700)]
+    want = [inst.tau_observables() for inst in insts]
+    errors = []
+
+    def calls(inst, w):
+        try:
+            for _ in range(200):
+                got = inst.tau_observables()
+                assert all(np.array_equal(x, y) for x, y in zip(got, w))
+        except Exception as e:   # noqa: BLE001 - reported below
+            errors.append(e)
+
+    threads = [threading.Thread(target=calls, args=a) for a in zip(insts, want)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for inst in insts:
+        inst.close()
