@@ -7,9 +7,10 @@
 // is the one qisg_create would give for the same parameters (sample 0).  The
 // persistent kernel walks a work-list of (instance, colour-site range) tiles
 // for the red and the blue half sweep, then one warp per (instance, replica)
-// chain for the PT pass (Sec. 2.1), then advances each instance's sweep
-// counter; grid-wide barriers with a bounded wait separate the phases.  The
-// launch is cooperative, so all blocks are resident.
+// chain for the PT pass (Sec. 2.1); grid-wide barriers with a bounded wait
+// separate the phases, and the instances' sweep counters advance once, after
+// the last sweep of the launch.  The launch is cooperative, so all blocks are
+// resident.
 //
 // Device memory comes from one arena (the batch's memory budget) managed by
 // a first-fit allocator on the host; instances are admitted into free slots

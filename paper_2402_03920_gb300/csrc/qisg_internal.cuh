@@ -342,10 +342,13 @@ __device__ __forceinline__ uint32_t pt_chain(int32_t *wa, unsigned long long *Ua
 // while the kernel before it on the stream is finishing; it must call
 // pdl_begin() before it touches global memory that kernel writes (the wait
 // returns once that kernel has completed and its writes are visible; with
-// no such dependency it returns at once).  No kernel triggers its
-// dependents early: the trigger is each block's exit, so the next kernel is
-// launched as the last blocks leave instead of taking SM room while this
-// one still runs (the early trigger made the sweep slower than no overlap).
+// no such dependency it returns at once), and it must read what that kernel
+// writes by plain loads: no __ldg, no const __restrict__ parameter, whose
+// loads may be moved above the wait.  The trigger is each block's exit, so the
+// next kernel is launched as the last blocks leave instead of taking SM room
+// while this one still runs (a trigger at the start made the sweep slower than
+// no overlap); only the blue pass with the PT chains in its last blocks
+// triggers by itself, each block once its own work is done (pdl_trigger).
 __device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Trigger: the dependent kernel may launch once every block has called this

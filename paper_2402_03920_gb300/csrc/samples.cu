@@ -32,13 +32,12 @@ template <typename Word>
 struct SamplesArgs {
   Word *spins;
   const Word *J;
-  const uint32_t *T;
   unsigned long long *U;
   const unsigned long long *d_t;
   uint2 key;
   PhiloxKeys rk;         // its round keys
-  int64_t N, half_N;
-  int L, Lt, plane, half_plane, n_slots, n_rep, n_q, W;
+  int64_t N;
+  int L, Lt, plane, n_slots, n_rep, n_q, W;
   int seg_sites;         // G: sites of one colour each quad walks along tau (the most of any thread)
   int n_seg;             // segments per column
   int seg_base, seg_rem; // W = 32 replica-quad kernel: segment g of a column holds seg_base + (g < seg_rem)
@@ -283,7 +282,6 @@ __global__ void __launch_bounds__(kBlock) samples_half_sweep_kernel(SamplesArgs<
         const Word us2 = c1 & c2;
         const Word ut0 = t1 ^ t2;
         const Word ut1 = t1 & t2;
-        // accept mask: mux tree over (u_t, u_s) of the per-class masks
         const Word nz = t1 | t2;
         const Word flip = count_only ? Word(0) : accept_word<Word>(R, T, us0, us1, us2, ut0, ut1, p.one);
         if (!count_only) base[(size_t)site * 4] = sc ^ flip;
@@ -1771,17 +1769,14 @@ SamplesArgs<Word> make_args(qisg_handle *h, int colour) {
   SamplesArgs<Word> p;
   p.spins = reinterpret_cast<Word *>(h->spins);
   p.J = reinterpret_cast<const Word *>(h->J);
-  p.T = h->d_T;
   p.U = h->d_U;
   p.d_t = h->d_t;
   p.key = make_uint2((uint32_t)h->seed, (uint32_t)(h->seed >> 32));
   p.rk = PhiloxKeys(p.key);
   p.N = h->N;
-  p.half_N = h->N / 2;
   p.L = h->L;
   p.Lt = h->Lt;
   p.plane = h->L * h->L;
-  p.half_plane = p.plane / 2;
   p.n_slots = h->n_slots;
   p.n_rep = h->n_rep;
   p.n_q = h->n_q;
@@ -1862,7 +1857,7 @@ void fill_thresholds(const qisg_handle *h, SlotThresholds &th) {
 // blocks), none beyond (the bound would spill).
 template <bool PF, int MINB, int KS>
 constexpr int blue_min_blocks() {
-  return MINB > 0 ? MINB : (PF && KS <= 7) ? (3) : 0;
+  return MINB > 0 ? MINB : (PF && KS <= 7) ? 3 : 0;
 }
 
 // The blue kernel for ks = 3 .. 9 counter planes (variant 0 or 2; 64-bit words
@@ -2458,8 +2453,10 @@ int samples_persistent(qisg_handle *h, int n_sweeps) {
   if (rc) return rc;
   a.red.n_zero_U = 0;
   // the blue phase's default segmentation fills the persistent grid (every
-  // form of the kernel is bounded to the same residency), walks of at most
-  // 32 sites, above 15 (seven counter planes, with which the kernel spills more)
+  // form of the kernel compiles to 168 registers, three blocks per SM, for
+  // which its shared memory, at most 60 KB with the ring, leaves room; were
+  // one to differ, this grid would be an estimate), walks of at most 32
+  // sites, above 15 (seven counter planes, with which the kernel spills more)
   // at a cost (us a sweep, 256 samples at L = 24, L_tau = 512, walks of 4 | 8 |
   // 16 | 32 sites: 1954 | 1873 | 1995 | 2228)
   int per_sm0 = 0;
