@@ -627,11 +627,11 @@ def transfer_entry(torch, qisg, reps=50):
     """The exact-diagonalisation code's transfer-matrix product (Sec. 2.2) at
     the largest lattice one GPU holds, L = 5 (even sector, 2^24 doubles):
     time per product, against the FP64 roofline (on this part FP64 issue, not
-    HBM, bounds it) with the HBM figure beside it.  Algorithmic work: the
-    paper's formulas, 2 multiplies + 1 add per element and round for the
-    L^2 - 1 rounds and the parity factor, 1 multiply for each of the two
-    Boltzmann factors (77 flops per element at L = 5); bytes: one read of the
-    input and one write of the output."""
+    HBM, bounds it) with the HBM figure beside it.  Algorithmic work: what
+    the rounds need with their common factor taken out, one fused multiply-add
+    per element and round for the L^2 - 1 rounds and the parity factor, and 1
+    multiply for each of the two Boltzmann factors (52 flops per element at
+    L = 5); bytes: one read of the input and one write of the output."""
     L, k = 5, 0.29
     rng = np.random.default_rng(5)
     J = np.where(rng.random((L * L, 2)) < 0.5, 1, -1).astype(np.int8)
@@ -649,7 +649,7 @@ def transfer_entry(torch, qisg, reps=50):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     pk, _ = peaks()
-    flops = float(n) * (3 * (L * L - 1) + 3 + 2)
+    flops = float(n) * (2 * L * L + 2)
     alg = 16.0 * n
     hbm = pk.get("hbm_gbs", 6800.0)
     gflops = flops / (ms * 1e-3) / 1e9
