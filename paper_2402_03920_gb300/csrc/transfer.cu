@@ -15,7 +15,7 @@
 // rounds are taken with the factor jP outside: with r = jM / jP a pair update
 // is x' = x + r y, y' = y + r x, one fused multiply-add per element, and jP^{L^2}
 // goes into the table of w used on load.  (jP x + jM y as y + jP (x - y) takes
-// three operations per pair: 1.351 ms at L = 5 in that form, 0.891 now.)  This is the
+// three operations per pair: 1.351 ms at L = 5 in that form, 0.889 now.)  This is the
 // paper's formula rearranged: the results differ by rounding only (relative
 // 1e-15 in norm after 25 rounds), and the scaled values stay below the
 // plain ones until the last round.
@@ -24,9 +24,9 @@
 // instead of once per round: a tile fixes all index bits except a low run
 // [0, c) (c = 5: 32 consecutive doubles, 256-byte segments) and the bits
 // [lo, hi) of the pass's rounds; the first pass takes bits [0, 12) whole.
-// Within a tile a thread takes up to four rounds on 16 elements in registers
-// (three in the last pass, which holds a tile and its complement), so shared
-// memory is crossed once per four rounds and, where the run of low bits makes
+// Within a tile a thread takes up to three rounds on 8 elements in registers
+// (in the last pass on 8 and their complement's 8), so shared memory is
+// crossed once per three rounds and, where the run of low bits makes
 // a warp's accesses whole segments, the first group reads HBM and the last
 // group writes it directly.  The last pass pairs every tile with its bit
 // complement (the tile holding 2^{n} - 1 - n for each n) for the parity
@@ -89,7 +89,7 @@ __device__ __forceinline__ uint32_t tile_index(const PassArgs &q, uint32_t t, ui
 }
 
 // Shared-memory place of tile element t: one double of padding per 16, so
-// that threads reading 16 consecutive elements each meet different banks.
+// that threads reading 8 consecutive elements each meet different banks.
 __device__ __forceinline__ uint32_t padded(uint32_t t) { return t + (t >> 4); }
 
 // G rounds on 2^G elements held in registers.
@@ -163,9 +163,7 @@ __device__ __forceinline__ void stage_g(int g, const double *src, double *dst, d
   switch (g) {
     case 1: stage<1, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
     case 2: stage<2, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
-    case 3: stage<3, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
-    default:
-      if constexpr (!PAIR) stage<4, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb);
+    default: stage<3, PAIR, FROM, TO>(src, dst, tile, wt, a, q, T_log, f, tb); break;
   }
 }
 
@@ -185,7 +183,10 @@ __global__ void __launch_bounds__(kTransferBlock) transfer_pass_kernel(const dou
     wt[64 + threadIdx.x] = a.wtab[threadIdx.x];
   }
   __syncthreads();
-  constexpr int GM = PAIR ? 3 : 4;
+  // three rounds on 8 elements a thread, fewer where that would leave less than
+  // four warps at work (the last pass at L = 4).  A call at L = 4 | 5: 26.8 | 912 us;
+  // four rounds in the unpaired passes 27.7 | 925, three everywhere 27.8 | 911
+  const int GM = min(3, max(1, T_log - 7));
   int tb = q.c, left = q.hi - q.lo;
   bool loaded = false;
   if (!PAIR && tb < 4) {   // consecutive elements per thread: load whole segments first
